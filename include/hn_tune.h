@@ -9,6 +9,11 @@
  * them and tail_level either live in the distributed shared memory of the whole cluster (`dsm`,
  * when they fit) or are read through L2.  The best split depends on the levels and the batch;
  * hn_mg_autotune measures candidates on the hierarchy itself.
+ *
+ * A hierarchy whose shape was not set by hn_mg_set_tuning (the default, or an autotuned shape with
+ * sweep 1 and mid 0) runs the larger levels of an FP32 / FP16 V(2,2) cycle, alone, in batches and in the
+ * server, as marching sweeps: one pass over the level each way.  hn_mg_set_tuning selects exactly
+ * the forms described below.
  */
 #ifndef HN_TUNE_H
 #define HN_TUNE_H
@@ -45,7 +50,8 @@ typedef struct {
                        another; 2: every level above tail_level and, on the finest level, the steps
                        after the first smoothing step (the second step, the defect, the
                        restriction) in one launch; 0: one launch per step.  Not combined with
-                       staged or mid; without effect in batches and in the server */
+                       staged or mid; 1 and 2 are for a hierarchy solved alone (in batches and in the
+                       server, without a set shape, 1 stands for the marching sweeps) */
 } hn_tuning;
 
 /* Set / read the launch shape used by mg's later solves.  HN_ERR_ARG on values out of range. */

@@ -99,12 +99,7 @@ void forget_batch(hn_mg* mg) {
 // one block per problem and a tail that fits in shared memory; few problems: the solo default)
 Tuning batch_tuning(const std::vector<hn_mg*>& list) {
   bool same = list[0]->tuned;
-  for (hn_mg* mg : list)
-    same = same && mg->tuned && mg->tuning.tail_level == list[0]->tuning.tail_level &&
-           mg->tuning.cluster == list[0]->tuning.cluster && mg->tuning.pdl == list[0]->tuning.pdl &&
-           mg->tuning.staged == list[0]->tuning.staged && mg->tuning.dsm == list[0]->tuning.dsm &&
-           mg->tuning.fuse_up == list[0]->tuning.fuse_up && mg->tuning.mid == list[0]->tuning.mid &&
-           mg->tuning.sweep == list[0]->tuning.sweep;
+  for (hn_mg* mg : list) same = same && mg->tuned && mg->tuning == list[0]->tuning;
   if (same) return list[0]->tuning;
   Tuning t;
   const int n = (int)list.size();
@@ -141,6 +136,36 @@ void fill_stats(const hn_mg* mg, const ProbState& st, long long t0, hn_mg_stats*
   out->relres = st.relres;
   out->setup_ns = mg->setup_ns;
   out->solve_ns = now_ns() - t0;
+}
+
+// march: whether the shape may run its levels as marching sweeps (Tuning::march)
+hn_status set_shape(hn_mg* mg, const hn_tuning* t, int march) {
+  clear_error();
+  if (!mg || !t) return set_error(HN_ERR_ARG, "null argument");
+  const int c = t->cluster;
+  if (t->tail_level < mg->coarse || t->tail_level > HN_MAX_LEVEL || !(c == 1 || c == 2 || c == 4 || c == 8 || c == 16))
+    return set_error(HN_ERR_ARG, "tail_level in [coarse_L, %d], cluster in {1,2,4,8,16}", HN_MAX_LEVEL);
+  HN_TRY(ensure_solo(mg));
+  if (t->pdl < 0 || t->pdl > 3) return set_error(HN_ERR_ARG, "pdl must be 0, 1, 2 or 3");
+  if (t->staged != 0 && t->staged != 1) return set_error(HN_ERR_ARG, "staged must be 0 or 1");
+  if (t->dsm != 0 && t->dsm != 1) return set_error(HN_ERR_ARG, "dsm must be 0 or 1");
+  if (t->fuse_up != 0 && t->fuse_up != 1) return set_error(HN_ERR_ARG, "fuse_up must be 0 or 1");
+  if (t->mid < 0 || t->mid > HN_MAX_LEVEL) return set_error(HN_ERR_ARG, "mid must be in [0, %d]", HN_MAX_LEVEL);
+  if (t->sweep < 0 || t->sweep > 2) return set_error(HN_ERR_ARG, "sweep must be 0, 1 or 2");
+  Tuning tu;
+  tu.tail_level = t->tail_level;
+  tu.cluster = c;
+  tu.pdl = t->pdl;
+  tu.staged = t->staged;
+  tu.dsm = t->dsm;
+  tu.fuse_up = t->fuse_up;
+  tu.mid = t->mid;
+  tu.sweep = t->sweep;
+  tu.march = march;
+  mg->solo->set_tuning(tu);
+  mg->tuning = tu;
+  mg->tuned = true;
+  return HN_OK;
 }
 
 }  // namespace
@@ -352,10 +377,7 @@ hn_status hn_mg_solve_batch(hn_mg* const* mgs, int count, const double* const* b
   Engine& e = *g_batch_engine;
   {
     const Tuning t = batch_tuning(list);
-    const Tuning& c = e.tuning();
-    if (t.tail_level != c.tail_level || t.cluster != c.cluster || t.pdl != c.pdl || t.staged != c.staged ||
-        t.dsm != c.dsm || t.fuse_up != c.fuse_up || t.mid != c.mid || t.sweep != c.sweep)
-      e.set_tuning(t);
+    if (!(t == e.tuning())) e.set_tuning(t);
   }
   cudaStream_t s = e.stream();
   std::vector<int> slots(count), guess(count, 0);
@@ -468,33 +490,7 @@ hn_status hn_mg_set_profiling(hn_mg* mg, int enable) {
   return HN_OK;
 }
 
-hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t) {
-  clear_error();
-  if (!mg || !t) return set_error(HN_ERR_ARG, "null argument");
-  const int c = t->cluster;
-  if (t->tail_level < mg->coarse || t->tail_level > HN_MAX_LEVEL || !(c == 1 || c == 2 || c == 4 || c == 8 || c == 16))
-    return set_error(HN_ERR_ARG, "tail_level in [coarse_L, %d], cluster in {1,2,4,8,16}", HN_MAX_LEVEL);
-  HN_TRY(ensure_solo(mg));
-  if (t->pdl < 0 || t->pdl > 3) return set_error(HN_ERR_ARG, "pdl must be 0, 1, 2 or 3");
-  if (t->staged != 0 && t->staged != 1) return set_error(HN_ERR_ARG, "staged must be 0 or 1");
-  if (t->dsm != 0 && t->dsm != 1) return set_error(HN_ERR_ARG, "dsm must be 0 or 1");
-  if (t->fuse_up != 0 && t->fuse_up != 1) return set_error(HN_ERR_ARG, "fuse_up must be 0 or 1");
-  if (t->mid < 0 || t->mid > HN_MAX_LEVEL) return set_error(HN_ERR_ARG, "mid must be in [0, %d]", HN_MAX_LEVEL);
-  if (t->sweep < 0 || t->sweep > 2) return set_error(HN_ERR_ARG, "sweep must be 0, 1 or 2");
-  Tuning tu;
-  tu.tail_level = t->tail_level;
-  tu.cluster = c;
-  tu.pdl = t->pdl;
-  tu.staged = t->staged;
-  tu.dsm = t->dsm;
-  tu.fuse_up = t->fuse_up;
-  tu.mid = t->mid;
-  tu.sweep = t->sweep;
-  mg->solo->set_tuning(tu);
-  mg->tuning = tu;
-  mg->tuned = true;
-  return HN_OK;
-}
+hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t) { return set_shape(mg, t, 0); }
 
 hn_status hn_mg_get_tuning(const hn_mg* mg, hn_tuning* t) {
   clear_error();
@@ -535,7 +531,7 @@ hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, 
   for (int T = mg->coarse; T <= tmax; ++T)
     for (int ci = 0; ci < 5; ++ci) {
       hn_tuning t{T, clusters[ci], 2, 0, 1, 0, mids[mi], sweeps[mi]};
-      HN_TRY(hn_mg_set_tuning(mg, &t));
+      HN_TRY(set_shape(mg, &t, 1));
       HN_TRY(hn_mg_solve(mg, b, x, 0, 0, nullptr));            // capture + warm-up
       HN_CUDA(cudaEventRecord(e0, mg->solo->stream()));
       for (int r = 0; r < reps; ++r) {
@@ -551,7 +547,7 @@ hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, 
       if (times_ms && idx < cap) times_ms[idx] = per;
       if (per < best_ms) { best_ms = per; bt = t; }
     }
-  HN_TRY(hn_mg_set_tuning(mg, &bt));
+  HN_TRY(set_shape(mg, &bt, 1));
   if (best) *best = bt;
   if (const char* path = std::getenv("HN_TUNE_CACHE")) {
     char gpu[256];

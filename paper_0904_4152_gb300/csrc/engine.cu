@@ -535,7 +535,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   // the control kernel's groups: as many as the largest problem's norm sum has
   const int ctl_groups = (int)((pitch_of(Lmax) / kTile + kSumGroup - 1) / kSumGroup);
   take(sizeof(double) * (size_t)cap * ctl_groups);
-  take(sizeof(unsigned) * (size_t)cap);
+  take(sizeof(unsigned) * (size_t)cap * ctl_groups);
   take(sizeof(int) * plan_ints());
   take(sizeof(TileList) * (kMaxLevel + 1));
   take(sizeof(unsigned long long) * 3);
@@ -562,7 +562,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   dTaken_ = b.take<unsigned>(4);
   dLaunches_ = b.take<unsigned long long>(1);
   double* gsum = b.take<double>((size_t)cap * ctl_groups);
-  unsigned* gticket = b.take<unsigned>((size_t)cap);
+  unsigned* gticket = b.take<unsigned>((size_t)cap * ctl_groups);
   dPlan_ = b.take<int>(plan_ints());
   dLists_ = b.take<TileList>(kMaxLevel + 1);
   dBar_ = b.take<unsigned long long>(3);
@@ -773,12 +773,16 @@ long long Engine::launch_bytes(int cls, int level) const {
       for (hn_mg* mg : members_) {
         if (!mg || level > mg->L || level <= mg->coarse) continue;
         const bool own = level == mg->L && prm_.solver != SOLVER_PCG;
-        const double pn = 9 * bb + vb + (own ? vb + wd : (prec == P64 ? 8 : 4)) + vb + 0.25 * vb;
+        // (a marching sweep also reads omega / D from a nonzero iterate)
+        const double wdm = march_level(level) ? 4 : wd;
+        const double pn = 9 * bb + vb + (own ? vb + wdm : (prec == P64 ? 8 : 4)) + vb + 0.25 * vb;
         sum += (long long)(pn * (double)N_of(level));
       }
       return sum;
     }
-    case KC_SWEEP_UP: per = 9 * bb + vb + 0.25 * vb + vb + wd + vb; break;   // bands, x, e_c, rhs; write
+    case KC_SWEEP_UP:                                          // bands, x, e_c, rhs; write
+      per = 9 * bb + vb + 0.25 * vb + vb + (march_level(level) ? 4 : wd) + vb;
+      break;
     case KC_MID_DOWN:
     case KC_MID_UP: {
       // the persistent kernels: the sum of their steps' bytes over levels T+1..level (the top
@@ -899,6 +903,17 @@ bool Engine::sweep_level(int l) const {
   return tune_.sweep == 2 || (!is_top(l) && l <= kSweepMaxLevel);
 }
 
+// Levels in marching sweeps: every level from kMarchMinLevel above the tail in an engine of several
+// problems; in an engine of one, those from kMarchSoloLevel.  Below that a solve alone is bound by the
+// latency of its launches, where the fused sweeps' few phases beat a march of 9 iterations (levels 6..8:
+// ~4 against ~6 us a launch; L = 8 solve 915 against 940 us), on level 9 they are alike (L = 10
+// solve with level 9 marching or not: 1.490 / 1.518 ms).
+bool Engine::march_level(int l) const {
+  const int T = std::max(tune_.tail_level, prm_.coarse);
+  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !tune_.staged &&
+         !tune_.fuse_up && mid_top() <= T && l >= (cap_ == 1 ? kMarchSoloLevel : kMarchMinLevel);
+}
+
 hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   const int c = prm_.coarse, pre = prm_.pre, post = prm_.post;
   const int T = std::max(tune_.tail_level, c);
@@ -917,6 +932,15 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   for (int l = Lmax_; l > std::max(T, M); --l) {
     // a finest level: lagged check (the PCG preconditioner's cycle has none)
     const bool top = prm_.solver != SOLVER_PCG && is_top(l);
+    if (march_level(l)) {
+      HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, 0, 0, s));
+      if (top) {
+        HN_LAUNCH(KC_CHECK, l, launch_march_check(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, s));
+        if (cap_ != 1) HN_LAUNCH(KC_CONTROL, l, launch_control(E_, CTRL_PRE, s, l));
+        HN_TRY(after_check());
+      }
+      continue;
+    }
     if (sweep_level(l) && !top) {
       // a zero iterate: both smoothing steps, the defect and the restriction in one launch
       HN_LAUNCH(KC_SWEEP_DOWN, l, launch_sweep_down(E_, lists_[l], l, want, 0, s));
@@ -955,6 +979,11 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   if (M > T) HN_LAUNCH(KC_MID_UP, M, launch_mid(E_, dLists_, M, T, want, 1, s));
   int e_sel = 0;                           // buffer of the coarse iterate (the tail's: 0)
   for (int l = std::max(T, M) + 1; l <= Lmax_; ++l) {
+    if (march_level(l)) {                  // prolongation and both post-smoothing steps, buffer 1 to 0
+      HN_LAUNCH(KC_SWEEP_UP, l, launch_march(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, 1, e_sel, s));
+      e_sel = 0;
+      continue;
+    }
     if (sweep_level(l) && !is_top(l)) {
       // prolongation and both post-smoothing steps in one launch; the result in buffer 1 (a
       // problem's own finest level keeps its iterate in buffer 0)

@@ -98,6 +98,14 @@ struct Tuning {
                     // level above the tail, with the finest level's steps after its first smoothing
                     // step.  Default 1 (measured at L = 9 / 10 / 12: FP32-inner DC -3.6 / -1.0 /
                     // -0.4 %, FP64 MG -11.5 / -2.3 / -0.3 %); 2 was slower from L = 10 up.
+  int march = 1;    // FP32 / FP16 hierarchies with V(2,2) cycles, sweep on: the levels from
+                    // kMarchMinLevel above the tail run as marching sweeps (k_march.cu), also in
+                    // batches and in the server.  A shape set by hn_mg_set_tuning has it off (the
+                    // forms hn_tune.h describes, as they are); not part of hn_tuning.
+  bool operator==(const Tuning& o) const {
+    return tail_level == o.tail_level && cluster == o.cluster && pdl == o.pdl && staged == o.staged && dsm == o.dsm &&
+           fuse_up == o.fuse_up && mid == o.mid && sweep == o.sweep && march == o.march;
+  }
 };
 
 class Engine;
@@ -258,6 +266,7 @@ class Engine {
   int mid_top() const;              // top level of the persistent kernels (<= tail level: none)
   bool sweep_on() const;            // the fused level sweeps run (tuning sweep, and they apply)
   bool sweep_level(int l) const;    // level l's down / up parts run as fused sweeps
+  bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
   bool fuse_control() const;        // the DC control steps fold into the outer defect and update
   // level l may be a member's own finest level (the server's engines: any level)
   bool is_top(int l) const { return topMaskAll_ || ((topMask_ >> l) & 1u); }
