@@ -95,17 +95,12 @@ void forget_batch(hn_mg* mg) {
   }
 }
 
-// launch shape of a batch: the members' common tuned shape, else by batch size (many problems:
-// one block per problem and a tail that fits in shared memory; few problems: the solo default)
+// launch shape of a batch: the members' common tuned shape, else group_tuning's
 Tuning batch_tuning(const std::vector<hn_mg*>& list) {
   bool same = list[0]->tuned;
   for (hn_mg* mg : list) same = same && mg->tuned && mg->tuning == list[0]->tuning;
   if (same) return list[0]->tuning;
-  Tuning t;
-  const int n = (int)list.size();
-  if (n >= 32) { t.tail_level = 5; t.cluster = 1; }
-  else if (n >= 8) { t.tail_level = 6; t.cluster = 4; }
-  return t;
+  return group_tuning(list[0]->prm, (int)list.size());
 }
 
 hn_status copy_in(double* dst, const double* src, long long N, int device_ptrs, cudaStream_t s) {

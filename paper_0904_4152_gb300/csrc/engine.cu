@@ -684,6 +684,15 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
     if (l > P.coarse) t.solo_c = P.lev[l - 1];
     if (l < P.L) t.solo_f = P.lev[l + 1];
   }
+  small_ = SmallSolo{};
+  if (cap_ == 1 && !slots.empty() && slots[0]) {
+    const ProblemDev& P = slots[0]->host;
+    small_.L = P.L;
+    small_.coarse = P.coarse;
+    small_.m = P.m;
+    small_.cinv = P.cinv;
+    for (int l = P.coarse; l <= std::min(P.L, kSmallTop); ++l) small_.lev[l - 2] = P.lev[l];
+  }
   // the persistent kernels read the tile lists (with the one-problem descriptors) from device
   // memory; the staging copy is free again once the previous upload finished (event above)
   std::memcpy(hLists_, lists_, sizeof(TileList) * (kMaxLevel + 1));
@@ -914,6 +923,13 @@ bool Engine::march_level(int l) const {
          !tune_.fuse_up && mid_top() <= T && l >= (cap_ == 1 ? kMarchSoloLevel : kMarchMinLevel);
 }
 
+// The levels of the tail in one block's shared memory (k_small) in place of the cluster kernel, under the
+// conditions of the marching sweeps and with the exact coarse solver.
+bool Engine::small_tail() const {
+  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
+         !tune_.staged && !tune_.fuse_up && std::max(tune_.tail_level, prm_.coarse) <= kSmallTop;
+}
+
 hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   const int c = prm_.coarse, pre = prm_.pre, post = prm_.post;
   const int T = std::max(tune_.tail_level, c);
@@ -975,7 +991,8 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
     HN_LAUNCH(KC_RESTRICT, l, launch_restrict(E_, lists_[l - 1], l, want, grid_[l - 1], s));
   }
   if (M > T) HN_LAUNCH(KC_MID_DOWN, M, launch_mid(E_, dLists_, M, T, want, 0, s));
-  HN_LAUNCH(KC_TAIL, T, launch_tail(E_, T, want, tune_.cluster, s));
+  if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, T, want, s));
+  else HN_LAUNCH(KC_TAIL, T, launch_tail(E_, T, want, tune_.cluster, s));
   if (M > T) HN_LAUNCH(KC_MID_UP, M, launch_mid(E_, dLists_, M, T, want, 1, s));
   int e_sel = 0;                           // buffer of the coarse iterate (the tail's: 0)
   for (int l = std::max(T, M) + 1; l <= Lmax_; ++l) {

@@ -108,6 +108,16 @@ struct Tuning {
   }
 };
 
+// Launch shape of an engine of several problems (slots): FP32 / FP16 hierarchies take the one-block tail
+// (levels to kSmallTop) below the marching sweeps; FP64 ones, whose levels 5 and 6 are too slow for one
+// SM, by the number of problems (many: one block per problem; few: the cluster tail).
+inline Tuning group_tuning(const Params& prm, int slots) {
+  Tuning t;
+  if (prm.prec != P64 || slots >= 32) { t.tail_level = kSmallTop; t.cluster = 1; }
+  else if (slots >= 8) { t.tail_level = 6; t.cluster = 4; }
+  return t;
+}
+
 class Engine;
 
 }  // namespace hn
@@ -267,6 +277,8 @@ class Engine {
   bool sweep_on() const;            // the fused level sweeps run (tuning sweep, and they apply)
   bool sweep_level(int l) const;    // level l's down / up parts run as fused sweeps
   bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
+  bool small_tail() const;          // the tail runs in one block's shared memory (k_small)
+  SmallSolo small_{};               // its descriptors, for an engine of one problem
   bool fuse_control() const;        // the DC control steps fold into the outer defect and update
   // level l may be a member's own finest level (the server's engines: any level)
   bool is_top(int l) const { return topMaskAll_ || ((topMask_ >> l) & 1u); }

@@ -232,6 +232,16 @@ bool pre_fuses(int prec);
 // the V cycle on levels coarse..min(T, L) of every problem in phase `want`, one thread-block
 // cluster of `cluster` blocks per problem slot
 cudaError_t launch_tail(const EngineDev& E, int T, int want, int cluster, cudaStream_t s);
+// the same on levels coarse..T <= kSmallTop of FP32 / FP16 hierarchies with V(2,2) cycles and the exact
+// coarse solver, one block per problem slot (k_small.cu).  solo: the descriptors of an engine of one
+// problem by value (L = 0: none)
+constexpr int kSmallTop = 5;
+struct SmallSolo {
+  int L = 0, coarse = 0, m = 0;
+  const double* cinv = nullptr;
+  LevelDev lev[kSmallTop - 1] = {};      // levels 2..min(L, kSmallTop)
+};
+cudaError_t launch_small(const EngineDev& E, const SmallSolo& solo, int T, int want, cudaStream_t s);
 // one-time kernel attributes (cluster-size opt-in); call outside stream capture
 cudaError_t prepare_kernels();
 

@@ -82,3 +82,24 @@ def test_host_issued_marching_iterations_give_the_bits_of_the_graph(hn):
         assert {"sweep_down", "sweep_up", "tail"} <= names and not {"jacobi", "defect", "prolong"} & names, names
     finally:
         hn.hn_mg_destroy(mg)
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("L,coarse_L,bc", [(2, 2, 15), (3, 2, 1), (3, 3, LR), (4, 3, 15), (5, 2, LR), (5, 4, 7), (6, 4, 15),
+                                           (7, 2, 5)])
+def test_one_block_tail_gives_the_bits_of_the_cluster_tail(hn, L, coarse_L, bc, prec):
+    # a finest level inside the tail (with its lagged checks) or above it, each coarsest level
+    coef, _ = I.batch_problem(L, L)
+    b = I.rhs_uniform_bc(L, 9 + L, bc)
+    guess = 0.01 * rand_unknowns(L, bc, 4)
+    mg = setup(hn, L, coef, bc, prec=prec, coarse_L=coarse_L)
+    try:
+        got = [hn.hn_mg_solve(mg, L, b), hn.hn_mg_solve(mg, L, b, guess.copy(), True)]
+        hn.hn_mg_set_tuning(mg, *STEPS)
+        want = [hn.hn_mg_solve(mg, L, b), hn.hn_mg_solve(mg, L, b, guess.copy(), True)]
+        for (x, st, status), (y, su, expected) in zip(got, want):
+            assert status == expected == hn.HN_OK
+            np.testing.assert_array_equal(x, y)
+            assert (st["cycles"], st["relres"]) == (su["cycles"], su["relres"])
+    finally:
+        hn.hn_mg_destroy(mg)
