@@ -535,7 +535,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   // the control kernel's groups: as many as the largest problem's norm sum has
   const int ctl_groups = (int)((pitch_of(Lmax) / kTile + kSumGroup - 1) / kSumGroup);
   take(sizeof(double) * (size_t)cap * ctl_groups);
-  take(sizeof(unsigned) * (size_t)cap * ctl_groups);
+  take(sizeof(unsigned) * (size_t)cap * (ctl_groups + 1));
   take(sizeof(int) * plan_ints());
   take(sizeof(TileList) * (kMaxLevel + 1));
   take(sizeof(unsigned long long) * 3);
@@ -562,7 +562,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   dTaken_ = b.take<unsigned>(4);
   dLaunches_ = b.take<unsigned long long>(1);
   double* gsum = b.take<double>((size_t)cap * ctl_groups);
-  unsigned* gticket = b.take<unsigned>((size_t)cap * ctl_groups);
+  unsigned* gticket = b.take<unsigned>((size_t)cap * (ctl_groups + 1));
   dPlan_ = b.take<int>(plan_ints());
   dLists_ = b.take<TileList>(kMaxLevel + 1);
   dBar_ = b.take<unsigned long long>(3);
@@ -920,7 +920,8 @@ bool Engine::sweep_level(int l) const {
 bool Engine::march_level(int l) const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
   return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !tune_.staged &&
-         !tune_.fuse_up && mid_top() <= T && l >= (cap_ == 1 ? kMarchSoloLevel : kMarchMinLevel);
+         !tune_.fuse_up && mid_top() <= T && l >= (cap_ == 1 ? kMarchSoloLevel : kMarchMinLevel) &&
+         (cap_ == 1 || T + 1 >= kMarchMinLevel);
 }
 
 // The levels of the tail in one block's shared memory (k_small) in place of the cluster kernel, under the
@@ -948,11 +949,23 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   for (int l = Lmax_; l > std::max(T, M); --l) {
     // a finest level: lagged check (the PCG preconditioner's cycle has none)
     const bool top = prm_.solver != SOLVER_PCG && is_top(l);
+    if (march_level(l) && cap_ != 1) {
+      // the finest level of every problem and its check, then level by level the problems above it
+      if (l == Lmax_) {
+        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, 0, T, want, 0, s));
+        if (prm_.solver != SOLVER_PCG) {
+          HN_LAUNCH(KC_CHECK, l, launch_march_check_group(E_, T, want, s));
+          HN_TRY(after_check());
+        }
+      } else {
+        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, l, T, want, 0, s));
+      }
+      continue;
+    }
     if (march_level(l)) {
-      HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, 0, 0, s));
+      HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march(E_, lists_[l], l, want, 0, 0, s));
       if (top) {
-        HN_LAUNCH(KC_CHECK, l, launch_march_check(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, s));
-        if (cap_ != 1) HN_LAUNCH(KC_CONTROL, l, launch_control(E_, CTRL_PRE, s, l));
+        HN_LAUNCH(KC_CHECK, l, launch_march_check(E_, lists_[l], l, want, s));
         HN_TRY(after_check());
       }
       continue;
@@ -997,7 +1010,8 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   int e_sel = 0;                           // buffer of the coarse iterate (the tail's: 0)
   for (int l = std::max(T, M) + 1; l <= Lmax_; ++l) {
     if (march_level(l)) {                  // prolongation and both post-smoothing steps, buffer 1 to 0
-      HN_LAUNCH(KC_SWEEP_UP, l, launch_march(E_, lists_[l], dPlan_ + (size_t)l * cap_, l, want, 1, e_sel, s));
+      if (cap_ != 1) HN_LAUNCH(KC_SWEEP_UP, l, launch_march_group(E_, l == Lmax_ ? 0 : l, T, want, 1, s));
+      else HN_LAUNCH(KC_SWEEP_UP, l, launch_march(E_, lists_[l], l, want, 1, e_sel, s));
       e_sel = 0;
       continue;
     }

@@ -203,8 +203,8 @@ struct EngineDev {
   int ctl_groups;              // blocks per problem of the control kernel (groups of the largest
                                // problem's norm partial sum)
   double* gsum;                // [nprob * ctl_groups] group sums of the control kernel
-  unsigned* gticket;           // [nprob * ctl_groups] blocks of a problem's control launch (of a group's
-                               // check) that finished
+  unsigned* gticket;           // [nprob * (ctl_groups + 1)] blocks of a problem's group (groups of the problem)
+                               // that finished their part of a norm sum
   unsigned* ticket;            // blocks of a first smoothing step with a fused check that finished
   unsigned long long* gbar;    // [3] grid barriers of the persistent kernels: arrivals of the
                                // down kernel, of the up kernel, barrier actions completed
@@ -264,20 +264,20 @@ SweepGeom sweep_geom(int level);
 size_t sweep_smem_bytes(int prec, const SweepGeom& g);
 cudaError_t launch_sweep_down(const EngineDev& E, TileList tl, int level, int want, int top, cudaStream_t s);
 cudaError_t launch_sweep_up(const EngineDev& E, TileList tl, int level, int want, int e_sel, cudaStream_t s);
-// Marching sweeps (k_march.cu) of level `level` for FP32 / FP16 hierarchies with V(2,2) cycles, levels
-// from kMarchMinLevel: the down part (both smoothing steps, from the zero iterate or from buffer 0 of a
+// Marching sweeps (k_march.cu) for FP32 / FP16 hierarchies with V(2,2) cycles, levels from
+// kMarchMinLevel: the down part (both smoothing steps, from the zero iterate or from buffer 0 of a
 // problem's own finest level, whose residual squares it leaves in the level's defect array; the defect,
-// the restriction) leaves the iterate in buffer 1, the up part (prolongation from the coarse iterate in
-// buffer e_sel, both smoothing steps) leaves it in buffer 0.  slots: the level's members (unused by an
-// engine of one problem).  launch_march_check after the down part of a level that may be a finest one:
-// the norm partials from the squares, and the whole lagged check of an engine of one problem (others:
-// CTRL_PRE).
+// the restriction) leaves the iterate in buffer 1, the up part (prolongation from the coarse iterate, in
+// buffer e_sel, both smoothing steps) leaves it in buffer 0.  launch_march: level `level` of an engine of
+// one problem; launch_march_group: of all problems that have a finer level, or (level 0) every problem's
+// own finest level above T.  launch_march_check / _group: the lagged check after the down part of the
+// finest level.
 constexpr int kMarchMinLevel = 6;
 constexpr int kMarchSoloLevel = 9;   // an engine of one problem: from here
-cudaError_t launch_march(const EngineDev& E, const TileList& tl, const int* slots, int level, int want, int up,
-                         int e_sel, cudaStream_t s);
-cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, const int* slots, int level, int want,
-                               cudaStream_t s);
+cudaError_t launch_march(const EngineDev& E, const TileList& tl, int level, int want, int up, int e_sel, cudaStream_t s);
+cudaError_t launch_march_group(const EngineDev& E, int level, int T, int want, int up, cudaStream_t s);
+cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, int level, int want, cudaStream_t s);
+cudaError_t launch_march_check_group(const EngineDev& E, int T, int want, cudaStream_t s);
 // x_sel: bit 0 the fine buffer corrected in place, bit 1 the buffer of the coarse iterate
 cudaError_t launch_prolong(const EngineDev& E, TileList tl, int level, int want, int x_sel,
                            int grid, cudaStream_t s);

@@ -2529,7 +2529,7 @@ __device__ bool control_sum(const EngineDev& E, int p, int j, const double* part
   if (threadIdx.x == 0) {
     E.gsum[(long long)p * E.ctl_groups + j] = g;
     __threadfence();
-    last = atomicAdd(E.gticket + p, 1u) == (unsigned)(ng - 1);
+    last = atomicAdd(E.gticket + (long long)p * (E.ctl_groups + 1), 1u) == (unsigned)(ng - 1);
   }
   __syncthreads();
   if (!last) return false;
@@ -2538,7 +2538,7 @@ __device__ bool control_sum(const EngineDev& E, int p, int j, const double* part
     double t = 0.0;
     for (int q = 0; q < ng; ++q) t += __ldcg(E.gsum + (long long)p * E.ctl_groups + q);
     *sum = t;
-    E.gticket[p] = 0u;                          // ready for the next launch
+    E.gticket[(long long)p * (E.ctl_groups + 1)] = 0u;   // ready for the next launch
   }
   return true;
 }

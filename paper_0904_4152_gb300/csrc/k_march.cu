@@ -36,7 +36,7 @@ namespace hn {
 
 namespace {
 
-constexpr int kMaxActive = 1024;         // problems a block can list (more: all are walked)
+constexpr int kListMax = 1024;           // problems a block lists at a time
 constexpr int kWarps = 2;                // independent warps of a block
 constexpr int kSlots = 4;                // rows of the ring: one in use, three on their way
 enum { DOWN_ZERO = 0, DOWN = 1, UP = 2 };
@@ -551,9 +551,9 @@ __host__ __device__ inline Geom march_strips(int L, int up) {
   g.rows = g.R;
   return g;
 }
-// Rows of a chunk so that S strips (of all problems) fill whole waves of G warps: a chunk of r rows
-// costs r + 6 iterations and about 6 to start
-__host__ __device__ inline void march_chunks(Geom& g, unsigned S, unsigned G) {
+// Rows of a chunk so that S strips fill whole waves of G warps: a chunk of r rows costs r + 6 iterations
+// and about 6 to start
+inline void march_chunks(Geom& g, unsigned S, unsigned G) {
   unsigned best = 0xffffffffu;
   for (unsigned w = 1; w <= 3; ++w) {
     unsigned c = w * G / S;
@@ -590,6 +590,19 @@ __device__ __forceinline__ void make_view(View& v, const LevelDev& d, const Leve
   __syncwarp();
 }
 
+__device__ __forceinline__ Item item_of(const Geom& g, int s) {
+  const int ch = s / g.strips;
+  Item it;
+  it.c0 = (s - ch * g.strips) * g.own;
+  it.r0 = ch * g.rows;
+  it.r1 = min(g.R, it.r0 + g.rows);
+  return it;
+}
+// the lane's columns belong to the widened strip (and to the level)
+__device__ __forceinline__ bool live_lane(const Strip& st, const Item& it, int lane, int level) {
+  return 4 * lane < st.own + 2 * st.side && it.c0 + 4 * lane < (1 << level) + 2 * st.side;
+}
+
 template <class Pol, bool UPWARD>
 __device__ __forceinline__ void sweep(const View& v, const Strip& st, const Item& it, unsigned char* ring, bool early, bool zero,
                                       int lane, bool live) {
@@ -603,102 +616,181 @@ __device__ __forceinline__ void sweep(const View& v, const Strip& st, const Item
   }
 }
 
-// One launch of a level's down or up part.  An engine of one problem passes its descriptors and the
-// cut of the level by value; otherwise the blocks list the level's members in phase `want` (slots:
-// the level's members, from the engine's plan) and share their strips and chunks among their warps.
-// e_sel (up): the coarse iterate's buffer.
+// A level's down or up part for an engine of one problem, which passes its descriptors and the cut of the
+// level by value.  e_sel (up): the coarse iterate's buffer.
 template <class Pol, bool UPWARD>
-__global__ void __launch_bounds__(kWarps * 32, 4) k_march(EngineDev E, TileList tl, const int* slots, int level, int want,
-                                                       int e_sel, Geom geom) {
+__global__ void __launch_bounds__(kWarps * 32, 4) k_march(EngineDev E, TileList tl, int level, int want, int e_sel, Geom g) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float scale[kWarps][8];
   __shared__ View views[kWarps];
-  __shared__ unsigned short active[kMaxActive];
-  __shared__ int s_active;
   pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char* ring = smem + warp * kSlots * slot_bytes<Pol>();
   const int gw = (int)blockIdx.x * kWarps + warp, G = (int)gridDim.x * kWarps;
-  const bool solo = tl.solo_tiles > 0;
   View& v = views[warp];                          // (in shared memory: its pointers take no registers)
-  Geom g = geom;
-  Strip st;
-  st.side = UPWARD ? 4 : 8;
-  st.own = g.own;
-  auto item = [&](int s) {
-    Item it;
-    const int ch = s / g.strips;
-    it.c0 = (s - ch * g.strips) * g.own;
-    it.r0 = ch * g.rows;
-    it.r1 = min(g.R, it.r0 + g.rows);
-    return it;
-  };
-  if (solo) {
-    if (tl.solo_c.n == 0) return;                 // (the coarsest level: nothing below it)
-    if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
-    // (a zero iterate leaves no squares)
-    make_view<Pol, UPWARD>(v, tl.solo_d, tl.solo_c, e_sel, scale[warp], E.prm.solver != SOLVER_PCG);
-    const int items = g.strips * g.chunks;
-    if (gw >= items) return;
-    Item it = item(gw);
-    // the bands and omega / D of the first rows are constant: fetched before the preceding launch ends
-    const bool wide = 4 * lane < st.own + 2 * st.side;
-    auto live = [&](const Item& t) { return wide && t.c0 + 4 * lane < (1 << level) + 2 * st.side; };
-    if (live(it)) {
-      const int first = it.r0 - (UPWARD ? 2 : 3), last = it.r1 + (UPWARD ? 1 : 2);
-      Cursor<Pol> cur;
-      cur.start(v, (first << level) + it.c0 + 4 * lane - st.side, 0);
-      for (int q = 0; q < kSlots && first + q <= last; ++q, cur.next(1 << level))
-        cur.constants(v.stride, smem_u32(ring) + q * slot_bytes<Pol>(), lane);
-    }
-    pdl_wait();
-    const ProbState& S = E.S[0];
-    if (S.phase != want) {
-      copy_commit();
-      copy_wait<0>();
-      return;
-    }
-    const bool zero = tl.solo_L > level || S.zero_top;
-    bool early = true;
-    for (int s = gw; s < items; s += G) {
-      it = item(s);
-      sweep<Pol, UPWARD>(v, st, it, ring, early, zero, lane, live(it));
-      early = false;
-    }
-    return;
+  if (tl.solo_c.n == 0) return;                   // (the coarsest level, or one that the problem does not have)
+  if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
+  // (a zero iterate leaves no squares)
+  make_view<Pol, UPWARD>(v, tl.solo_d, tl.solo_c, e_sel, scale[warp], E.prm.solver != SOLVER_PCG);
+  const int items = g.strips * g.chunks;
+  if (gw >= items) return;
+  const Strip st{g.own, UPWARD ? 4 : 8};
+  Item it = item_of(g, gw);
+  // the bands and omega / D of the first rows are constant: fetched before the preceding launch ends
+  if (live_lane(st, it, lane, level)) {
+    const int first = it.r0 - (UPWARD ? 2 : 3), last = it.r1 + (UPWARD ? 1 : 2);
+    Cursor<Pol> cur;
+    cur.start(v, (first << level) + it.c0 + 4 * lane - st.side, 0);
+    for (int q = 0; q < kSlots && first + q <= last; ++q, cur.next(1 << level))
+      cur.constants(v.stride, smem_u32(ring) + q * slot_bytes<Pol>(), lane);
   }
   pdl_wait();
-  const int tiles = (int)((((1LL << level) + 1) * ((1LL << level) + 1) + kTile - 1) / kTile);
-  const int n = *tl.count / tiles;
-  const bool compact = n <= kMaxActive;
-  if (compact && threadIdx.x < 32) {
-    int have = 0;
-    for (int b = 0; b < n; b += 32) {
-      const int m = b + lane;
-      const int p = m < n ? slots[m] : 0;
-      const bool on = m < n && dbg_item(E, p, 0, level, __LINE__) && E.S[p].phase == want && E.P[p].coarse < level;
-      const unsigned mask = __ballot_sync(kFull, on);
-      if (on) active[have + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)p;
-      have += __popc(mask);
+  const ProbState& S = E.S[0];
+  if (S.phase != want) {
+    copy_commit();
+    copy_wait<0>();
+    return;
+  }
+  const bool zero = tl.solo_L > level || S.zero_top;
+  for (int s = gw; s < items; s += G) {
+    it = item_of(g, s);
+    sweep<Pol, UPWARD>(v, st, it, ring, s == gw, zero, lane, live_lane(st, it, lane, level));
+  }
+}
+
+// The problems of an engine that a launch serves: those in phase `want` (< 0: in any) whose finest level is
+// above `above`, at most kListMax of the slots from `base`, in slot order, with the levels they are taken at (level,
+// or 0: their own finest).  The whole block; returns the number of problems.  Every block of a launch has
+// to find the same list, so a launch that changes phases lists problems in any.
+struct Served {
+  unsigned short slot[kListMax];
+  unsigned char level[kListMax];
+  int start[kListMax + 1];
+  int count[32];
+};
+__device__ int list_served(const EngineDev& E, Served& q, int base, int want, int above, int level) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+  const int n = min(kListMax, E.nprob - base);
+  // slots of a warp: a contiguous share, read in one go (the loads of a round do not depend on each other)
+  const int share = (n + nw * 32 - 1) / (nw * 32);
+  const int lo = warp * share * 32;
+  unsigned take = 0;
+  for (int k = 0; k < share; ++k) {
+    const int p = lo + k * 32 + lane;
+    const bool on = p < n && (want < 0 || E.S[base + p].phase == want) && E.P[base + p].L > above;
+    take |= on ? 1u << k : 0u;
+  }
+  int mine = 0;
+  for (int k = 0; k < share; ++k) mine += __popc(__ballot_sync(kFull, (take >> k) & 1u));
+  if (lane == 0) q.count[warp] = mine;
+  __syncthreads();
+  int at = 0, total = 0;
+  for (int w = 0; w < nw; ++w) {
+    if (w < warp) at += q.count[w];
+    total += q.count[w];
+  }
+  for (int k = 0; k < share; ++k) {
+    const bool on = (take >> k) & 1u;
+    const unsigned m = __ballot_sync(kFull, on);
+    if (on) {
+      const int i = at + __popc(m & ((1u << lane) - 1u)), p = base + lo + k * 32 + lane;
+      q.slot[i] = (unsigned short)p;
+      q.level[i] = (unsigned char)(level ? level : E.P[p].L);
     }
-    if (lane == 0) s_active = have;
+    at += __popc(m);
   }
   __syncthreads();
-  const int nact = compact ? s_active : n;
-  if (nact == 0) return;
-  march_chunks(g, (unsigned)(nact * g.strips), (unsigned)G);
-  const int per = g.strips * g.chunks;
-  for (long long q = gw; q < (long long)nact * per; q += G) {
-    const int m = (int)(q / per), s = (int)(q - (long long)m * per);
-    const int p = compact ? active[m] : slots[m];
-    const ProbState& S = E.S[p];
-    const ProblemDev& P = E.P[p];
-    if (!compact && (!dbg_item(E, p, 0, level, __LINE__) || S.phase != want || P.coarse >= level)) continue;
-    const LevelDev& d = P.lev[level];
-    make_view<Pol, UPWARD>(v, d, P.lev[level - 1], e_sel, scale[warp], E.prm.solver != SOLVER_PCG);
-    const Item it = item(s);
-    const bool live = 4 * lane < st.own + 2 * st.side && it.c0 + 4 * lane < (1 << level) + 2 * st.side;
-    sweep<Pol, UPWARD>(v, st, it, ring, false, P.L > level || S.zero_top, lane, live);
+  return total;
+}
+// running numbers of the problems' work items (items: of a level; 32-bit arithmetic only: a round of 32
+// problems is on every block's way to its first load); the whole block; returns their sum
+template <class F>
+__device__ int number_items(Served& q, int n, F&& items) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    int run = 0;
+    for (int b = 0; b < n; b += 32) {
+      const int c = b + lane < n ? items((int)q.level[b + lane]) : 0;
+      int s = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, s, o);
+        if (lane >= o) s += t;
+      }
+      if (b + lane < n) q.start[b + lane] = run + s - c;
+      run += __shfl_sync(kFull, s, 31);
+    }
+    if (lane == 0) q.start[n] = run;
+  }
+  __syncthreads();
+  return q.start[n];
+}
+// the problem of work item `it`
+__device__ __forceinline__ int served_of(const Served& q, int n, int it) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (q.start[mid] <= it) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// The down or up part of level `level` for the problems with a finer level, or (level 0) of every problem's
+// own finest level above the tail level T, in one launch: the strips of all problems in the phase are cut
+// into chunks of one height, so that they fill one wave of warps.
+template <class Pol, bool UPWARD>
+__global__ void __launch_bounds__(kWarps * 32, 4) k_march_group(EngineDev E, int level, int T, int want) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ float scale[kWarps][8];
+  __shared__ View views[kWarps];
+  __shared__ Served q;
+  __shared__ int2 cut[kMaxLevel + 1];             // strips and rows of a level
+  __shared__ int hist[kMaxLevel + 1], s_rows;
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char* ring = smem + warp * kSlots * slot_bytes<Pol>();
+  const int gw = (int)blockIdx.x * kWarps + warp, G = (int)gridDim.x * kWarps;
+  View& v = views[warp];
+  if (threadIdx.x <= kMaxLevel) {
+    const Geom g = march_strips((int)threadIdx.x, UPWARD);
+    cut[threadIdx.x] = make_int2(g.strips, g.R);
+  }
+  pdl_wait();
+  for (int base = 0; base < E.nprob; base += kListMax) {
+    const int n = list_served(E, q, base, want, level ? level : T, level);
+    if (n == 0) continue;
+    // one height for all chunks: the smallest of 32 candidates that takes no more items than warps
+    if (threadIdx.x < kMaxLevel + 1) hist[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&hist[q.level[i]], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      int total = 0;
+      for (int l = kMarchMinLevel; l <= kMaxLevel; ++l) total += hist[l] * cut[l].x * cut[l].y;
+      const int least = max(2, (total + G - 1) / G), rows = least + lane * max(1, least / 16);
+      int items = 0;
+      for (int l = kMarchMinLevel; l <= kMaxLevel; ++l)
+        if (hist[l]) items += hist[l] * cut[l].x * ((cut[l].y + rows - 1) / rows);
+      const unsigned fits = __ballot_sync(kFull, items <= G);
+      const int best = fits ? __ffs(fits) - 1 : 31;
+      if (lane == best) s_rows = rows;
+    }
+    __syncthreads();
+    const int rows = s_rows;
+    const int items = number_items(q, n, [&](int l) { return cut[l].x * ((cut[l].y + rows - 1) / rows); });
+    for (int it = gw; it < items; it += G) {
+      const int m = served_of(q, n, it), p = q.slot[m], l = q.level[m];
+      if (!dbg_item(E, p, 0, l, __LINE__)) continue;
+      const ProblemDev& P = E.P[p];
+      const bool zero = P.L > l || E.S[p].zero_top;
+      make_view<Pol, UPWARD>(v, P.lev[l], P.lev[l - 1], 0, scale[warp], E.prm.solver != SOLVER_PCG);
+      Geom g = march_strips(l, UPWARD);
+      g.rows = rows;
+      const Strip st{g.own, UPWARD ? 4 : 8};
+      const Item t = item_of(g, it - q.start[m]);
+      sweep<Pol, UPWARD>(v, st, t, ring, false, zero, lane, live_lane(st, t, lane, l));
+    }
+    __syncthreads();
   }
 }
 
@@ -728,70 +820,94 @@ __device__ __forceinline__ float2 tile_pairs(const float* r, int tile0, int ntil
   return q[0];
 }
 
-// An engine of one problem takes the lagged check here as well: the last block of a group of kSumGroup
-// tiles sums the group, the last group adds the groups in order and decides.  Others: blocks of a member
-// in turn (nb blocks each), and the control launch sums.
-__global__ void __launch_bounds__(256) k_march_check(EngineDev E, TileList tl, const int* slots, int level, int want, int nb) {
+// The lagged check of problem p with finest level `level`, by the blocks that hold its squares: block `blk`
+// of nb that serve group j of the problem's tiles sums its tiles; the last block of a group sums the
+// group; the last group adds the groups in order and decides.  want: the phase of the cycle.
+__device__ void check_part(const EngineDev& E, int p, const float* squares, int level, int j, int blk, int nb, int want, double* sh) {
+  __shared__ int s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tiles = fine_tiles(level), groups = sum_groups(tiles);
+  double* part = E.partial + E.fine_off[p];
+  const int lo = j * kSumGroup, hi = min(tiles, lo + kSumGroup);
+  for (int t = lo + (blk * 8 + warp) * 32; t < hi; t += nb * 256) {
+    const float2 q = tile_pairs(squares, t, hi);
+    if (t + lane < hi) store_partial(part + t + lane, q);
+  }
+  unsigned* ticket = E.gticket + (long long)p * (E.ctl_groups + 1);
+  double* gsum = E.gsum + (long long)p * E.ctl_groups;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket + j, 1u) == (unsigned)nb - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const double g = group_partial_sum(part, tiles, j, sh, true);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ticket[j] = 0u;
+    s_last = 1;
+    if (groups > 1) {
+      gsum[j] = g;
+      __threadfence();
+      s_last = atomicAdd(ticket + E.ctl_groups, 1u) == (unsigned)groups - 1u;
+    }
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  double sum = g;
+  if (groups > 1) {
+    __threadfence();
+    sum = 0.0;
+    for (int b = 0; b < groups; b += 32) {        // group sums in group order, as problem_norm_sum
+      const double mine = b + lane < groups ? __ldcg(gsum + b + lane) : 0.0;
+      for (int k = 0; k < 32 && b + k < groups; ++k) sum += __shfl_sync(kFull, mine, k);
+    }
+  }
+  if (threadIdx.x == 0) {
+    ProbState& st = E.S[p];
+    if (groups > 1) ticket[E.ctl_groups] = 0u;
+    pre_check(st, E.prm, sqrt(sum));
+    if (st.phase == want) cond_set(E.prm.cond, 0, 1u);
+  }
+}
+
+// after the down part of the finest level: of an engine of one problem, nb blocks per group ...
+__global__ void __launch_bounds__(256) k_march_check(EngineDev E, TileList tl, int level, int want, int nb) {
   pdl_start();
   __shared__ double sh[32];
-  __shared__ int s_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tiles = fine_tiles(level);
-  if (tl.solo_tiles == 0) {
-    const int n = *tl.count / tiles;
-    for (int m = (int)blockIdx.x / nb; m < n; m += (int)gridDim.x / nb) {
-      const int p = slots[m];
-      if (!dbg_item(E, p, 0, level, __LINE__)) continue;
-      const ProbState& S = E.S[p];
-      const ProblemDev& P = E.P[p];
-      if (S.phase != want || P.L != level || S.zero_top) continue;
-      const float* r = static_cast<const float*>(P.lev[level].r);
-      double* part = E.partial + E.fine_off[p];
-      for (int t = (((int)blockIdx.x % nb) * 8 + warp) * 32; t < tiles; t += nb * 256) {
-        const float2 q = tile_pairs(r, t, tiles);
-        if (t + lane < tiles) store_partial(part + t + lane, q);
-      }
-    }
-    return;
-  }
-  ProbState& st = E.S[0];
+  const ProbState& st = E.S[0];
   if (st.phase != want) return;
   if (tl.solo_L != level || st.zero_top) {        // nothing to check: the cycle goes on
     if (blockIdx.x == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 0, 1u);
     return;
   }
-  // nb blocks per group
-  const int groups = sum_groups(tiles), j = (int)blockIdx.x / nb;
-  const int lo = j * kSumGroup, hi = min(tiles, lo + kSumGroup);
-  for (int t = lo + (((int)blockIdx.x % nb) * 8 + warp) * 32; t < hi; t += nb * 256) {
-    const float2 q = tile_pairs(static_cast<const float*>(tl.solo_d.r), t, hi);
-    if (t + lane < hi) store_partial(E.partial + t + lane, q);
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(E.gticket + j, 1u) == (unsigned)nb - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const double g = group_partial_sum(E.partial, tiles, j, sh, true);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    E.gticket[j] = 0u;
-    E.gsum[j] = g;
-    __threadfence();
-    s_last = atomicAdd(E.ticket, 1u) == (unsigned)groups - 1u;
-  }
-  __syncthreads();
-  if (!s_last || threadIdx.x >= 32) return;
-  __threadfence();
-  double sum = 0.0;
-  for (int b = 0; b < groups; b += 32) {          // group sums in group order, as problem_norm_sum
-    const double mine = b + lane < groups ? __ldcg(E.gsum + b + lane) : 0.0;
-    for (int q = 0; q < 32 && b + q < groups; ++q) sum += __shfl_sync(kFull, mine, q);
-  }
-  if (threadIdx.x == 0) {
-    pre_check(st, E.prm, sqrt(groups == 1 ? g : sum));
-    if (st.phase == want) cond_set(E.prm.cond, 0, 1u);
-    *E.ticket = 0u;
+  check_part(E, 0, static_cast<const float*>(tl.solo_d.r), level, (int)blockIdx.x / nb, (int)blockIdx.x % nb, nb, want, sh);
+}
+// ... and of all problems whose finest level is above the tail, one block per 1024 tiles at most
+__global__ void __launch_bounds__(256) k_march_check_group(EngineDev E, int T, int want) {
+  pdl_start();
+  __shared__ double sh[32];
+  __shared__ Served q;
+  auto blocks = [T](int l) {                      // of a problem: whole groups of kSumGroup tiles
+    const int tiles = fine_tiles(l);
+    return l <= T ? 1 : sum_groups(tiles) * ((min(tiles, kSumGroup) + 1023) / 1024);
+  };
+  for (int base = 0; base < E.nprob; base += kListMax) {
+    const int n = list_served(E, q, base, -1, HN_MIN_LEVEL - 1, 0);
+    if (n == 0) continue;
+    const int items = number_items(q, n, blocks);
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+      const int m = served_of(q, n, it), p = q.slot[m], l = q.level[m], blk = it - q.start[m];
+      // (a problem leaves the phase only after every block of its check has counted itself in)
+      if (!dbg_item(E, p, 0, l, __LINE__) || __ldcg(&E.S[p].phase) != want) continue;
+      if (l <= T || E.S[p].zero_top) {            // no check (or the tail's own): the cycle goes on
+        if (blk == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 0, 1u);
+        continue;
+      }
+      const int nb = (min(fine_tiles(l), kSumGroup) + 1023) / 1024;
+      check_part(E, p, static_cast<const float*>(E.P[p].lev[l].r), l, blk / nb, blk % nb, nb, want, sh);
+      __syncthreads();
+    }
+    __syncthreads();
   }
 }
 
@@ -812,53 +928,64 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int threads, size_t sme
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// resident blocks per SM of a marching kernel (its shared memory allowed on the first call); 0: none
+template <class K>
+int march_resident(K kern, int smem) {
+  int b = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kWarps * 32, smem) != cudaSuccess)
+    return 0;
+  return b;
+}
+
 template <class Pol, bool UPWARD>
-cudaError_t launch_march_t(const EngineDev& E, const TileList& tl, const int* slots, int level, int want, int e_sel,
-                           cudaStream_t s) {
-  auto kern = k_march<Pol, UPWARD>;
+cudaError_t launch_march_t(const EngineDev& E, const TileList& tl, int level, int want, int e_sel, cudaStream_t s) {
   constexpr int smem = kWarps * kSlots * slot_bytes<Pol>();
-  static const int per_sm = [&] {
-    int b = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kWarps * 32, smem) != cudaSuccess)
-      return 0;
-    return b;
-  }();
+  static const int per_sm = march_resident(k_march<Pol, UPWARD>, smem);
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  int grid = per_sm * sm_count();
   Geom g = march_strips(level, UPWARD ? 1 : 0);
-  if (tl.solo_tiles > 0) {
-    march_chunks(g, (unsigned)g.strips, (unsigned)(grid * kWarps));
-    grid = std::min(grid, (g.strips * g.chunks + kWarps - 1) / kWarps);
-  }
-  return launch_pdl(kern, grid, kWarps * 32, smem, s, E.pdl, E, tl, slots, level, want, e_sel, g);
+  march_chunks(g, (unsigned)g.strips, (unsigned)(per_sm * sm_count() * kWarps));
+  const int grid = std::min(per_sm * sm_count(), (g.strips * g.chunks + kWarps - 1) / kWarps);
+  return launch_pdl(k_march<Pol, UPWARD>, grid, kWarps * 32, smem, s, E.pdl, E, tl, level, want, e_sel, g);
+}
+
+template <class Pol, bool UPWARD>
+cudaError_t launch_group_t(const EngineDev& E, int level, int T, int want, cudaStream_t s) {
+  constexpr int smem = kWarps * kSlots * slot_bytes<Pol>();
+  static const int per_sm = march_resident(k_march_group<Pol, UPWARD>, smem);
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  return launch_pdl(k_march_group<Pol, UPWARD>, per_sm * sm_count(), kWarps * 32, smem, s, E.pdl, E, level, T, want);
 }
 
 }  // namespace
 
-cudaError_t launch_march(const EngineDev& E, const TileList& tl, const int* slots, int level, int want, int up, int e_sel,
-                         cudaStream_t s) {
+cudaError_t launch_march(const EngineDev& E, const TileList& tl, int level, int want, int up, int e_sel, cudaStream_t s) {
   if (level < kMarchMinLevel) return cudaErrorInvalidValue;
   if (E.prm.prec == P32)
-    return up ? launch_march_t<F32, true>(E, tl, slots, level, want, e_sel, s)
-              : launch_march_t<F32, false>(E, tl, slots, level, want, e_sel, s);
+    return up ? launch_march_t<F32, true>(E, tl, level, want, e_sel, s) : launch_march_t<F32, false>(E, tl, level, want, e_sel, s);
   if (E.prm.prec == P16)
-    return up ? launch_march_t<F16, true>(E, tl, slots, level, want, e_sel, s)
-              : launch_march_t<F16, false>(E, tl, slots, level, want, e_sel, s);
+    return up ? launch_march_t<F16, true>(E, tl, level, want, e_sel, s) : launch_march_t<F16, false>(E, tl, level, want, e_sel, s);
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, const int* slots, int level, int want,
-                               cudaStream_t s) {
-  // 256 tiles a block: per group of an engine of one problem, else per member, in one wave of blocks
+cudaError_t launch_march_group(const EngineDev& E, int level, int T, int want, int up, cudaStream_t s) {
+  if ((level ? level : T + 1) < kMarchMinLevel) return cudaErrorInvalidValue;
+  if (E.prm.prec == P32)
+    return up ? launch_group_t<F32, true>(E, level, T, want, s) : launch_group_t<F32, false>(E, level, T, want, s);
+  if (E.prm.prec == P16)
+    return up ? launch_group_t<F16, true>(E, level, T, want, s) : launch_group_t<F16, false>(E, level, T, want, s);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, int level, int want, cudaStream_t s) {
+  // 256 tiles a block, whole groups
   const int tiles = (int)(pitch_of(level) / kTile);
-  if (tl.solo_tiles > 0) {
-    const int groups = (tiles + kSumGroup - 1) / kSumGroup, nb = (std::min(tiles, kSumGroup) + 255) / 256;
-    return launch_pdl(k_march_check, groups * nb, 256, 0, s, E.pdl, E, tl, slots, level, want, nb);
-  }
-  const int wave = 4 * sm_count(), nb = std::min((tiles + 255) / 256, wave);
-  const int members = std::max(1, std::min(E.nprob, wave / nb));
-  return launch_pdl(k_march_check, members * nb, 256, 0, s, E.pdl, E, tl, slots, level, want, nb);
+  const int groups = (tiles + kSumGroup - 1) / kSumGroup, nb = (std::min(tiles, kSumGroup) + 255) / 256;
+  return launch_pdl(k_march_check, groups * nb, 256, 0, s, E.pdl, E, tl, level, want, nb);
+}
+
+cudaError_t launch_march_check_group(const EngineDev& E, int T, int want, cudaStream_t s) {
+  return launch_pdl(k_march_check_group, 2 * sm_count(), 256, 0, s, E.pdl, E, T, want);
 }
 
 }  // namespace hn
