@@ -202,36 +202,22 @@ hn_status validate_opts(const hn_mg_opts& o, int L) {
 
 namespace {
 
-// the work lists of Engine::set_members: block row y = level (items and chunks), y = kMaxLevel + 1
-// the fine list
-__global__ void __launch_bounds__(256) k_work_lists(WorkListOut o, const int* slots, const int* fslots,
-                                                    const int* foff, int cap) {
+// the work lists of Engine::set_members: block row y = level
+__global__ void __launch_bounds__(256) k_work_lists(WorkListOut o, const int* slots, int cap) {
   const int l = blockIdx.y;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l <= kMaxLevel) {
-    const int n = o.n[l], nt = o.nt[l];
-    if (n == 0) return;
-    const int cpl = (nt + kChunkTiles - 1) / kChunkTiles;
-    for (long long i = i0; i < (long long)n * nt; i += stride) {
-      const int k = (int)(i / nt);
-      o.items[l][i] = make_int2(slots[(size_t)l * cap + k], (int)(i - (long long)k * nt));
-    }
-    for (long long j = i0; j < (long long)n * cpl; j += stride) {
-      const int k = (int)(j / cpl);
-      const int t = (int)(j - (long long)k * cpl) * kChunkTiles;
-      o.chunks[l][j] = make_int4(slots[(size_t)l * cap + k], t, min(kChunkTiles, nt - t), 0);
-    }
-  } else {
-    const int nf = o.nfine;
-    for (long long i = i0; i < foff[nf]; i += stride) {
-      int lo = 0, hi = nf - 1;                      // the member k with foff[k] <= i < foff[k + 1]
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (foff[mid] <= i) lo = mid; else hi = mid - 1;
-      }
-      o.fine[i] = make_int2(fslots[lo], (int)(i - foff[lo]));
-    }
+  const int n = o.n[l], nt = o.nt[l];
+  if (n == 0) return;
+  const int cpl = (nt + kChunkTiles - 1) / kChunkTiles;
+  for (long long i = i0; i < (long long)n * nt; i += stride) {
+    const int k = (int)(i / nt);
+    o.items[l][i] = make_int2(slots[(size_t)l * cap + k], (int)(i - (long long)k * nt));
+  }
+  for (long long j = i0; j < (long long)n * cpl; j += stride) {
+    const int k = (int)(j / cpl);
+    const int t = (int)(j - (long long)k * cpl) * kChunkTiles;
+    o.chunks[l][j] = make_int4(slots[(size_t)l * cap + k], t, min(kChunkTiles, nt - t), 0);
   }
 }
 
@@ -516,7 +502,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   take(sizeof(ProblemDev) * cap);
   take(sizeof(ProbState) * cap);
   take(sizeof(int) * cap);
-  take(sizeof(int) * (kMaxLevel + 2));
+  take(sizeof(int) * (kMaxLevel + 1));
   for (int l = 0; l <= kMaxLevel; ++l) {
     itemCap_[l] = l < (int)tiles_cap.size() ? tiles_cap[l] : 0;
     take(sizeof(int2) * (size_t)std::max<long long>(itemCap_[l], 1));
@@ -526,8 +512,6 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   take(sizeof(int) * (kMaxLevel + 1));
   take(sizeof(int) * 4);
   fineCap_ = fine_cap;
-  take(sizeof(int2) * (size_t)std::max<long long>(fine_cap, 1));
-  take(sizeof(double) * (size_t)std::max<long long>(fine_cap, 1));
   take(sizeof(double) * (size_t)std::max<long long>(fine_cap, 1));
   take(sizeof(unsigned));
   take(sizeof(unsigned) * 4);
@@ -535,7 +519,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   // the control kernel's groups: as many as the largest problem's norm sum has
   const int ctl_groups = (int)((pitch_of(Lmax) / kTile + kSumGroup - 1) / kSumGroup);
   take(sizeof(double) * (size_t)cap * ctl_groups);
-  take(sizeof(unsigned) * (size_t)cap * (ctl_groups + 1));
+  take(sizeof(unsigned) * (size_t)cap * ticket_words(ctl_groups));
   take(sizeof(int) * plan_ints());
   take(sizeof(TileList) * (kMaxLevel + 1));
   take(sizeof(unsigned long long) * 3);
@@ -548,21 +532,19 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   dP_ = b.take<ProblemDev>(cap);
   dS_ = b.take<ProbState>(cap);
   dFineOff_ = b.take<int>(cap);
-  dCounts_ = b.take<int>(kMaxLevel + 2);
+  dCounts_ = b.take<int>(kMaxLevel + 1);
   for (int l = 0; l <= kMaxLevel; ++l) {
     dItems_[l] = b.take<int2>((size_t)std::max<long long>(itemCap_[l], 1));
     dChunks_[l] = b.take<int4>((size_t)std::max<long long>(chunkCap_[l], 1));
   }
   dChunkCounts_ = b.take<int>(kMaxLevel + 1);
   dErr_ = b.take<int>(4);
-  dFine_ = b.take<int2>((size_t)std::max<long long>(fine_cap, 1));
   double* part = b.take<double>((size_t)std::max<long long>(fine_cap, 1));
-  double* part2 = b.take<double>((size_t)std::max<long long>(fine_cap, 1));
   unsigned* iter = b.take<unsigned>(1);
   dTaken_ = b.take<unsigned>(4);
   dLaunches_ = b.take<unsigned long long>(1);
   double* gsum = b.take<double>((size_t)cap * ctl_groups);
-  unsigned* gticket = b.take<unsigned>((size_t)cap * (ctl_groups + 1));
+  unsigned* gticket = b.take<unsigned>((size_t)cap * ticket_words(ctl_groups));
   dPlan_ = b.take<int>(plan_ints());
   dLists_ = b.take<TileList>(kMaxLevel + 1);
   dBar_ = b.take<unsigned long long>(3);
@@ -579,7 +561,6 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   E_.S = dS_;
   E_.fine_off = dFineOff_;
   E_.partial = part;
-  E_.partial2 = part2;
   E_.nprob = cap;
   E_.prm = prm;
   E_.active_host = dActive;
@@ -598,9 +579,6 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
     lists_[l] = TileList{dItems_[l], dCounts_ + l, dChunks_[l], dChunkCounts_ + l, (int)chunkCap_[l]};
     grid_[l] = grid_for(itemCap_[l]);
   }
-  fine_ = TileList{dFine_, dCounts_ + kMaxLevel + 1};
-  fineGrid_ = grid_for(fine_cap);
-  hCounts_.assign(kMaxLevel + 2, 0);
   members_.assign(cap, nullptr);
   return HN_OK;
 }
@@ -608,23 +586,19 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
 hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
   if ((int)slots.size() > cap_) return set_error(HN_ERR_ARG, "too many problems for the engine");
   // The work lists hold, per level, the (problem, tile) pairs of every member having that level,
-  // members in slot order; the chunk lists the same in chunks of kChunkTiles tiles; the fine list
-  // each member's tiles of its finest level.  Every member contributes the same tiles to a level,
+  // members in slot order; the chunk lists the same in chunks of kChunkTiles tiles.  Every member contributes the same tiles to a level,
   // so the host only ranks the members (O(slots)) and k_work_lists writes the pairs.
   HN_CUDA(cudaEventSynchronize(upEv_));        // the previous upload has left the staging area
   char* stage = static_cast<char*>(hStage_);
-  int* h_counts = reinterpret_cast<int*>(stage);                 // kMaxLevel + 2
-  int* h_ccounts = h_counts + (kMaxLevel + 2);                   // kMaxLevel + 1
+  int* h_counts = reinterpret_cast<int*>(stage);                 // kMaxLevel + 1
+  int* h_ccounts = h_counts + (kMaxLevel + 1);                   // kMaxLevel + 1
   int* h_fine_off = h_ccounts + (kMaxLevel + 1);                 // cap
   int* h_plan = h_fine_off + cap_;                               // plan_ints()
   int* h_slots = h_plan;                                         // (kMaxLevel + 1) x cap
-  int* h_fslots = h_slots + (size_t)(kMaxLevel + 1) * cap_;      // cap
-  int* h_foff = h_fslots + cap_;                                 // cap + 1
   ProblemDev* h_probs = reinterpret_cast<ProblemDev*>(stage + stage_probs_off());
   std::memset(h_probs, 0, sizeof(ProblemDev) * cap_);
   std::memset(h_fine_off, 0, sizeof(int) * cap_);
   WorkListOut o{};
-  int nfine = 0;
   long long fine_total = 0;
   for (int p = 0; p < (int)slots.size(); ++p) {
     hn_mg* mg = slots[p];
@@ -633,37 +607,30 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
     h_probs[p] = mg->host;
     for (int l = mg->coarse; l <= mg->L; ++l) h_slots[(size_t)l * cap_ + o.n[l]++] = p;
     h_fine_off[p] = (int)fine_total;
-    h_fslots[nfine] = p;
-    h_foff[nfine++] = (int)fine_total;
     fine_total += pitch_of(mg->L) / kTile;
   }
-  h_foff[nfine] = (int)fine_total;
-  o.nfine = nfine;
-  long long most = fine_total;
+  long long most = 0;
   for (int l = 0; l <= kMaxLevel; ++l) {
     o.nt[l] = (int)(pitch_of(l) / kTile);
     const long long items = (long long)o.n[l] * o.nt[l];
     const long long chunks = (long long)o.n[l] * ((o.nt[l] + kChunkTiles - 1) / kChunkTiles);
     if (items > itemCap_[l] || chunks > chunkCap_[l])
       return set_error(HN_ERR_ARG, "work list of level %d exceeds the engine capacity", l);
-    hCounts_[l] = h_counts[l] = (int)items;
+    h_counts[l] = (int)items;
     h_ccounts[l] = (int)chunks;
     o.items[l] = dItems_[l];
     o.chunks[l] = dChunks_[l];
     most = std::max(most, items);
   }
   if (fine_total > fineCap_) return set_error(HN_ERR_ARG, "fine work list exceeds capacity");
-  hCounts_[kMaxLevel + 1] = h_counts[kMaxLevel + 1] = (int)fine_total;
-  o.fine = dFine_;
-  HN_CUDA(cudaMemcpyAsync(dCounts_, h_counts, sizeof(int) * (kMaxLevel + 2), cudaMemcpyHostToDevice, s_));
+  HN_CUDA(cudaMemcpyAsync(dCounts_, h_counts, sizeof(int) * (kMaxLevel + 1), cudaMemcpyHostToDevice, s_));
   HN_CUDA(cudaMemcpyAsync(dChunkCounts_, h_ccounts, sizeof(int) * (kMaxLevel + 1), cudaMemcpyHostToDevice, s_));
   HN_CUDA(cudaMemcpyAsync(dFineOff_, h_fine_off, sizeof(int) * cap_, cudaMemcpyHostToDevice, s_));
   HN_CUDA(cudaMemcpyAsync(dPlan_, h_plan, sizeof(int) * plan_ints(), cudaMemcpyHostToDevice, s_));
   HN_CUDA(cudaMemcpyAsync(dP_, h_probs, sizeof(ProblemDev) * cap_, cudaMemcpyHostToDevice, s_));
   if (most > 0) {
     const int gx = (int)std::min<long long>((most + 255) / 256, 1024);
-    k_work_lists<<<dim3((unsigned)gx, kMaxLevel + 2), 256, 0, s_>>>(
-        o, dPlan_, dPlan_ + (size_t)(kMaxLevel + 1) * cap_, dPlan_ + (size_t)(kMaxLevel + 2) * cap_, cap_);
+    k_work_lists<<<dim3((unsigned)gx, kMaxLevel + 1), 256, 0, s_>>>(o, dPlan_, cap_);
     HN_CUDA(cudaGetLastError());
   }
   HN_CUDA(cudaEventRecord(upEv_, s_));
@@ -684,6 +651,7 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
     if (l > P.coarse) t.solo_c = P.lev[l - 1];
     if (l < P.L) t.solo_f = P.lev[l + 1];
   }
+  soloTiles_ = cap_ == 1 && !slots.empty() && slots[0] ? (int)(pitch_of(slots[0]->L) / kTile) : 0;
   small_ = SmallSolo{};
   if (cap_ == 1 && !slots.empty() && slots[0]) {
     const ProblemDev& P = slots[0]->host;
@@ -1042,93 +1010,48 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
 }
 
 hn_status Engine::issue_init(cudaStream_t s, cudaGraphConditionalHandle h, int use_h) {
-  HN_LAUNCH0(launch_boundary_check(E_, s));
-  HN_LAUNCH0(launch_norm_b(E_, fine_, fineGrid_, s));
-  HN_LAUNCH0(launch_control(E_, CTRL_INIT, s));
-  if (prm_.solver == SOLVER_PCG) {
-    // the initial residual r = b - A x and its check (then the first cycle preconditions it)
-    HN_LAUNCH0(launch_outer_defect(E_, fine_, fineGrid_, s));
-    HN_LAUNCH0(launch_control(E_, CTRL_OUTER, s));
-  }
-  HN_LAUNCH0(launch_summary(E_, h, use_h, 0, s));
+  // the boundary check and ||b||; CG: the initial residual r = b - A x and its check (then the first
+  // cycle preconditions it).  An engine of one problem ends the start in the last of these kernels.
+  const bool pcg = prm_.solver == SOLVER_PCG;
+  HN_LAUNCH0(launch_fine(E_, FINE_NORM_B, soloTiles_, cap_ == 1 && !pcg ? 2 : 0, h, use_h, s));
+  if (pcg) HN_LAUNCH0(launch_fine(E_, FINE_OUTER, soloTiles_, cap_ == 1 ? 2 : 0, h, use_h, s));
+  if (cap_ != 1) HN_LAUNCH0(launch_summary(E_, h, use_h, 0, s));
   return HN_OK;
 }
 
 hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h, int use_h) {
   cudaStream_t s = s0;
   const int start = counting_;
-  if (prm_.solver == SOLVER_PCG && fuse_control()) {
-    // the same steps with each control step in the last block of the kernel before it, and the
-    // summary in the last one's
-    HN_TRY(issue_vcycle(s, PH_PRECOND));
-    HN_LAUNCH(KC_PCG_DOT, -1, launch_pcg_dot(E_, fine_, fineGrid_, s, 1));
-    HN_LAUNCH(KC_PCG_P, -1, launch_pcg_p(E_, fine_, fineGrid_, s, 1));
-    HN_LAUNCH(KC_PCG_Q, -1, launch_pcg_q(E_, fine_, fineGrid_, s, 1));
-    if (condCapture_) {
-      const CondDev& cd = E_.prm.cond;
-      E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle - cd.n_outer - cd.n_update;
-    }
-    HN_LAUNCH(KC_PCG_X, -1, launch_pcg_x(E_, fine_, fineGrid_, s, 1, h, use_h));
-    return HN_OK;
-  } else if (prm_.solver == SOLVER_PCG) {
+  // the kernels outside the IF node, those still to be launched included
+  auto count_base = [&](int to_come) {
+    if (!condCapture_) return;
+    const CondDev& cd = E_.prm.cond;
+    E_.prm.cond.n_base = (unsigned)(counting_ + to_come - start) - cd.n_cycle - cd.n_outer - cd.n_update;
+  };
+  // an engine of one problem ends the iteration in its last vector step
+  const int end = cap_ == 1 ? 1 : 0;
+  if (prm_.solver == SOLVER_PCG) {
     // z = M r (one cycle from zero), rho' = (r, z), beta, p = z + beta p, then the CG step
     // q = A p, alpha, x += alpha p, r -= alpha q, and its check
     HN_TRY(issue_vcycle(s, PH_PRECOND));
-    HN_LAUNCH(KC_PCG_DOT, -1, launch_pcg_dot(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_PCG_BETA, s));
-    HN_LAUNCH(KC_PCG_P, -1, launch_pcg_p(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_POST, s));
-    HN_LAUNCH(KC_PCG_Q, -1, launch_pcg_q(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_PCG_ALPHA, s));
-    HN_LAUNCH(KC_PCG_X, -1, launch_pcg_x(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_OUTER, s));
+    HN_LAUNCH(KC_PCG_DOT, -1, launch_fine(E_, FINE_PCG_DOT, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_PCG_P, -1, launch_fine(E_, FINE_PCG_P, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_PCG_Q, -1, launch_fine(E_, FINE_PCG_Q, soloTiles_, 0, h, use_h, s));
+    count_base(end ? 1 : 2);
+    HN_LAUNCH(KC_PCG_X, -1, launch_fine(E_, FINE_PCG_X, soloTiles_, end, h, use_h, s));
   } else if (prm_.prec == P64) {
     HN_TRY(issue_vcycle(s, PH_CYCLE));
-  } else if (fuse_control()) {
-    // an engine of one problem: the outer control step inside the outer defect, the control step
-    // after the update and the iteration's summary inside the update (their last blocks)
-    HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_outer_defect(E_, fine_, fineGrid_, s, 1));
-    HN_TRY(issue_vcycle(s, PH_INNER));
-    if (condCapture_) {                            // the launches outside IF nodes, the update's too
-      const CondDev& cd = E_.prm.cond;
-      E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle - cd.n_outer - cd.n_update;
-    }
-    HN_LAUNCH(KC_UPDATE, -1, launch_update(E_, fine_, fineGrid_, s, 1, h, use_h));
+    count_base(1);
+    HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
     return HN_OK;
   } else {
-    if (cond_on(1)) HN_TRY(open_if(s, 1));
-    int c0 = counting_;
-    HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_outer_defect(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_OUTER, s));
-    if (cond_on(1)) {
-      E_.prm.cond.n_outer = (unsigned)(counting_ - c0);
-      HN_TRY(close_if(s, s0));
-    }
+    HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_fine(E_, FINE_OUTER, soloTiles_, 0, h, use_h, s));
     HN_TRY(issue_vcycle(s, PH_INNER));
-    if (cond_on(2)) HN_TRY(open_if(s, 2));
-    c0 = counting_;
-    HN_LAUNCH(KC_UPDATE, -1, launch_update(E_, fine_, fineGrid_, s));
-    HN_LAUNCH(KC_CONTROL, -1, launch_control(E_, CTRL_POST, s));
-    if (cond_on(2)) {
-      E_.prm.cond.n_update = (unsigned)(counting_ - c0);
-      HN_TRY(close_if(s, s0));
-    }
+    count_base(end ? 1 : 2);
+    HN_LAUNCH(KC_UPDATE, -1, launch_fine(E_, FINE_UPDATE, soloTiles_, end, h, use_h, s));
   }
-  if (condCapture_) {
-    const CondDev& cd = E_.prm.cond;
-    E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle - cd.n_outer - cd.n_update;
-  }
-  HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
+  if (!end) HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
   return HN_OK;
-}
-
-// The defect correction and CG of an engine of one problem fold their control steps and the
-// iteration summary into the kernels before them when the fine norm is one group of partials (one
-// block sums it) and no step has an IF node of its own.
-bool Engine::fuse_control() const {
-  const bool dc = prm_.solver != SOLVER_PCG && prm_.prec != P64;
-  return cap_ == 1 && (dc || prm_.solver == SOLVER_PCG) && !cond_on(1) && !cond_on(2) &&
-         pitch_of(Lmax_) / kTile <= kSumGroup;
 }
 
 hn_status Engine::capture_graphs() {
@@ -1426,7 +1349,7 @@ hn_status Engine::read_error(int* err) {
 }
 
 hn_status Engine::apply_check_norm(cudaStream_t s) {
-  HN_CUDA(launch_check(E_, fine_, PH_CHECK, 0, fineGrid_, s));
+  HN_CUDA(launch_check(E_, lists_[Lmax_], Lmax_, PH_CHECK, 0, grid_[Lmax_], s));
   HN_CUDA(launch_control(E_, CTRL_CHECK0, s));
   return HN_OK;
 }

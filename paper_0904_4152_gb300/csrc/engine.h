@@ -127,10 +127,8 @@ namespace hn {
 struct WorkListOut {
   int2* items[kMaxLevel + 1];
   int4* chunks[kMaxLevel + 1];
-  int2* fine;
   int n[kMaxLevel + 1];              // members having level l
   int nt[kMaxLevel + 1];             // tiles of level l
-  int nfine;                         // members
 };
 }  // namespace hn
 
@@ -258,17 +256,16 @@ class Engine {
   ProblemDev* dP_ = nullptr;
   ProbState* dS_ = nullptr;
   int* dFineOff_ = nullptr;
-  int* dCounts_ = nullptr;          // [kMaxLevel + 2]: per level, then the fine list
+  int* dCounts_ = nullptr;          // [kMaxLevel + 1]: items per level
   int2* dItems_[kMaxLevel + 1] = {};
   int4* dChunks_[kMaxLevel + 1] = {};
   int* dChunkCounts_ = nullptr;
   long long chunkCap_[kMaxLevel + 1] = {};
   int* dErr_ = nullptr;
-  int2* dFine_ = nullptr;
   long long itemCap_[kMaxLevel + 1] = {};
   long long fineCap_ = 0;
   TileList lists_[kMaxLevel + 1] = {};
-  TileList fine_{};
+  int soloTiles_ = 0;               // an engine of one problem: the tiles of its finest level
   int grid_[kMaxLevel + 1] = {};
   TileList* dLists_ = nullptr;      // device copy of lists_ (read by the persistent kernels)
   TileList* hLists_ = nullptr;      // its pinned staging copy
@@ -279,20 +276,17 @@ class Engine {
   bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
   bool small_tail() const;          // the tail runs in one block's shared memory (k_small)
   SmallSolo small_{};               // its descriptors, for an engine of one problem
-  bool fuse_control() const;        // the DC control steps fold into the outer defect and update
   // level l may be a member's own finest level (the server's engines: any level)
   bool is_top(int l) const { return topMaskAll_ || ((topMask_ >> l) & 1u); }
-  int fineGrid_ = 1;
   int maxGrid_ = 1;
   std::vector<hn_mg*> members_;
-  std::vector<int> hCounts_;
   // set_members' plan (device) and its pinned staging area: counts, fine offsets, plan, problems
   int* dPlan_ = nullptr;
   void* hStage_ = nullptr;
   cudaEvent_t upEv_ = nullptr;       // the last upload from the staging area
-  size_t plan_ints() const { return (size_t)(kMaxLevel + 2) * cap_ + cap_ + 1; }
+  size_t plan_ints() const { return (size_t)(kMaxLevel + 1) * cap_; }
   size_t stage_probs_off() const {
-    return (((size_t)(kMaxLevel + 2) + (kMaxLevel + 1) + cap_ + plan_ints()) * sizeof(int) + 255) & ~size_t(255);
+    return ((2 * (size_t)(kMaxLevel + 1) + cap_ + plan_ints()) * sizeof(int) + 255) & ~size_t(255);
   }
   size_t stage_bytes() const { return stage_probs_off() + sizeof(ProblemDev) * cap_; }
   cudaGraphExec_t gSolve_ = nullptr, gInit_ = nullptr, gIter_ = nullptr;

@@ -182,13 +182,16 @@ cudaError_t launch_band_to_f32(int L, const BandPtrs64c& src, const BandPtrs32& 
 cudaError_t launch_band_to_f16(int L, const BandPtrs64c& src, unsigned long long* absmax9,
                                const BandPtrs16& dst, float* scales_dev, cudaStream_t s);
 
+// counters of a problem's norm sums: [0] the control launch's blocks, [1] the problem's parts, then per group of
+// kSumGroup tiles its parts, then 32 chains per group
+__host__ __device__ inline int ticket_words(int ctl_groups) { return 2 + 33 * ctl_groups; }
+
 // solver kernels (k_cycle.cu).  All take the engine's device arrays.
 struct EngineDev {
   const ProblemDev* P;   // problems
   ProbState* S;          // states
   const int* fine_off;   // first partial slot of each problem (fine-level tile list order)
   double* partial;       // one slot per fine-level tile
-  double* partial2;      // second set (||b|| at start)
   int nprob;
   int pad;
   Params prm;
@@ -203,8 +206,7 @@ struct EngineDev {
   int ctl_groups;              // blocks per problem of the control kernel (groups of the largest
                                // problem's norm partial sum)
   double* gsum;                // [nprob * ctl_groups] group sums of the control kernel
-  unsigned* gticket;           // [nprob * (ctl_groups + 1)] blocks of a problem's group (groups of the problem)
-                               // that finished their part of a norm sum
+  unsigned* gticket;           // [nprob * ticket_words(ctl_groups)] counts of finished parts of a problem's norm sum
   unsigned* ticket;            // blocks of a first smoothing step with a fused check that finished
   unsigned long long* gbar;    // [3] grid barriers of the persistent kernels: arrivals of the
                                // down kernel, of the up kernel, barrier actions completed
@@ -220,7 +222,7 @@ cudaError_t launch_defect(const EngineDev& E, TileList tl, int level, int want, 
                           int grid, cudaStream_t s);
 cudaError_t launch_spmv(const EngineDev& E, TileList tl, int level, int want, int in_sel, int grid,
                         cudaStream_t s);
-cudaError_t launch_check(const EngineDev& E, TileList fine, int want, int x_sel, int grid,
+cudaError_t launch_check(const EngineDev& E, TileList tl, int level, int want, int x_sel, int grid,
                          cudaStream_t s);
 // first two smoothing steps: fused from a zero iterate (PRE12 alone), else step 1 (PRE12) and
 // step 2 (PRE2B); pre_fuses(prec) tells whether the zero-iterate fusion exists for a precision
@@ -286,28 +288,17 @@ cudaError_t launch_prolong(const EngineDev& E, TileList tl, int level, int want,
 cudaError_t launch_prolong_jacobi(const EngineDev& E, TileList tl, int level, int want, int x_sel,
                                   int grid, cudaStream_t s);
 cudaError_t launch_coarse(const EngineDev& E, TileList tl, int want, int grid, cudaStream_t s);
-// fuse: an engine of one problem whose fine norm is one group of partials takes the outer control
-// step in the last block of the outer defect, and the control step after the update plus the
-// end-of-iteration summary (WHILE handle h if use_handle) in the last block of the update
-cudaError_t launch_outer_defect(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0);
-// PCG vector steps on each problem's finest level (FP64): q = A p with partials (p, q); x += alpha
-// p, r -= alpha q with partials ||r||^2 and the scaled residual as the cycle's right-hand side;
-// partials (r, z); p = z / s + beta p
-cudaError_t launch_pcg_q(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0);
-// fuse (one problem): the kernels' last blocks take the control steps (pcg_x also the summary)
-cudaError_t launch_pcg_x(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0,
-                         cudaGraphConditionalHandle h = 0, int use_handle = 0);
-cudaError_t launch_pcg_dot(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0);
-cudaError_t launch_pcg_p(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0);
-cudaError_t launch_update(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse = 0,
-                          cudaGraphConditionalHandle h = 0, int use_handle = 0);
-cudaError_t launch_norm_b(const EngineDev& E, TileList fine, int grid, cudaStream_t s);
+// The FP64 vector steps on each problem's finest level (k_fine.cu), with the problems' control steps in the
+// last block.  solo_tiles: the tiles of an engine of one problem, else 0.  summary (an engine of one
+// problem): 1: the iteration ends here (WHILE handle h if use_handle), 2: the start of a solve ends here.
+enum FineKind { FINE_NORM_B = 0, FINE_OUTER, FINE_UPDATE, FINE_PCG_Q, FINE_PCG_X, FINE_PCG_DOT, FINE_PCG_P };
+cudaError_t launch_fine(const EngineDev& E, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+                        int use_handle, cudaStream_t s);
 // kind: ControlKind; level: for CTRL_PRE, the finest level whose problems are checked
 cudaError_t launch_control(const EngineDev& E, int kind, cudaStream_t s, int level = -1);
 // end_of_iteration: clear the zero-iterate flag of running cycles (iteration graph only)
 cudaError_t launch_summary(const EngineDev& E, cudaGraphConditionalHandle h, int use_handle,
                            int end_of_iteration, cudaStream_t s);
-cudaError_t launch_boundary_check(const EngineDev& E, cudaStream_t s);
 
 enum ControlKind {
   CTRL_INIT = 0, CTRL_CHECK = 1, CTRL_OUTER = 2, CTRL_POST = 4, CTRL_CHECK0 = 5,

@@ -532,24 +532,6 @@ __device__ void coarse_cg(const double* ab, int n, int m, double* x, double* r, 
 // a few bytes at 5 blocks and is still faster than at 4: 89.8 vs 96.3 us at L = 12), except the
 // FP16 defect, faster at 4 with its band loads hoisted; the fused pre-smoothing (4 blocks) and
 // check modes run once per cycle and get more registers per thread.
-__device__ void control_apply(const EngineDev& E, ProbState& st, int kind, double sum);
-__device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, int use_handle,
-                              int end_of_iteration, double* sh);
-
-// The last block of a launch of an engine of one problem takes control step `kind` in place of a
-// control launch: with the launch's FP64 partials summed in the fixed order (sum_partials), if
-// the problem was in the phase the step serves (mine: block-uniform, read at the launch's start)
-__device__ void solo_fused_control(const EngineDev& E, int kind, bool mine, bool sum_partials) {
-  if (!solo_last_block(E)) return;
-  __shared__ double sh[32];
-  double sum = 0.0;
-  if (mine && sum_partials) sum = problem_norm_sum(E.partial, fine_tiles(E.P[0].L), sh);
-  if (threadIdx.x == 0) {
-    if (mine) control_apply(E, E.S[0], kind, sum);
-    *E.ticket = 0u;
-  }
-}
-
 template <class Pol, int MODE> constexpr int band_min_blocks() {
   if (MODE == M_CHECK) return Pol::prec == P64 ? 2 : 3;
   if (MODE == M_PRE12) return Pol::prec == P64 ? 2 : 4;
@@ -2217,298 +2199,6 @@ __global__ void __launch_bounds__(mid_threads<Pol>(), 1) k_mid_up(EngineDev E, c
   }
 }
 
-// FP64 outer defect of the defect correction: d = b - A x (FP64 bands, FP64 x), written to the
-// inner top-level right-hand side as V(d * s); partial[g] = sum d^2.  x = 0 gives d = b.  PCG:
-// the initial residual (before the first cycle), also kept in FP64 (r64).
-template <class V>
-// fuse (an engine of one problem whose norm is one group of partials): the last block to finish
-// sums the partials in the fixed order and takes the outer control step (in place of a control
-// launch)
-__global__ void __launch_bounds__(256) k_outer_defect(EngineDev E, TileList tl, int fuse) {
-  pdl_start();
-  if (solo_idle(E, PH_OUTER)) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const int p = it.x;
-    const ProbState& st = E.S[p];
-    if (st.phase != PH_OUTER) continue;
-    const bool pcg = E.prm.solver == SOLVER_PCG;
-    if (pcg && st.cycles > 0) continue;
-    const ProblemDev& P = E.P[p];
-    const LevelDev& top = P.lev[P.L];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    double b[4], r[4];
-    ld4<LD_EF>(P.b64 + i0, b);
-    if (st.x_zero) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) r[j] = b[j];
-    } else {
-      double w[3][8], dg[4];
-#pragma unroll
-      for (int dy = -1; dy <= 1; ++dy) load_row<double, LD_NC>(P.x64, i0 + dy * (1LL << P.L), lane, w[dy + 1]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) r[j] = b[j];       // r = b - A x as one chain from b
-      stencil_windows<F64, LD_EF, true>(reinterpret_cast<const void* const*>(P.band64), nullptr, w, i0, r, dg);
-    }
-    const double s = st.s;
-    V out[4];
-    double q = 0.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      out[j] = V(r[j] * s);
-      q += r[j] * r[j];
-    }
-    st4(static_cast<V*>(top.rhs) + i0, out);
-    if (pcg) st4(P.r64 + i0, r);
-    q = warp_sum(q);
-    if (lane == 0) E.partial[g] = q;
-  }
-  if (fuse && solo_last_block(E)) {               // (every block was in the outer phase)
-    __shared__ double sh[32];
-    const double sum = problem_norm_sum(E.partial, fine_tiles(E.P[0].L), sh);
-    if (threadIdx.x == 0) {
-      control_apply(E, E.S[0], CTRL_OUTER, sum);
-      *E.ticket = 0u;
-    }
-  }
-}
-
-// ----------------------------------------------------------------- PCG vector steps (FP64)
-// Conjugate gradients on each problem's finest level with the V cycle as preconditioner (a
-// solver plugged into another, Sec. 4.1): every step below is one pass over the fine work list.
-
-// q = A p (FP64 bands, p with zero halos), partial[g] = sum p q, for problems in their CG step
-__global__ void __launch_bounds__(256) k_pcg_q(EngineDev E, TileList tl, int fuse) {
-  pdl_start();
-  if (solo_idle(E, PH_OUTER)) return;
-  const bool mine = E.S[0].cycles > 0;            // (fuse: one problem, in the outer phase)
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const ProbState& st = E.S[it.x];
-    if (st.phase != PH_OUTER || st.cycles == 0) continue;
-    const ProblemDev& P = E.P[it.x];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    double w[3][8], acc[4], dg[4];
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy) load_row<double, LD_NC>(P.p64, i0 + dy * (1LL << P.L), lane, w[dy + 1]);
-    stencil_windows<F64, LD_NC>(reinterpret_cast<const void* const*>(P.band64), nullptr, w, i0, acc, dg);
-    st4(P.q64 + i0, acc);
-    double t = 0.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) t = fma(w[1][j + 2], acc[j], t);
-    t = warp_sum(t);
-    if (lane == 0) E.partial[g] = t;
-  }
-  if (fuse) solo_fused_control(E, CTRL_PCG_ALPHA, mine, true);
-}
-
-// x += alpha p, r -= alpha q; partial[g] = sum r^2; the cycle's right-hand side V(s r)
-// fuse (one problem): the last block takes the check after the step and the iteration's summary;
-// every block then runs to the end whatever the phase
-template <class V>
-__global__ void __launch_bounds__(256) k_pcg_x(EngineDev E, TileList tl, int fuse,
-                                               cudaGraphConditionalHandle h, int use_handle) {
-  pdl_start();
-  const bool outer = E.nprob != 1 || E.S[0].phase == PH_OUTER;
-  if (!fuse && !outer) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const ProbState& st = E.S[it.x];
-    if (st.phase != PH_OUTER || st.cycles == 0) continue;
-    const ProblemDev& P = E.P[it.x];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    double x[4], r[4], pv[4], qv[4];
-    ld4c(P.x64 + i0, x);
-    ld4c(P.r64 + i0, r);
-    ld4<LD_NC>(P.p64 + i0, pv);
-    ld4<LD_NC>(P.q64 + i0, qv);
-    const double alpha = st.alpha, sc = st.s;
-    V out[4];
-    double t = 0.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      x[j] = fma(alpha, pv[j], x[j]);
-      r[j] = fma(-alpha, qv[j], r[j]);
-      t = fma(r[j], r[j], t);
-      out[j] = V(r[j] * sc);
-    }
-    st4(P.x64 + i0, x);
-    st4(P.r64 + i0, r);
-    st4(static_cast<V*>(P.lev[P.L].rhs) + i0, out);
-    t = warp_sum(t);
-    if (lane == 0) E.partial[g] = t;
-  }
-  if (fuse && solo_last_block(E)) {
-    __shared__ double sh[32];
-    double sum = 0.0;
-    if (outer) sum = problem_norm_sum(E.partial, fine_tiles(E.P[0].L), sh);
-    if (threadIdx.x == 0) {
-      if (outer) control_apply(E, E.S[0], CTRL_OUTER, sum);
-      *E.ticket = 0u;
-    }
-    __syncthreads();
-    summary_apply(E, h, use_handle, 1, sh);
-  }
-}
-
-// partial[g] = sum r c, c = the cycle's result (top-level buffer 0, z = c / s)
-template <class V>
-__global__ void __launch_bounds__(256) k_pcg_dot(EngineDev E, TileList tl, int fuse) {
-  pdl_start();
-  if (solo_idle(E, PH_PRECOND)) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    if (E.S[it.x].phase != PH_PRECOND) continue;
-    const ProblemDev& P = E.P[it.x];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    double r[4];
-    V c[4];
-    ld4<LD_NC>(P.r64 + i0, r);
-    ld4<LD_NC>(static_cast<const V*>(P.lev[P.L].x[0]) + i0, c);
-    double t = 0.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) t = fma(r[j], double(c[j]), t);
-    t = warp_sum(t);
-    if (lane == 0) E.partial[g] = t;
-  }
-  if (fuse) solo_fused_control(E, CTRL_PCG_BETA, true, true);
-}
-
-// p = c / s + beta p (the new search direction), for problems in PH_UPDATE
-template <class V>
-__global__ void __launch_bounds__(256) k_pcg_p(EngineDev E, TileList tl, int fuse) {
-  pdl_start();
-  if (solo_idle(E, PH_UPDATE)) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const ProbState& st = E.S[it.x];
-    if (st.phase != PH_UPDATE) continue;
-    const ProblemDev& P = E.P[it.x];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    V c[4];
-    double pv[4];
-    ld4<LD_NC>(static_cast<const V*>(P.lev[P.L].x[0]) + i0, c);
-    ld4c(P.p64 + i0, pv);
-    const double beta = st.beta, inv_s = st.inv_s;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) pv[j] = fma(beta, pv[j], double(c[j]) * inv_s);
-    st4(P.p64 + i0, pv);
-  }
-  if (fuse) solo_fused_control(E, CTRL_POST, true, false);
-}
-
-// x64 += c / s (c = inner top-level iterate, buffer 0), for problems in PH_UPDATE
-// fuse (an engine of one problem, defect correction): the last block to finish takes the control
-// step after the update and the end-of-iteration summary (in place of two launches); then every
-// block runs to the end whatever the phase
-__global__ void __launch_bounds__(256) k_update(EngineDev E, TileList tl, int fuse,
-                                                cudaGraphConditionalHandle h, int use_handle) {
-  pdl_start();
-  const bool updating = E.nprob != 1 || E.S[0].phase == PH_UPDATE;
-  if (!fuse && !updating) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const int p = it.x;
-    const ProbState& st = E.S[p];
-    if (st.phase != PH_UPDATE) continue;
-    const ProblemDev& P = E.P[p];
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    float c[4];
-    ld4<LD_NC>(static_cast<const float*>(P.lev[P.L].x[0]) + i0, c);
-    double x[4];
-    ld4c(P.x64 + i0, x);
-    const double inv_s = st.inv_s;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = fma(double(c[j]), inv_s, x[j]);
-    st4(P.x64 + i0, x);
-  }
-  if (fuse && solo_last_block(E)) {
-    __shared__ double sh[32];
-    if (threadIdx.x == 0) {
-      if (updating) control_apply(E, E.S[0], CTRL_POST, 0.0);
-      *E.ticket = 0u;
-    }
-    __syncthreads();
-    summary_apply(E, h, use_handle, 1, sh);
-  }
-}
-
-// ||b||^2 partials for problems starting a solve
-__global__ void __launch_bounds__(256) k_norm_b(EngineDev E, TileList tl) {
-  pdl_start();
-  if (solo_idle(E, PH_INIT)) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int count = *tl.count;
-  for (int g = gw; g < count; g += nw) {
-    const int2 it = tl.items[g];
-    if (!dbg_item(E, it.x, it.y, -1, __LINE__)) continue;   // a tile of the finest level
-    const int p = it.x;
-    if (E.S[p].phase != PH_INIT) continue;
-    const long long i0 = (long long)it.y * kTile + lane * kLaneNodes;
-    double b[4];
-    ld4<LD_NC>(E.P[p].b64 + i0, b);
-    double q = b[0] * b[0] + b[1] * b[1] + b[2] * b[2] + b[3] * b[3];
-    q = warp_sum(q);
-    if (lane == 0) E.partial2[g] = q;
-  }
-}
-
-// Reject right-hand sides with non-zero entries on Dirichlet nodes (one block per problem).
-__global__ void __launch_bounds__(256) k_boundary_check(EngineDev E) {
-  pdl_start();
-  const int p = blockIdx.x;
-  if (p >= E.nprob) return;
-  ProbState& st = E.S[p];
-  if (st.phase != PH_INIT) return;
-  const ProblemDev& P = E.P[p];
-  const long long n = n_of_dev(P.L);
-  const int bc = P.lev[P.L].bc;
-  int bad = 0;
-  for (long long t = threadIdx.x; t < 4 * (n - 1); t += blockDim.x) {
-    const long long side = t / (n - 1), k = t - side * (n - 1);
-    long long ix, iy;
-    if (side == 0) { ix = k; iy = 0; }                     // bottom row, ix = 0..n-2
-    else if (side == 1) { ix = n - 1; iy = k; }            // right column
-    else if (side == 2) { ix = n - 1 - k; iy = n - 1; }    // top row
-    else { ix = 0; iy = n - 1 - k; }                       // left column
-    if (is_dirichlet(ix, iy, n, bc) && P.b64[iy * n + ix] != 0.0) bad = 1;
-  }
-  bad = __syncthreads_or(bad);
-  if (bad && threadIdx.x == 0) { st.status = HN_ERR_ARG; st.phase = PH_DONE; }
-}
-
 // Per-problem control of the solver state machine: reduce the problem's norm partials in a fixed
 // order (bit-reproducible, independent of the batch), then update its state.
 // The norm of problem p from its tile partials, by the ctl_groups blocks of p in this launch
@@ -2529,7 +2219,7 @@ __device__ bool control_sum(const EngineDev& E, int p, int j, const double* part
   if (threadIdx.x == 0) {
     E.gsum[(long long)p * E.ctl_groups + j] = g;
     __threadfence();
-    last = atomicAdd(E.gticket + (long long)p * (E.ctl_groups + 1), 1u) == (unsigned)(ng - 1);
+    last = atomicAdd(E.gticket + (long long)p * ticket_words(E.ctl_groups), 1u) == (unsigned)(ng - 1);
   }
   __syncthreads();
   if (!last) return false;
@@ -2538,106 +2228,9 @@ __device__ bool control_sum(const EngineDev& E, int p, int j, const double* part
     double t = 0.0;
     for (int q = 0; q < ng; ++q) t += __ldcg(E.gsum + (long long)p * E.ctl_groups + q);
     *sum = t;
-    E.gticket[(long long)p * (E.ctl_groups + 1)] = 0u;   // ready for the next launch
+    E.gticket[(long long)p * ticket_words(E.ctl_groups)] = 0u;   // ready for the next launch
   }
   return true;
-}
-
-// The state transition of control step `kind` for problem state st, given the summed partials
-// (thread 0 of one block; the control kernel, or the last block of a kernel that folds the step in)
-__device__ void control_apply(const EngineDev& E, ProbState& st, int kind, double sum) {
-  const int ph = st.phase;
-  const Params& prm = E.prm;
-  const double nrm = sqrt(sum);
-  switch (kind) {
-    case CTRL_INIT:
-      if (st.status == HN_ERR_ARG) { st.phase = PH_DONE; break; }
-      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; break; }
-      if (nrm == 0.0) { st.bnorm = 0.0; st.relres = 0.0; st.status = HN_OK; st.phase = PH_DONE; break; }
-      st.bnorm = nrm;
-      st.s = 1.0 / nrm;
-      st.inv_s = 1.0 / st.s;
-      st.relres = 1.0;
-      if (prm.prec == P64 && prm.solver != SOLVER_PCG) {
-        // a zero initial guess starts its first cycle unchecked (relres 1); a given guess is
-        // checked by the first smoothing step of its first cycle
-        st.phase = PH_CYCLE;
-        st.cycles = st.x_zero ? 1 : 0;
-      } else {
-        st.phase = PH_OUTER;
-      }
-      break;
-    case CTRL_CHECK0:
-    case CTRL_CHECK:
-      if (ph == PH_CYCLE) { st.cycles += 1; st.zero_top = 0; st.x_zero = 0; }
-      st.dnorm = nrm;
-      st.relres = nrm / st.bnorm;
-      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
-      else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
-      else if (st.cycles >= prm.max_cycles) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
-      else st.phase = PH_CYCLE;
-      break;
-    case CTRL_OUTER:
-      if (prm.solver == SOLVER_PCG) {
-        // after the initial residual or a CG step: check, then precondition the new residual
-        if (st.cycles > 0) st.outer_iters += 1;
-        st.dnorm = nrm;
-        st.relres = nrm / st.bnorm;
-        if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
-        else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
-        else if (st.outer_iters >= prm.max_outer || st.cycles >= prm.max_cycles) {
-          st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE;
-        } else {
-          st.phase = PH_PRECOND; st.zero_top = 1; st.cycles += 1;
-          if (prm.prec != P64) st.inner_cycles += 1;
-        }
-        break;
-      }
-      st.dnorm = nrm;
-      st.relres = nrm / st.bnorm;
-      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
-      else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
-      else if (st.outer_iters >= prm.max_outer || st.inner_cycles >= prm.max_cycles) {
-        st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE;
-      } else {
-        // the first inner cycle starts from zero: it runs unchecked and is counted here
-        st.phase = PH_INNER; st.zero_top = 1; st.inner_ref = st.s * nrm;
-        st.inner_k = 1; st.inner_cycles += 1; st.cycles += 1;
-      }
-      break;
-    case CTRL_PCG_ALPHA:
-      // sum = (p, q); a breakdown (not positive: the preconditioned operator is not definite in
-      // this arithmetic) stops the solve
-      if (!isfinite(sum) || !(sum > 0.0)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
-      else st.alpha = st.rho / sum;
-      break;
-    case CTRL_PCG_BETA: {
-      // sum = (r, c) with z = c / s: rho' = (r, z); the first direction is z itself
-      const double rho = sum / st.s;
-      if (!isfinite(rho) || !(rho > 0.0)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; break; }
-      st.beta = st.cycles > 1 ? rho / st.rho : 0.0;
-      st.rho = rho;
-      st.phase = PH_UPDATE;
-      break;
-    }
-    case CTRL_POST: {
-      if (prm.solver == SOLVER_PCG) {
-        // the next cycle's right-hand side is scaled by 1 / ||r|| of this step
-        if (st.dnorm > 0.0 && isfinite(st.dnorm)) { st.s = 1.0 / st.dnorm; st.inv_s = 1.0 / st.s; }
-        st.phase = PH_OUTER;
-        break;
-      }
-      st.outer_iters += 1;
-      st.x_zero = 0;
-      // scale for the next defect: the inner solve reduced the defect by about inner_res/inner_ref
-      const double red = st.inner_ref > 0.0 ? st.inner_res / st.inner_ref : 1.0;
-      const double pred = st.dnorm * fmax(red, 1e-7);
-      if (pred > 0.0 && isfinite(pred)) { st.s = 1.0 / pred; st.inv_s = 1.0 / st.s; }
-      st.phase = PH_OUTER;
-      break;
-    }
-    default: break;
-  }
 }
 
 __global__ void __launch_bounds__(256) k_control(EngineDev E, int kind, int level) {
@@ -2659,62 +2252,13 @@ __global__ void __launch_bounds__(256) k_control(EngineDev E, int kind, int leve
       cond_set(E.prm.cond, 0, 1u);
     return;
   }
-  const bool mine = (kind == CTRL_INIT && ph == PH_INIT) ||
-                    (kind == CTRL_CHECK0 && ph == PH_CHECK) ||
-                    (kind == CTRL_CHECK && ph == PH_CYCLE) ||
-                    (kind == CTRL_OUTER && ph == PH_OUTER) ||
-                    (kind == CTRL_POST && ph == PH_UPDATE) ||
-                    (kind == CTRL_PCG_ALPHA && ph == PH_OUTER && st.cycles > 0) ||
-                    (kind == CTRL_PCG_BETA && ph == PH_PRECOND);
-  if (!mine) return;
+  // (the steps on the finest level's FP64 norms are taken by the kernels that form them, k_fine.cu)
+  if (!(kind == CTRL_CHECK0 && ph == PH_CHECK) && !(kind == CTRL_CHECK && ph == PH_CYCLE)) return;
   double sum = 0.0;
-  if (kind != CTRL_POST) {
-    const double* part = kind == CTRL_INIT ? E.partial2 : E.partial;
-    // the checks of the cycle's own precision: double-float partials in FP32 / FP16 cycles
-    const bool df = (kind == CTRL_CHECK || kind == CTRL_CHECK0) && E.prm.prec != P64;
-    if (!control_sum(E, p, j, part + E.fine_off[p], fine_tiles(E.P[p].L), sh, &sum, df)) return;
-  } else if (j != 0) {
-    return;
-  }
+  // the checks of the cycle's own precision: double-float partials in FP32 / FP16 cycles
+  if (!control_sum(E, p, j, E.partial + E.fine_off[p], fine_tiles(E.P[p].L), sh, &sum, E.prm.prec != P64)) return;
   if (threadIdx.x != 0) return;
   control_apply(E, st, kind, sum);
-}
-
-// Count problems still running; publish to the host word and, inside a device-side loop, to the
-// graph's while-condition.  Past the iteration limit every running problem is stopped as not
-// converged, so a device-side loop always ends.
-__device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, int use_handle,
-                              int end_of_iteration, double* sh) {
-  __shared__ unsigned over;
-  if (threadIdx.x == 0) {
-    const unsigned it = E.iter ? (*E.iter += 1) : 0u;
-    over = (E.iter && it > E.iter_limit) ? 1u : 0u;
-  }
-  __syncthreads();
-  double c = 0.0, o = 0.0;
-  for (int p = threadIdx.x; p < E.nprob; p += blockDim.x) {
-    ProbState& st = E.S[p];
-    if (st.phase != PH_DONE && over) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
-    // after an iteration the finest-level iterate of a running cycle is no longer zero
-    if (end_of_iteration && (st.phase == PH_INNER || st.phase == PH_CYCLE)) st.zero_top = 0;
-    c += st.phase != PH_DONE ? 1.0 : 0.0;
-    o += st.phase == PH_OUTER ? 1.0 : 0.0;
-  }
-  c = block_sum256(c, sh);
-  o = block_sum256(o, sh);
-  if (threadIdx.x == 0) {
-    const unsigned active = (unsigned)c;
-    if (E.active_host) *E.active_host = active;
-    if (use_handle) cudaGraphSetConditional(h, active > 0 ? 1u : 0u);
-    const CondDev& cd = E.prm.cond;
-    if (cd.mask) {
-      *cd.launches += cd.n_base + (cd.taken[0] ? cd.n_cycle : 0u) + (cd.taken[1] ? cd.n_outer : 0u) +
-                      (cd.taken[2] ? cd.n_update : 0u);
-      cond_set(cd, 0, 0u);
-      cond_set(cd, 2, 0u);
-      cond_set(cd, 1, o > 0.0 ? 1u : 0u);
-    }
-  }
 }
 
 __global__ void __launch_bounds__(256) k_summary(EngineDev E, cudaGraphConditionalHandle h,
@@ -3057,37 +2601,6 @@ cudaError_t launch_coarse(const EngineDev& E, TileList tl, int want, int grid, c
   return launch_k(k_coarse<float>, grid, 0, s, E.pdl, 0, E, tl, want);
 }
 
-cudaError_t launch_outer_defect(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse) {
-  if (E.prm.prec == P64) return launch_k(k_outer_defect<double>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-  return launch_k(k_outer_defect<float>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-}
-
-cudaError_t launch_pcg_q(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse) {
-  return launch_k(k_pcg_q, grid, 0, s, E.pdl, 0, E, fine, fuse);
-}
-cudaError_t launch_pcg_x(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse,
-                         cudaGraphConditionalHandle h, int use_handle) {
-  if (E.prm.prec == P64) return launch_k(k_pcg_x<double>, grid, 0, s, E.pdl, 0, E, fine, fuse, h, use_handle);
-  return launch_k(k_pcg_x<float>, grid, 0, s, E.pdl, 0, E, fine, fuse, h, use_handle);
-}
-cudaError_t launch_pcg_dot(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse) {
-  if (E.prm.prec == P64) return launch_k(k_pcg_dot<double>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-  return launch_k(k_pcg_dot<float>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-}
-cudaError_t launch_pcg_p(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse) {
-  if (E.prm.prec == P64) return launch_k(k_pcg_p<double>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-  return launch_k(k_pcg_p<float>, grid, 0, s, E.pdl, 0, E, fine, fuse);
-}
-
-cudaError_t launch_update(const EngineDev& E, TileList fine, int grid, cudaStream_t s, int fuse,
-                          cudaGraphConditionalHandle h, int use_handle) {
-  return launch_k(k_update, grid, 0, s, E.pdl, 0, E, fine, fuse, h, use_handle);
-}
-
-cudaError_t launch_norm_b(const EngineDev& E, TileList fine, int grid, cudaStream_t s) {
-  return launch_k(k_norm_b, grid, 0, s, E.pdl, 0, E, fine);
-}
-
 cudaError_t launch_control(const EngineDev& E, int kind, cudaStream_t s, int level) {
   return launch_k(k_control, E.nprob * E.ctl_groups, 0, s, E.pdl, 0, E, kind, level);
 }
@@ -3097,15 +2610,9 @@ cudaError_t launch_summary(const EngineDev& E, cudaGraphConditionalHandle h, int
   return launch_k(k_summary, 1, 0, s, E.pdl, 0, E, h, use_handle, end_of_iteration);
 }
 
-cudaError_t launch_boundary_check(const EngineDev& E, cudaStream_t s) {
-  return launch_k(k_boundary_check, E.nprob, 0, s, 0, 0, E);
-}
-
-// the fine-level defect norm of the V-cycle's own precision (convergence check)
-cudaError_t launch_check(const EngineDev& E, TileList fine_by_problem_top, int want, int x_sel,
-                         int grid, cudaStream_t s) {
-  // the fine work list enumerates every problem's top level; the level is taken per problem
-  return launch_band(M_CHECK, E, fine_by_problem_top, -1, want, x_sel, grid, s);
+// the defect norm of the finest level in the V-cycle's own precision (an engine of one problem)
+cudaError_t launch_check(const EngineDev& E, TileList tl, int level, int want, int x_sel, int grid, cudaStream_t s) {
+  return launch_band(M_CHECK, E, tl, level, want, x_sel, grid, s);
 }
 
 }  // namespace hn

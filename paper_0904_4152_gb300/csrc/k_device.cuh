@@ -577,6 +577,15 @@ __device__ __forceinline__ bool prolong_value(int ix, int iy, int nf, int nc, in
   return prolong_value_xy<V>(ix, iy, nf, bc, [&](int cy, int cx) { return ec(cy * nc + cx); }, add);
 }
 
+// node coordinates of flat index f in [0, n^2)
+__device__ __forceinline__ void node_xy(int f, int L, int& x, int& y) {
+  const int q = f >> L, c = f & ((1 << L) - 1), n = (1 << L) + 1;
+  y = q;
+  x = c - q;
+  if (x < 0) { x += n; --y; }
+  if (x < 0) { x += n; --y; }
+}
+
 // mbarrier and bulk-copy (TMA engine, 1D) helpers
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
@@ -669,6 +678,219 @@ __device__ void solo_fused_check(const EngineDev& E, int level, bool checked, in
     if (st.phase == want && (st.phase == PH_INNER || st.phase == PH_CYCLE)) cond_set(E.prm.cond, 0, 1u);
     *E.ticket = 0u;                                 // ready for the next launch
   }
+}
+
+// The state transition of control step `kind` for problem state st, given the summed partials
+// (thread 0 of one block; the control kernel, or the last block of a kernel that folds the step in)
+__device__ void control_apply(const EngineDev& E, ProbState& st, int kind, double sum) {
+  const int ph = st.phase;
+  const Params& prm = E.prm;
+  const double nrm = sqrt(sum);
+  switch (kind) {
+    case CTRL_INIT:
+      if (st.status == HN_ERR_ARG) { st.phase = PH_DONE; break; }
+      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; break; }
+      if (nrm == 0.0) { st.bnorm = 0.0; st.relres = 0.0; st.status = HN_OK; st.phase = PH_DONE; break; }
+      st.bnorm = nrm;
+      st.s = 1.0 / nrm;
+      st.inv_s = 1.0 / st.s;
+      st.relres = 1.0;
+      if (prm.prec == P64 && prm.solver != SOLVER_PCG) {
+        // a zero initial guess starts its first cycle unchecked (relres 1); a given guess is
+        // checked by the first smoothing step of its first cycle
+        st.phase = PH_CYCLE;
+        st.cycles = st.x_zero ? 1 : 0;
+      } else {
+        st.phase = PH_OUTER;
+      }
+      break;
+    case CTRL_CHECK0:
+    case CTRL_CHECK:
+      if (ph == PH_CYCLE) { st.cycles += 1; st.zero_top = 0; st.x_zero = 0; }
+      st.dnorm = nrm;
+      st.relres = nrm / st.bnorm;
+      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
+      else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
+      else if (st.cycles >= prm.max_cycles) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
+      else st.phase = PH_CYCLE;
+      break;
+    case CTRL_OUTER:
+      if (prm.solver == SOLVER_PCG) {
+        // after the initial residual or a CG step: check, then precondition the new residual
+        if (st.cycles > 0) st.outer_iters += 1;
+        st.dnorm = nrm;
+        st.relres = nrm / st.bnorm;
+        if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
+        else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
+        else if (st.outer_iters >= prm.max_outer || st.cycles >= prm.max_cycles) {
+          st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE;
+        } else {
+          st.phase = PH_PRECOND; st.zero_top = 1; st.cycles += 1;
+          if (prm.prec != P64) st.inner_cycles += 1;
+        }
+        break;
+      }
+      st.dnorm = nrm;
+      st.relres = nrm / st.bnorm;
+      if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
+      else if (st.relres <= prm.tol) { st.status = HN_OK; st.phase = PH_DONE; }
+      else if (st.outer_iters >= prm.max_outer || st.inner_cycles >= prm.max_cycles) {
+        st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE;
+      } else {
+        // the first inner cycle starts from zero: it runs unchecked and is counted here
+        st.phase = PH_INNER; st.zero_top = 1; st.inner_ref = st.s * nrm;
+        st.inner_k = 1; st.inner_cycles += 1; st.cycles += 1;
+      }
+      break;
+    case CTRL_PCG_ALPHA:
+      // sum = (p, q); a breakdown (not positive: the preconditioned operator is not definite in
+      // this arithmetic) stops the solve
+      if (!isfinite(sum) || !(sum > 0.0)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
+      else st.alpha = st.rho / sum;
+      break;
+    case CTRL_PCG_BETA: {
+      // sum = (r, c) with z = c / s: rho' = (r, z); the first direction is z itself
+      const double rho = sum / st.s;
+      if (!isfinite(rho) || !(rho > 0.0)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; break; }
+      st.beta = st.cycles > 1 ? rho / st.rho : 0.0;
+      st.rho = rho;
+      st.phase = PH_UPDATE;
+      break;
+    }
+    case CTRL_POST: {
+      if (prm.solver == SOLVER_PCG) {
+        // the next cycle's right-hand side is scaled by 1 / ||r|| of this step
+        if (st.dnorm > 0.0 && isfinite(st.dnorm)) { st.s = 1.0 / st.dnorm; st.inv_s = 1.0 / st.s; }
+        st.phase = PH_OUTER;
+        break;
+      }
+      st.outer_iters += 1;
+      st.x_zero = 0;
+      // scale for the next defect: the inner solve reduced the defect by about inner_res/inner_ref
+      const double red = st.inner_ref > 0.0 ? st.inner_res / st.inner_ref : 1.0;
+      const double pred = st.dnorm * fmax(red, 1e-7);
+      if (pred > 0.0 && isfinite(pred)) { st.s = 1.0 / pred; st.inv_s = 1.0 / st.s; }
+      st.phase = PH_OUTER;
+      break;
+    }
+    default: break;
+  }
+}
+
+// Count problems still running; publish to the host word and, inside a device-side loop, to the
+// graph's while-condition.  Past the iteration limit every running problem is stopped as not
+// converged, so a device-side loop always ends.
+__device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, int use_handle,
+                              int end_of_iteration, double* sh) {
+  __shared__ unsigned over;
+  if (threadIdx.x == 0) {
+    const unsigned it = E.iter ? (*E.iter += 1) : 0u;
+    over = (E.iter && it > E.iter_limit) ? 1u : 0u;
+  }
+  __syncthreads();
+  double c = 0.0, o = 0.0;
+  for (int p = threadIdx.x; p < E.nprob; p += blockDim.x) {
+    ProbState& st = E.S[p];
+    if (st.phase != PH_DONE && over) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
+    // after an iteration the finest-level iterate of a running cycle is no longer zero
+    if (end_of_iteration && (st.phase == PH_INNER || st.phase == PH_CYCLE)) st.zero_top = 0;
+    c += st.phase != PH_DONE ? 1.0 : 0.0;
+    o += st.phase == PH_OUTER ? 1.0 : 0.0;
+  }
+  c = block_sum256(c, sh);
+  o = block_sum256(o, sh);
+  if (threadIdx.x == 0) {
+    const unsigned active = (unsigned)c;
+    if (E.active_host) *E.active_host = active;
+    if (use_handle) cudaGraphSetConditional(h, active > 0 ? 1u : 0u);
+    const CondDev& cd = E.prm.cond;
+    if (cd.mask) {
+      *cd.launches += cd.n_base + (cd.taken[0] ? cd.n_cycle : 0u) + (cd.taken[1] ? cd.n_outer : 0u) +
+                      (cd.taken[2] ? cd.n_update : 0u);
+      cond_set(cd, 0, 0u);
+      cond_set(cd, 2, 0u);
+      cond_set(cd, 1, o > 0.0 ? 1u : 0u);
+    }
+  }
+}
+
+// The problems of an engine that a launch serves: those of at most kListMax slots from `base` that on(state,
+// finest level) chooses, in slot order, with the levels they are taken at (level, or 0: their own finest).
+// The whole block; returns the number of problems.  Every block of a launch has to find the same list, so
+// what `on` looks at must not change before every block has listed.
+constexpr int kListMax = 1024;
+struct Served {
+  unsigned short slot[kListMax];
+  unsigned char level[kListMax];
+  int start[kListMax + 1];
+  int count[32];
+};
+template <class F>
+__device__ int list_served(const EngineDev& E, Served& q, int base, int level, F&& chosen) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+  const int n = min(kListMax, E.nprob - base);
+  // slots of a warp: a contiguous share, read in one go (the loads of a round do not depend on each other)
+  const int share = (n + nw * 32 - 1) / (nw * 32);
+  const int lo = warp * share * 32;
+  unsigned take = 0;
+  for (int k = 0; k < share; ++k) {
+    const int p = lo + k * 32 + lane;
+    const bool on = p < n && chosen(E.S[base + p], E.P[base + p].L);
+    take |= on ? 1u << k : 0u;
+  }
+  int mine = 0;
+  for (int k = 0; k < share; ++k) mine += __popc(__ballot_sync(kFull, (take >> k) & 1u));
+  if (lane == 0) q.count[warp] = mine;
+  __syncthreads();
+  int at = 0, total = 0;
+  for (int w = 0; w < nw; ++w) {
+    if (w < warp) at += q.count[w];
+    total += q.count[w];
+  }
+  for (int k = 0; k < share; ++k) {
+    const bool on = (take >> k) & 1u;
+    const unsigned m = __ballot_sync(kFull, on);
+    if (on) {
+      const int i = at + __popc(m & ((1u << lane) - 1u)), p = base + lo + k * 32 + lane;
+      q.slot[i] = (unsigned short)p;
+      q.level[i] = (unsigned char)(level ? level : E.P[p].L);
+    }
+    at += __popc(m);
+  }
+  __syncthreads();
+  return total;
+}
+// running numbers of the problems' work items (items: of a level; 32-bit arithmetic only: a round of 32
+// problems is on every block's way to its first load); the whole block; returns their sum
+template <class F>
+__device__ int number_items(Served& q, int n, F&& items) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    int run = 0;
+    for (int b = 0; b < n; b += 32) {
+      const int c = b + lane < n ? items((int)q.level[b + lane]) : 0;
+      int s = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, s, o);
+        if (lane >= o) s += t;
+      }
+      if (b + lane < n) q.start[b + lane] = run + s - c;
+      run += __shfl_sync(kFull, s, 31);
+    }
+    if (lane == 0) q.start[n] = run;
+  }
+  __syncthreads();
+  return q.start[n];
+}
+// the problem of work item `it`
+__device__ __forceinline__ int served_of(const Served& q, int n, int it) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (q.start[mid] <= it) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 }  // namespace

@@ -36,7 +36,6 @@ namespace hn {
 
 namespace {
 
-constexpr int kListMax = 1024;           // problems a block lists at a time
 constexpr int kWarps = 2;                // independent warps of a block
 constexpr int kSlots = 4;                // rows of the ring: one in use, three on their way
 enum { DOWN_ZERO = 0, DOWN = 1, UP = 2 };
@@ -144,15 +143,6 @@ struct View {
   const float* scale;
   int L, n, pitch, bc;
 };
-
-// node coordinates of flat index f in [0, n^2)
-__device__ __forceinline__ void node_xy(int f, int L, int& x, int& y) {
-  const int q = f >> L, c = f & ((1 << L) - 1), n = (1 << L) + 1;
-  y = q;
-  x = c - q;
-  if (x < 0) { x += n; --y; }
-  if (x < 0) { x += n; --y; }
-}
 
 // The copies of a lane, row by row into the ring's slots: the sources of the row that comes next
 template <class Pol>
@@ -658,83 +648,6 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march(EngineDev E, TileList 
   }
 }
 
-// The problems of an engine that a launch serves: those in phase `want` (< 0: in any) whose finest level is
-// above `above`, at most kListMax of the slots from `base`, in slot order, with the levels they are taken at (level,
-// or 0: their own finest).  The whole block; returns the number of problems.  Every block of a launch has
-// to find the same list, so a launch that changes phases lists problems in any.
-struct Served {
-  unsigned short slot[kListMax];
-  unsigned char level[kListMax];
-  int start[kListMax + 1];
-  int count[32];
-};
-__device__ int list_served(const EngineDev& E, Served& q, int base, int want, int above, int level) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
-  const int n = min(kListMax, E.nprob - base);
-  // slots of a warp: a contiguous share, read in one go (the loads of a round do not depend on each other)
-  const int share = (n + nw * 32 - 1) / (nw * 32);
-  const int lo = warp * share * 32;
-  unsigned take = 0;
-  for (int k = 0; k < share; ++k) {
-    const int p = lo + k * 32 + lane;
-    const bool on = p < n && (want < 0 || E.S[base + p].phase == want) && E.P[base + p].L > above;
-    take |= on ? 1u << k : 0u;
-  }
-  int mine = 0;
-  for (int k = 0; k < share; ++k) mine += __popc(__ballot_sync(kFull, (take >> k) & 1u));
-  if (lane == 0) q.count[warp] = mine;
-  __syncthreads();
-  int at = 0, total = 0;
-  for (int w = 0; w < nw; ++w) {
-    if (w < warp) at += q.count[w];
-    total += q.count[w];
-  }
-  for (int k = 0; k < share; ++k) {
-    const bool on = (take >> k) & 1u;
-    const unsigned m = __ballot_sync(kFull, on);
-    if (on) {
-      const int i = at + __popc(m & ((1u << lane) - 1u)), p = base + lo + k * 32 + lane;
-      q.slot[i] = (unsigned short)p;
-      q.level[i] = (unsigned char)(level ? level : E.P[p].L);
-    }
-    at += __popc(m);
-  }
-  __syncthreads();
-  return total;
-}
-// running numbers of the problems' work items (items: of a level; 32-bit arithmetic only: a round of 32
-// problems is on every block's way to its first load); the whole block; returns their sum
-template <class F>
-__device__ int number_items(Served& q, int n, F&& items) {
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < 32) {
-    int run = 0;
-    for (int b = 0; b < n; b += 32) {
-      const int c = b + lane < n ? items((int)q.level[b + lane]) : 0;
-      int s = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, s, o);
-        if (lane >= o) s += t;
-      }
-      if (b + lane < n) q.start[b + lane] = run + s - c;
-      run += __shfl_sync(kFull, s, 31);
-    }
-    if (lane == 0) q.start[n] = run;
-  }
-  __syncthreads();
-  return q.start[n];
-}
-// the problem of work item `it`
-__device__ __forceinline__ int served_of(const Served& q, int n, int it) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (q.start[mid] <= it) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // The down or up part of level `level` for the problems with a finer level, or (level 0) of every problem's
 // own finest level above the tail level T, in one launch: the strips of all problems in the phase are cut
 // into chunks of one height, so that they fill one wave of warps.
@@ -757,7 +670,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march_group(EngineDev E, int
   }
   pdl_wait();
   for (int base = 0; base < E.nprob; base += kListMax) {
-    const int n = list_served(E, q, base, want, level ? level : T, level);
+    const int n = list_served(E, q, base, level, [&](const ProbState& S, int L) { return S.phase == want && L > (level ? level : T); });
     if (n == 0) continue;
     // one height for all chunks: the smallest of 32 candidates that takes no more items than warps
     if (threadIdx.x < kMaxLevel + 1) hist[threadIdx.x] = 0;
@@ -832,23 +745,23 @@ __device__ void check_part(const EngineDev& E, int p, const float* squares, int 
     const float2 q = tile_pairs(squares, t, hi);
     if (t + lane < hi) store_partial(part + t + lane, q);
   }
-  unsigned* ticket = E.gticket + (long long)p * (E.ctl_groups + 1);
+  unsigned* ticket = E.gticket + (long long)p * ticket_words(E.ctl_groups);
   double* gsum = E.gsum + (long long)p * E.ctl_groups;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(ticket + j, 1u) == (unsigned)nb - 1u;
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket + 2 + j, 1u) == (unsigned)nb - 1u;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   const double g = group_partial_sum(part, tiles, j, sh, true);
   __syncthreads();
   if (threadIdx.x == 0) {
-    ticket[j] = 0u;
+    ticket[2 + j] = 0u;
     s_last = 1;
     if (groups > 1) {
       gsum[j] = g;
       __threadfence();
-      s_last = atomicAdd(ticket + E.ctl_groups, 1u) == (unsigned)groups - 1u;
+      s_last = atomicAdd(ticket + 1, 1u) == (unsigned)groups - 1u;
     }
   }
   __syncthreads();
@@ -864,7 +777,7 @@ __device__ void check_part(const EngineDev& E, int p, const float* squares, int 
   }
   if (threadIdx.x == 0) {
     ProbState& st = E.S[p];
-    if (groups > 1) ticket[E.ctl_groups] = 0u;
+    if (groups > 1) ticket[1] = 0u;
     pre_check(st, E.prm, sqrt(sum));
     if (st.phase == want) cond_set(E.prm.cond, 0, 1u);
   }
@@ -892,7 +805,7 @@ __global__ void __launch_bounds__(256) k_march_check_group(EngineDev E, int T, i
     return l <= T ? 1 : sum_groups(tiles) * ((min(tiles, kSumGroup) + 1023) / 1024);
   };
   for (int base = 0; base < E.nprob; base += kListMax) {
-    const int n = list_served(E, q, base, -1, HN_MIN_LEVEL - 1, 0);
+    const int n = list_served(E, q, base, 0, [](const ProbState&, int L) { return L >= HN_MIN_LEVEL; });
     if (n == 0) continue;
     const int items = number_items(q, n, blocks);
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
