@@ -899,6 +899,13 @@ bool Engine::small_tail() const {
          !tune_.staged && !tune_.fuse_up && std::max(tune_.tail_level, prm_.coarse) <= kSmallTop;
 }
 
+// The FP64 counterpart over a cluster of 16 blocks (k_wide).
+bool Engine::wide_tail() const {
+  const int T = std::max(tune_.tail_level, prm_.coarse);
+  return tune_.march && tune_.sweep == 1 && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
+         tune_.cluster == 16 && T > 4 && T <= kWideTop;
+}
+
 hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   const int c = prm_.coarse, pre = prm_.pre, post = prm_.post;
   const int T = std::max(tune_.tail_level, c);
@@ -973,6 +980,7 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   }
   if (M > T) HN_LAUNCH(KC_MID_DOWN, M, launch_mid(E_, dLists_, M, T, want, 0, s));
   if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, T, want, s));
+  else if (wide_tail()) HN_LAUNCH(KC_TAIL, T, launch_wide(E_, T, want, Lmax_ <= T, s));
   else HN_LAUNCH(KC_TAIL, T, launch_tail(E_, T, want, tune_.cluster, s));
   if (M > T) HN_LAUNCH(KC_MID_UP, M, launch_mid(E_, dLists_, M, T, want, 1, s));
   int e_sel = 0;                           // buffer of the coarse iterate (the tail's: 0)

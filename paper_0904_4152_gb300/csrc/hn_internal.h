@@ -244,6 +244,10 @@ struct SmallSolo {
   LevelDev lev[kSmallTop - 1] = {};      // levels 2..min(L, kSmallTop)
 };
 cudaError_t launch_small(const EngineDev& E, const SmallSolo& solo, int T, int want, cudaStream_t s);
+// the same on levels coarse..T <= kWideTop of FP64 hierarchies by a cluster of 16 blocks per problem slot
+// (k_wide.cu).  loop: a problem whose finest level is here runs its cycles until it leaves the phase
+constexpr int kWideTop = 6;
+cudaError_t launch_wide(const EngineDev& E, int T, int want, int loop, cudaStream_t s);
 // one-time kernel attributes (cluster-size opt-in); call outside stream capture
 cudaError_t prepare_kernels();
 
