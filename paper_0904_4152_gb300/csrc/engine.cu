@@ -896,7 +896,14 @@ bool Engine::march_level(int l) const {
 // conditions of the marching sweeps and with the exact coarse solver.
 bool Engine::small_tail() const {
   return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
-         !tune_.staged && !tune_.fuse_up && std::max(tune_.tail_level, prm_.coarse) <= kSmallTop;
+         !tune_.staged && !tune_.fuse_up && std::min(std::max(tune_.tail_level, prm_.coarse), cap_ == 1 ? Lmax_ : kMaxLevel) <= kSmallTop;
+}
+
+// An FP32 / FP16 problem alone: the tail over a cluster of 16 blocks (k_span).
+bool Engine::span_tail() const {
+  const int T = std::max(tune_.tail_level, prm_.coarse);
+  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
+         !tune_.staged && !tune_.fuse_up && tune_.cluster == 16 && cap_ == 1 && std::min(T, Lmax_) > kSmallTop && T <= kSpanTop;
 }
 
 // The FP64 counterpart over a cluster of 16 blocks (k_wide).
@@ -979,7 +986,8 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
     HN_LAUNCH(KC_RESTRICT, l, launch_restrict(E_, lists_[l - 1], l, want, grid_[l - 1], s));
   }
   if (M > T) HN_LAUNCH(KC_MID_DOWN, M, launch_mid(E_, dLists_, M, T, want, 0, s));
-  if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, T, want, s));
+  if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, std::min(T, kSmallTop), want, s));
+  else if (span_tail()) HN_LAUNCH(KC_TAIL, T, launch_span(E_, T, want, Lmax_ <= T, s));
   else if (wide_tail()) HN_LAUNCH(KC_TAIL, T, launch_wide(E_, T, want, Lmax_ <= T, s));
   else HN_LAUNCH(KC_TAIL, T, launch_tail(E_, T, want, tune_.cluster, s));
   if (M > T) HN_LAUNCH(KC_MID_UP, M, launch_mid(E_, dLists_, M, T, want, 1, s));

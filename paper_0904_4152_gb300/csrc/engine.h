@@ -281,6 +281,7 @@ class Engine {
   bool sweep_level(int l) const;    // level l's down / up parts run as fused sweeps
   bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
   bool wide_tail() const;           // the FP64 tail of a cluster of 16 blocks (k_wide)
+  bool span_tail() const;           // the FP32 / FP16 tail of a cluster of 16 blocks (k_span)
   bool small_tail() const;          // the tail runs in one block's shared memory (k_small)
   SmallSolo small_{};               // its descriptors, for an engine of one problem
   // level l may be a member's own finest level (the server's engines: any level)

@@ -248,6 +248,9 @@ cudaError_t launch_small(const EngineDev& E, const SmallSolo& solo, int T, int w
 // (k_wide.cu).  loop: a problem whose finest level is here runs its cycles until it leaves the phase
 constexpr int kWideTop = 6;
 cudaError_t launch_wide(const EngineDev& E, int T, int want, int loop, cudaStream_t s);
+// the same on levels coarse..T <= kSpanTop of FP32 / FP16 hierarchies (k_span.cu); finest levels above 5 only
+constexpr int kSpanTop = 8;
+cudaError_t launch_span(const EngineDev& E, int T, int want, int loop, cudaStream_t s);
 // one-time kernel attributes (cluster-size opt-in); call outside stream capture
 cudaError_t prepare_kernels();
 

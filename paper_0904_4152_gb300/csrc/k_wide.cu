@@ -389,7 +389,7 @@ __device__ __forceinline__ void run(const Job& j, const Peers& c, Node* q, bool 
   }
 }
 
-__global__ void __launch_bounds__(kWideThreads, 1) k_wide(EngineDev E, int T, int want, int loop) {
+__global__ void __launch_bounds__(kWideThreads, 1) k_wide(const __grid_constant__ EngineDev E, int T, int want, int loop) {
   __shared__ Wide s;
   pdl_trigger();
   cg::cluster_group cl = cg::this_cluster();
