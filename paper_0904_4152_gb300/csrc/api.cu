@@ -8,6 +8,8 @@
 #include <memory>
 #include <mutex>
 
+#include <cuda.h>
+
 #include "engine.h"
 #include "../../include/hn_profile.h"
 #include "../../include/hn_tune.h"
@@ -34,9 +36,8 @@ void exact_caps(const std::vector<hn_mg*>& mgs, std::vector<long long>& caps, lo
 
 // the engine's device error words after a solve: a bounded wait that gave up, or (debug builds) a
 // failed index check
-hn_status device_error(Engine& e) {
-  int d[4] = {0, 0, 0, 0};
-  HN_TRY(e.read_error_detail(d));
+hn_status device_error(const Engine& e) {
+  const int* d = e.error();
   switch (d[0]) {
     case 0: return HN_OK;
     case 3: return set_error(HN_ERR_CUDA, "a grid barrier of the persistent kernels timed out");
@@ -124,6 +125,34 @@ hn_status check_ptr(const void* p, int device_ptrs) {
   if (device_ptrs && (reinterpret_cast<uintptr_t>(p) & 15))
     return set_error(HN_ERR_ARG, "device vectors must be 16-byte aligned");
   return HN_OK;
+}
+
+// Whether the n doubles at p are one allocation in the current device's own memory, which a kernel may read or write
+// as they are (anything else goes through the runtime's copies, which check it).
+bool in_device_memory(const void* p, long long n) {
+  using Fn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Fn query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Fn>(f);
+  }();
+  int dev = 0;
+  if (!query || cudaGetDevice(&dev) != cudaSuccess) return false;
+  CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                 CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  unsigned type = 0, managed = 0;
+  int ordinal = -1;
+  CUdeviceptr base = 0, at = reinterpret_cast<uintptr_t>(p);
+  size_t size = 0;
+  void* out[5] = {&type, &ordinal, &managed, &base, &size};
+  return query(5, what, out, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && !managed && ordinal == dev &&
+         at >= base && at - base + (size_t)n * 8 <= size;
 }
 
 void fill_stats(const hn_mg* mg, const ProbState& st, long long t0, hn_mg_stats* out) {
@@ -311,16 +340,23 @@ hn_status hn_mg_solve(hn_mg* mg, const double* b, double* x, int x_is_guess, int
   cudaStream_t s = e.stream();
   const long long N = N_of(mg->L);
   ProblemDev& P = mg->host;
-  HN_TRY(copy_in(P.b64, b, N, device_ptrs, s));
-  if (x_is_guess) HN_TRY(copy_in(P.x64, x, N, device_ptrs, s));
-  else HN_CUDA(cudaMemsetAsync(P.x64, 0, (size_t)N * 8, s));
-  HN_TRY(e.start({0}, {x_is_guess ? 1 : 0}));
-  HN_TRY(e.run_to_completion());
+  std::vector<IoItem> io(1, IoItem{});
   std::vector<ProbState> st;
-  HN_TRY(e.read_states(st));
+  const bool b_here = device_ptrs && in_device_memory(b, N), x_here = device_ptrs && in_device_memory(x, N);
+  io[0].guess = x_is_guess ? 1 : 0;
+  io[0].clear = !x_is_guess;
+  if (b_here) io[0].b = b;
+  else HN_TRY(copy_in(P.b64, b, N, device_ptrs, s));
+  if (x_is_guess) {
+    if (x_here) io[0].x = x;
+    else HN_TRY(copy_in(P.x64, x, N, device_ptrs, s));
+  }
+  HN_TRY(e.begin(io));
+  HN_TRY(e.run_to_completion());
+  io[0].x = x_here ? x : nullptr;
+  HN_TRY(e.finish(io, st));
   HN_TRY(device_error(e));
-  if (st[0].status != HN_ERR_ARG) {
-    if (st[0].status == HN_OK && st[0].bnorm == 0.0) HN_CUDA(cudaMemsetAsync(P.x64, 0, (size_t)N * 8, s));
+  if (!x_here && st[0].status != HN_ERR_ARG) {
     HN_TRY(copy_out(x, P.x64, N, device_ptrs, s));
     HN_CUDA(cudaStreamSynchronize(s));
   }
@@ -379,30 +415,39 @@ hn_status hn_mg_solve_batch(hn_mg* const* mgs, int count, const double* const* b
     if (!(t == e.tuning())) e.set_tuning(t);
   }
   cudaStream_t s = e.stream();
-  std::vector<int> slots(count), guess(count, 0);
-  for (int j = 0; j < count; ++j) {
-    slots[j] = j;
-    ProblemDev& P = list[j]->host;
-    const long long N = N_of(list[j]->L);
-    HN_TRY(copy_in(P.b64, b[j], N, device_ptrs, s));
-    HN_CUDA(cudaMemsetAsync(P.x64, 0, (size_t)N * 8, s));
-  }
-  HN_TRY(e.start(slots, guess));
-  HN_TRY(e.run_to_completion());
+  std::vector<IoItem> io(count, IoItem{});
   std::vector<ProbState> st;
-  HN_TRY(e.read_states(st));
+  // results that overlap are copied out one after the other
+  std::vector<std::pair<uintptr_t, int>> order(count);
+  for (int j = 0; j < count; ++j) order[j] = {reinterpret_cast<uintptr_t>(x[j]), j};
+  std::sort(order.begin(), order.end());
+  bool apart = true;
+  for (int j = 0; j + 1 < count; ++j)
+    apart = apart && order[j].first + (uintptr_t)N_of(list[order[j].second]->L) * 8 <= order[j + 1].first;
+  std::vector<char> x_here(count);
+  for (int j = 0; j < count; ++j) {
+    const long long N = N_of(list[j]->L);
+    io[j].slot = j;
+    io[j].clear = 1;
+    x_here[j] = device_ptrs && apart && in_device_memory(x[j], N);
+    if (device_ptrs && in_device_memory(b[j], N)) io[j].b = b[j];
+    else HN_TRY(copy_in(list[j]->host.b64, b[j], N, device_ptrs, s));
+  }
+  HN_TRY(e.begin(io));
+  HN_TRY(e.run_to_completion());
+  for (int j = 0; j < count; ++j) io[j].x = x_here[j] ? x[j] : nullptr;
+  HN_TRY(e.finish(io, st));
   HN_TRY(device_error(e));
   hn_status first_bad = HN_OK;
+  bool copied = false;
   for (int j = 0; j < count; ++j) {
-    ProblemDev& P = list[j]->host;
-    const long long N = N_of(list[j]->L);
-    if (st[j].status != HN_ERR_ARG) {
-      if (st[j].status == HN_OK && st[j].bnorm == 0.0) HN_CUDA(cudaMemsetAsync(P.x64, 0, (size_t)N * 8, s));
-      HN_TRY(copy_out(x[j], P.x64, N, device_ptrs, s));
+    if (!x_here[j] && st[j].status != HN_ERR_ARG) {
+      HN_TRY(copy_out(x[j], list[j]->host.x64, N_of(list[j]->L), device_ptrs, s));
+      copied = true;
     }
     if (st[j].status != HN_OK && first_bad == HN_OK) first_bad = (hn_status)st[j].status;
   }
-  HN_CUDA(cudaStreamSynchronize(s));
+  if (copied) HN_CUDA(cudaStreamSynchronize(s));
   for (int j = 0; j < count; ++j) fill_stats(list[j], st[j], t0, stats ? stats + j : nullptr);
   if (first_bad != HN_OK) return set_error(first_bad, "at least one batch member did not converge cleanly");
   return HN_OK;

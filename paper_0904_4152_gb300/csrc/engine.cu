@@ -473,7 +473,7 @@ void Engine::destroy_graphs() {
   if (gInit_) cudaGraphExecDestroy(gInit_);
   if (gIter_) cudaGraphExecDestroy(gIter_);
   gSolve_ = gInit_ = gIter_ = nullptr;
-  graphsValid_ = false;
+  drop_graphs();
 }
 
 int Engine::grid_for(long long tiles) const {
@@ -553,17 +553,17 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   HN_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&hLists_), sizeof(TileList) * (kMaxLevel + 1),
                         cudaHostAllocDefault));
   HN_CUDA(cudaEventCreateWithFlags(&upEv_, cudaEventDisableTiming));
-  HN_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&hActive_), sizeof(unsigned), cudaHostAllocMapped));
-  *hActive_ = 0;
-  unsigned* dActive = nullptr;
-  HN_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dActive), hActive_, 0));
+  const size_t mapped = 128 + sizeof(ProbState) * cap;
+  HN_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&hActive_), mapped, cudaHostAllocMapped));
+  std::memset(hActive_, 0, mapped);
+  HN_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dActive_), hActive_, 0));
   E_.P = dP_;
   E_.S = dS_;
   E_.fine_off = dFineOff_;
   E_.partial = part;
   E_.nprob = cap;
   E_.prm = prm;
-  E_.active_host = dActive;
+  E_.active_host = reinterpret_cast<unsigned*>(dActive_);
   E_.iter = iter;
   E_.pdl = tune_.pdl;
   E_.err = dErr_;
@@ -636,7 +636,7 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
   HN_CUDA(cudaEventRecord(upEv_, s_));
   // an engine of one problem passes its descriptors to the kernels by value (captured into its
   // graphs, which therefore must be captured again when its member changes)
-  if (cap_ == 1) graphsValid_ = false;
+  if (cap_ == 1) drop_graphs();
   for (int l = 0; l <= kMaxLevel; ++l) {
     TileList& t = lists_[l];
     t.solo_tiles = 0;
@@ -671,34 +671,51 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
   unsigned mask = 0;
   for (hn_mg* mg : members_)
     if (mg) mask |= 1u << mg->L;
-  if (mask != topMask_ && !topMaskAll_) graphsValid_ = false;
+  if (mask != topMask_ && !topMaskAll_) drop_graphs();
   topMask_ = mask;
   return HN_OK;
 }
 
-hn_status Engine::start(const std::vector<int>& slots, const std::vector<int>& have_guess) {
-  for (size_t q = 0; q < slots.size(); ++q) {
-    ProbState st;
-    std::memset(&st, 0, sizeof st);
-    st.phase = PH_INIT;
-    st.status = HN_PENDING;
-    const int g = q < have_guess.size() ? have_guess[q] : 0;
-    st.zero_top = g ? 0 : 1;
-    st.x_zero = g ? 0 : 1;
-    st.s = 1.0;
-    st.inv_s = 1.0;
-    HN_CUDA(cudaMemcpyAsync(dS_ + slots[q], &st, sizeof st, cudaMemcpyHostToDevice, s_));
+// the kernels of k_io.cu over the items, kIoMax at a time
+hn_status Engine::io_launches(std::vector<IoItem>& io, bool begin) {
+  for (size_t at = 0; at < io.size(); at += kIoMax) {
+    IoBatch p;
+    p.n = (int)std::min<size_t>(kIoMax, io.size() - at);
+    p.first = at == 0;
+    long long most = 0;
+    for (int k = 0; k < p.n; ++k) {
+      p.item[k] = io[at + k];
+      const hn_mg* mg = members_[p.item[k].slot];
+      if (mg && (p.item[k].b || p.item[k].x || p.item[k].clear)) most = std::max(most, N_of(mg->L));
+    }
+    if (begin) HN_CUDA(launch_begin(E_, p, most, dTaken_, dLaunches_, s_));
+    else HN_CUDA(launch_finish(E_, p, most, dLaunches_, reinterpret_cast<ProbState*>(dActive_ + 128),
+                               reinterpret_cast<IoResult*>(dActive_ + 64), s_));
   }
-  // the iteration counter restarts with every closed-world solve (serving keeps counting and
-  // relies on per-problem caps; its limit is set out of reach)
-  HN_CUDA(cudaMemsetAsync(E_.iter, 0, sizeof(unsigned), s_));
-  HN_CUDA(cudaMemsetAsync(dErr_, 0, sizeof(int) * 4, s_));
-  HN_CUDA(cudaMemsetAsync(dBar_, 0, sizeof(unsigned long long) * 3, s_));
-  HN_CUDA(cudaMemsetAsync(E_.ticket, 0, sizeof(unsigned), s_));
-  // mirrors of the IF values as the closed-world graph sets them at its launch
-  static const unsigned taken0[4] = {0u, 1u, 0u, 0u};
-  HN_CUDA(cudaMemcpyAsync(dTaken_, taken0, sizeof taken0, cudaMemcpyHostToDevice, s_));
-  HN_CUDA(cudaMemsetAsync(dLaunches_, 0, sizeof(unsigned long long), s_));
+  return HN_OK;
+}
+
+hn_status Engine::start(const std::vector<int>& slots, const std::vector<int>& have_guess) {
+  std::vector<IoItem> io(slots.size(), IoItem{});
+  for (size_t q = 0; q < slots.size(); ++q) {
+    io[q].slot = slots[q];
+    io[q].guess = q < have_guess.size() ? have_guess[q] : 0;
+  }
+  return io_launches(io, true);
+}
+
+hn_status Engine::begin(std::vector<IoItem>& io) { return io_launches(io, true); }
+
+hn_status Engine::finish(std::vector<IoItem>& io, std::vector<ProbState>& out) {
+  HN_TRY(io_launches(io, false));
+  HN_CUDA(cudaStreamSynchronize(s_));
+  out.assign(host_states(), host_states() + cap_);
+  if (!profiling_) {
+    // the init graph's summary also counts one iteration; with IF nodes the loop counts the
+    // kernels it ran, otherwise each body iteration runs iterLaunches_ kernels
+    const long long iters = result()->iterations;
+    lastLaunches_ = initLaunches_ + (condUsed_ ? (long long)result()->launches : (iters > 0 ? iters - 1 : 0) * iterLaunches_);
+  }
   return HN_OK;
 }
 
@@ -1070,9 +1087,10 @@ hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h,
   return HN_OK;
 }
 
-hn_status Engine::capture_graphs() {
-  destroy_graphs();
-  clear_marks();
+// one host-driven piece: the init, or an iteration
+hn_status Engine::capture_piece(cudaGraphExec_t* out, int* launches, bool init) {
+  if (*out) cudaGraphExecDestroy(*out);
+  *out = nullptr;
   cudaStream_t cs;
   HN_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   // graphs carry no profiling events (profiled iterations are issued directly)
@@ -1082,43 +1100,37 @@ hn_status Engine::capture_graphs() {
   } guard{cs, profiling_, profiling_};
   profiling_ = false;
   const cudaGraphConditionalHandle none = 0;
-  // host-driven pieces: init and one iteration
-  {
-    cudaGraph_t g;
-    HN_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    counting_ = 0;
-    hn_status st = issue_init(cs, none, 0);
-    initLaunches_ = counting_;
-    cudaError_t e = cudaStreamEndCapture(cs, &g);
-    HN_TRY(st);
-    HN_CUDA(e);
-    e = cudaGraphInstantiate(&gInit_, g, 0);
-    cudaGraphDestroy(g);
-    HN_CUDA(e);
+  cudaGraph_t g;
+  HN_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+  counting_ = 0;
+  const hn_status st = init ? issue_init(cs, none, 0) : issue_iteration(cs, none, 0);
+  *launches = counting_;
+  cudaError_t e = cudaStreamEndCapture(cs, &g);
+  HN_TRY(st);
+  HN_CUDA(e);
+  e = cudaGraphInstantiate(out, g, 0);
+  cudaGraphDestroy(g);
+  HN_CUDA(e);
+  return HN_OK;
+}
+
+hn_status Engine::capture_steps() {
+  clear_marks();
+  HN_TRY(capture_piece(&gInit_, &initLaunches_, true));
+  HN_TRY(capture_piece(&gIter_, &iterLaunches_, false));
+  stepsValid_ = true;
+  return HN_OK;
+}
+
+// closed-world solve: init, then while (any problem running) { iteration }, with the IF node
+// that skips the rest of a cycle no problem is in; the flat loop if that does not build
+hn_status Engine::capture_loop() {
+  clear_marks();
+  if (capture_solve(true) != HN_OK) {
+    cudaGetLastError();
+    HN_TRY(capture_solve(false));
   }
-  {
-    cudaGraph_t g;
-    HN_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    counting_ = 0;
-    hn_status st = issue_iteration(cs, none, 0);
-    iterLaunches_ = counting_;
-    cudaError_t e = cudaStreamEndCapture(cs, &g);
-    HN_TRY(st);
-    HN_CUDA(e);
-    e = cudaGraphInstantiate(&gIter_, g, 0);
-    cudaGraphDestroy(g);
-    HN_CUDA(e);
-  }
-  // closed-world solve: init, then while (any problem running) { iteration }, with the IF node
-  // that skips the rest of a cycle no problem is in; the flat loop if that does not build
-  {
-    hn_status st = capture_solve(true);
-    if (st != HN_OK) {
-      cudaGetLastError();
-      HN_TRY(capture_solve(false));
-    }
-  }
-  graphsValid_ = true;
+  solveValid_ = true;
   return HN_OK;
 }
 
@@ -1173,7 +1185,9 @@ hn_status Engine::capture_solve(bool cond) {
   }
   cudaGraph_t init;
   HN_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+  counting_ = 0;
   hn_status st = issue_init(cs, none, 0);
+  initLaunches_ = counting_;
   cudaError_t e = cudaStreamEndCapture(cs, &init);
   HN_TRY(st);
   HN_CUDA(e);
@@ -1197,6 +1211,7 @@ hn_status Engine::capture_solve(bool cond) {
   condCapture_ = cd.mask != 0;
   counting_ = 0;
   st = issue_iteration(cs, h, 0);
+  iterLaunches_ = counting_;
   if (st == HN_OK) {
     CondDev cd2 = cd;
     cd2.h_cycle = hCond_[1][0];
@@ -1234,17 +1249,8 @@ hn_status Engine::run_to_completion() {
     }
     return HN_OK;
   }
-  if (!graphsValid_) HN_TRY(capture_graphs());
+  if (!solveValid_) HN_TRY(capture_loop());
   HN_CUDA(cudaGraphLaunch(gSolve_, s_));
-  unsigned iters = 0;
-  unsigned long long body = 0;
-  HN_CUDA(cudaMemcpyAsync(&iters, E_.iter, sizeof iters, cudaMemcpyDeviceToHost, s_));
-  HN_CUDA(cudaMemcpyAsync(&body, dLaunches_, sizeof body, cudaMemcpyDeviceToHost, s_));
-  HN_CUDA(cudaStreamSynchronize(s_));
-  // the init graph's summary also counts one iteration; with IF nodes the loop counts the
-  // kernels it ran, otherwise each body iteration runs iterLaunches_ kernels
-  lastLaunches_ = initLaunches_ + (condUsed_ ? (long long)body
-                                             : (long long)(iters > 0 ? iters - 1 : 0) * iterLaunches_);
   return HN_OK;
 }
 
@@ -1258,7 +1264,7 @@ hn_status Engine::run_init() {
     initLaunches_ = counting_;
     return HN_OK;
   }
-  if (!graphsValid_) HN_TRY(capture_graphs());
+  if (!stepsValid_) HN_TRY(capture_steps());
   HN_CUDA(cudaGraphLaunch(gInit_, s_));
   return HN_OK;
 }
@@ -1278,7 +1284,7 @@ hn_status Engine::launch_iteration() {
     HN_TRY(accumulate_marks());
     clear_marks();
   } else {
-    if (!graphsValid_) HN_TRY(capture_graphs());
+    if (!stepsValid_) HN_TRY(capture_steps());
     HN_CUDA(cudaGraphLaunch(gIter_, s_));
   }
   return HN_OK;
@@ -1312,7 +1318,7 @@ hn_status Engine::accumulate_marks() {
 
 void Engine::set_profiling(bool on) {
   profiling_ = on;
-  graphsValid_ = false;
+  drop_graphs();
   for (auto& row : acc_)
     for (auto& a : row) a = Acc{};
 }
@@ -1346,12 +1352,6 @@ int Engine::kernel_times(hn_kernel_time* out, int max) const {
 hn_status Engine::read_states(std::vector<ProbState>& out) {
   out.resize(cap_);
   HN_CUDA(cudaMemcpyAsync(out.data(), dS_, sizeof(ProbState) * cap_, cudaMemcpyDeviceToHost, s_));
-  HN_CUDA(cudaStreamSynchronize(s_));
-  return HN_OK;
-}
-
-hn_status Engine::read_error_detail(int (&err)[4]) {
-  HN_CUDA(cudaMemcpyAsync(err, dErr_, sizeof(int) * 4, cudaMemcpyDeviceToHost, s_));
   HN_CUDA(cudaStreamSynchronize(s_));
   return HN_OK;
 }

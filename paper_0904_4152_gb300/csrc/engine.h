@@ -196,10 +196,15 @@ class Engine {
                    long long fine_cap, cudaStream_t s);
   // assign hierarchies to slots (nullptr = empty slot) and rewrite the device work lists
   hn_status set_members(const std::vector<hn_mg*>& slots);
-  // reset the state of the given slots for a new solve
+  // reset the state of the given slots for a new solve, whose vectors are in place
   hn_status start(const std::vector<int>& slots, const std::vector<int>& have_guess);
-  // closed-world solve of all members: device-side loop in one graph launch
+  // the same for a closed-world solve of the members in slots 0, 1, ..: io[j] copies slot j's vectors in
+  hn_status begin(std::vector<IoItem>& io);
+  // closed-world solve of all members: device-side loop in one graph launch (returns without waiting unless profiling)
   hn_status run_to_completion();
+  // its end: results out (io[j].x), all states, and error() and last_launches() of this solve
+  hn_status finish(std::vector<IoItem>& io, std::vector<ProbState>& out);
+  const int* error() const { return result()->err; }
   // host-driven steps (serving / profiling)
   hn_status run_init();
   hn_status run_iteration(unsigned* active_out);
@@ -210,8 +215,6 @@ class Engine {
   hn_status read_states(std::vector<ProbState>& out);
   // the device error word (a bounded wait gave up); reset by start()
   hn_status read_error(int* err);
-  // the device error word and the details a failed debug check recorded (source line, two indices)
-  hn_status read_error_detail(int (&err)[4]);
   // the guards of the engine's device block (debug builds)
   hn_status check_guards() const;
   hn_status read_states_async(ProbState* host_dst);
@@ -221,14 +224,14 @@ class Engine {
   hn_status set_phase(int slot, int phase, int zero_top);
 
   void set_profiling(bool on);
-  void set_iter_limit(unsigned lim) { E_.iter_limit = lim; graphsValid_ = false; }
+  void set_iter_limit(unsigned lim) { E_.iter_limit = lim; drop_graphs(); }
   void set_tuning(const Tuning& t) {
-    tune_ = t; E_.pdl = t.pdl; E_.staged = t.staged; E_.dsm = t.dsm; graphsValid_ = false;
+    tune_ = t; E_.pdl = t.pdl; E_.staged = t.staged; E_.dsm = t.dsm; drop_graphs();
   }
   const Tuning& tuning() const { return tune_; }
   // levels that may be some problem's finest level (their first smoothing step may start from a
   // nonzero iterate); all levels for the server
-  void set_top_mask_all() { topMaskAll_ = true; graphsValid_ = false; }
+  void set_top_mask_all() { topMaskAll_ = true; drop_graphs(); }
   int kernel_times(hn_kernel_time* out, int max) const;
 
   long long last_launches() const { return lastLaunches_; }
@@ -237,7 +240,13 @@ class Engine {
   cudaStream_t stream() const { return s_; }
 
  private:
-  hn_status capture_graphs();
+  hn_status capture_steps();        // gInit_, gIter_: the host-driven pieces (serving)
+  hn_status capture_loop();         // gSolve_: closed-world solves
+  hn_status capture_piece(cudaGraphExec_t* out, int* launches, bool init);
+  void drop_graphs() { solveValid_ = stepsValid_ = false; }
+  hn_status io_launches(std::vector<IoItem>& io, bool begin);
+  IoResult* result() const { return reinterpret_cast<IoResult*>(reinterpret_cast<char*>(hActive_) + 64); }
+  ProbState* host_states() const { return reinterpret_cast<ProbState*>(reinterpret_cast<char*>(hActive_) + 128); }
   hn_status issue_init(cudaStream_t s, cudaGraphConditionalHandle h, int use_h);
   hn_status issue_iteration(cudaStream_t s, cudaGraphConditionalHandle h, int use_h);
   hn_status issue_vcycle(cudaStream_t s, int want);
@@ -257,7 +266,8 @@ class Engine {
   void* mem_ = nullptr;
   void* memBase_ = nullptr;      // mem_ with its guards
   size_t memBytes_ = 0;
-  unsigned* hActive_ = nullptr;  // mapped pinned
+  unsigned* hActive_ = nullptr;  // mapped pinned: running problems; at 64 the end of a solve, at 128 its states
+  char* dActive_ = nullptr;      // its device address
   EngineDev E_{};
   ProblemDev* dP_ = nullptr;
   ProbState* dS_ = nullptr;
@@ -298,7 +308,7 @@ class Engine {
   }
   size_t stage_bytes() const { return stage_probs_off() + sizeof(ProblemDev) * cap_; }
   cudaGraphExec_t gSolve_ = nullptr, gInit_ = nullptr, gIter_ = nullptr;
-  bool graphsValid_ = false;
+  bool solveValid_ = false, stepsValid_ = false;
   int initLaunches_ = 0, iterLaunches_ = 0, counting_ = 0;
   Tuning tune_{};
   unsigned topMask_ = 0;

@@ -251,6 +251,17 @@ cudaError_t launch_wide(const EngineDev& E, int T, int want, int loop, cudaStrea
 // the same on levels coarse..T <= kSpanTop of FP32 / FP16 hierarchies (k_span.cu); finest levels above 5 only
 constexpr int kSpanTop = 8;
 cudaError_t launch_span(const EngineDev& E, int T, int want, int loop, cudaStream_t s);
+// The start and the end of a solve (k_io.cu).  b: right-hand side to copy in (or null: it is in place); x: at the start
+// the given iterate to copy in (or null: clear: start from zeros, else it is in place), at the end where the result
+// goes (or null).  Device vectors, 16-byte aligned.  first: reset / read the engine's counters too.
+constexpr int kIoMax = 96;
+struct IoItem { const double* b; const double* x; int slot, guess, clear, pad; };
+struct IoBatch { IoItem item[kIoMax]; int n, first; };
+struct IoResult { unsigned long long launches; unsigned iterations; int err[4]; };
+cudaError_t launch_begin(const EngineDev& E, const IoBatch& io, long long most, unsigned* taken, unsigned long long* launches,
+                         cudaStream_t s);
+cudaError_t launch_finish(const EngineDev& E, const IoBatch& io, long long most, const unsigned long long* launches,
+                          ProbState* states, IoResult* result, cudaStream_t s);
 // one-time kernel attributes (cluster-size opt-in); call outside stream capture
 cudaError_t prepare_kernels();
 
