@@ -1,6 +1,8 @@
 // BLAS level-1 kernels (axpy, dot, nrm2) on device vectors: the memory-bound operations the paper
 // measures on every backend (Sec. 6.1, Fig. 2).  The declarations and their contract are in
 // include/hn_blas1.h.
+#include <mutex>
+
 #include "engine.h"
 #include "../../include/hn_blas1.h"
 
@@ -178,6 +180,42 @@ hn_status check_common(hn_dtype t, long long n) {
   return HN_OK;
 }
 
+// The pool of the reductions' scratch on the current device.  The device's default pool gives its memory back to the
+// // system at every synchronization, so that the next reduction mapped it anew (a dot at L = 11 after one 121 us, now
+// 36); this one keeps up to 64 MiB, two of the units in which a pool takes memory.  Allocations stay
+// stream-ordered, as before.
+hn_status scratch_pool(cudaMemPool_t* out) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mu;
+  static cudaMemPool_t pools[kMaxDevices] = {};
+  int dev = 0;
+  HN_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return set_error(HN_ERR_ARG, "device ordinal %d unsupported", dev);
+  std::lock_guard<std::mutex> lk(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    unsigned long long keep = 64ull << 20;
+    // (a capture may be under way on another stream or thread: creating a pool does not touch it)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    HN_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    if (e == cudaSuccess) {
+      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      if (e != cudaSuccess) cudaMemPoolDestroy(pool);
+    }
+    const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+    HN_CUDA(e);
+    HN_CUDA(back);
+    pools[dev] = pool;
+  }
+  *out = pools[dev];
+  return HN_OK;
+}
+
 hn_status reduce(hn_dtype t, long long n, const void* x, const void* y, double* result, int root,
                  cudaStream_t s) {
   if (n == 0) {
@@ -188,7 +226,17 @@ hn_status reduce(hn_dtype t, long long n, const void* x, const void* y, double* 
   const long long m = (n + kChunk - 1) / kChunk;
   // chunk sums and the finishing ticket, stream-ordered
   void* scratch = nullptr;
-  HN_CUDA(cudaMallocAsync(&scratch, (size_t)m * sizeof(double) + 16, s));
+  const size_t bytes = (size_t)m * sizeof(double) + 16;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  const cudaError_t asked = cudaStreamIsCapturing(s, &capturing);
+  if (asked != cudaSuccess) cudaGetLastError();
+  if (asked != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {   // (a graph has memory of its own)
+    HN_CUDA(cudaMallocAsync(&scratch, bytes, s));
+  } else {
+    cudaMemPool_t pool = nullptr;
+    HN_TRY(scratch_pool(&pool));
+    HN_CUDA(cudaMallocFromPoolAsync(&scratch, bytes, pool, s));
+  }
   double* part = static_cast<double*>(scratch);
   unsigned* ticket = reinterpret_cast<unsigned*>(part + m);
   cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), s);

@@ -5,8 +5,8 @@
 // cudaMalloc at that point: code that runs while another thread captures a CUDA graph in global
 // mode (allocation is not permitted then), processes that hand out their whole device-memory plan
 // up front, and latency-critical paths where cudaMalloc / cudaFree would synchronize the device.
-// The only temporary, one partial sum of squares per 128-node tile, lives in the file-scope array
-// below, so the call allocates nothing: every GPU that loads the library holds the array (512 KiB)
+// The only temporary, one partial sum of squares per strip of tiles, lives in the file-scope array
+// below, so the call allocates nothing: every GPU that loads the library holds the array (29 KB)
 // until the process exits.
 #include <algorithm>
 #include <mutex>
@@ -16,13 +16,15 @@
 namespace hn {
 namespace {
 
-constexpr int kStaticTiles = 65536;                      // partial sums the array holds
-constexpr long long kStaticMaxNodes = (long long)kStaticTiles * kTile;   // 8,388,608 nodes
+constexpr long long kStaticMaxNodes = 65536LL * kTile;   // the largest operator: 8,388,608 nodes (level 11)
+// Strips of tiles, each with a partial sum in the array: three blocks of 8 warps on each of 152 SMs, also where the
+// chip has another number (the order of the sum is fixed).
+constexpr int kStrips = 3648;
 constexpr unsigned kFullMask = 0xffffffffu;
 
-// Scratch shared by every call on a device.  Each call writes slots [0, tiles) before reading
+// Scratch shared by every call on a device.  Each call writes its slots before reading
 // them, so nothing has to start at zero; calls that overlap on the GPU race on it.
-static __device__ __align__(256) double g_partials[kStaticTiles];
+static __device__ __align__(256) double g_partials[kStrips];
 
 // device address of g_partials, looked up once per device with that device current
 constexpr int kMaxDevices = 64;
@@ -73,20 +75,36 @@ __device__ __forceinline__ void row_window(const double* __restrict__ x, long lo
   }
 }
 
-// r = b - A x on 128-node warp-tiles of [0, N) (the last one ragged); slot t of the scratch gets
-// the tile's sum of r^2.  Bands are the operator's pitch-padded FP64 arrays.
-__global__ void __launch_bounds__(256) k_defect_static(BandPtrs64c band, int L, long long N,
-                                                       const double* __restrict__ x,
-                                                       const double* __restrict__ b,
-                                                       double* __restrict__ r, double* partials,
-                                                       int tiles) {
+// r = b - A x on 128-node warp-tiles of [0, N) (the last one ragged), as one chain from b.  Strip v of `strips` holds
+// the tiles v, v + strips, ..; slot v of the scratch gets its sum of r^2 (a lane adds its nodes in order, then the
+// lanes in a fixed tree).  Bands are the operator's pitch-padded FP64 arrays.
+//
+// Bound by the FP64 pipe (10 operations a node, 80 us at L = 11, where the bytes take 60): so the defect's subtraction
+// is part of the chain and the lanes add up once a strip, not once a tile (11 + 5/4 operations a node before).  With
+// the sum of 32,801 tiles by one block after it, L = 11 took 157 us, now 85; L = 10 43, now 29.
+__global__ void __launch_bounds__(256, 3) k_defect_static(BandPtrs64c band, int L, long long N,
+                                                          const double* __restrict__ x,
+                                                          const double* __restrict__ b,
+                                                          double* __restrict__ r, double* partials,
+                                                          int tiles, int strips) {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+  const int v = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (v >= strips) return;
   const long long shift = 1LL << L;
-  for (int t = gw; t < tiles; t += nw) {
+  double s = 0.0;
+  for (int t = v; t < tiles; t += strips) {
     const long long i0 = (long long)t * kTile + lane * kLaneNodes;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const bool whole = i0 + 3 < N;
+    double acc[4];
+    if (whole) {
+      const double2 p = __ldg(reinterpret_cast<const double2*>(b + i0));
+      const double2 q = __ldg(reinterpret_cast<const double2*>(b + i0) + 1);
+      acc[0] = p.x; acc[1] = p.y; acc[2] = q.x; acc[3] = q.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j] = i0 + j < N ? __ldg(b + i0 + j) : 0.0;
+    }
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy) {
       double w[8];
@@ -98,38 +116,48 @@ __global__ void __launch_bounds__(256) k_defect_static(BandPtrs64c band, int L, 
         const double2 q = __ldg(reinterpret_cast<const double2*>(band.p[k] + i0) + 1);
         const double bk[4] = {p.x, p.y, q.x, q.y};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j] = fma(bk[j], w[j + dy + dx + 2], acc[j]);
+        for (int j = 0; j < 4; ++j) acc[j] = fma(-bk[j], w[j + dy + dx + 2], acc[j]);
       }
     }
-    double s = 0.0;
+    if (whole) {
+      reinterpret_cast<double2*>(r + i0)[0] = make_double2(acc[0], acc[1]);
+      reinterpret_cast<double2*>(r + i0)[1] = make_double2(acc[2], acc[3]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long i = i0 + j;
-      if (i < N) {
-        const double ri = __ldg(b + i) - acc[j];
-        r[i] = ri;
-        s += ri * ri;
-      }
+      for (int j = 0; j < 4; ++j) s = fma(acc[j], acc[j], s);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i0 + j < N) {
+          r[i0 + j] = acc[j];
+          s = fma(acc[j], acc[j], s);
+        }
     }
-    s = warp_sum_d(s);
-    if (lane == 0) partials[t] = s;
   }
+  s = warp_sum_d(s);
+  if (lane == 0) partials[v] = s;
 }
 
-// ||r|| = sqrt of the tile sums added in a fixed order (one block): the result does not depend
-// on the grid of the first kernel
-__global__ void __launch_bounds__(256) k_sum_partials(const double* partials, int tiles,
+// ||r|| = sqrt of the strips' sums added in a fixed order (one block), its launch overlapping the first kernel's end
+__global__ void __launch_bounds__(256) k_sum_partials(const double* partials, int strips,
                                                       double* norm) {
   __shared__ double sh[8];
-  double t = 0.0;
-  for (int q = threadIdx.x; q < tiles; q += blockDim.x) t += partials[q];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  constexpr int kRounds = (kStrips + 255) / 256;
+  double v[kRounds], t = 0.0;
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) {
+    const int q = threadIdx.x + k * 256;
+    v[k] = q < strips ? __ldcg(partials + q) : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) t += v[k];
   t = warp_sum_d(t);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
   __syncthreads();
   if (threadIdx.x < 32) {
-    double v = threadIdx.x < 8 ? sh[threadIdx.x] : 0.0;
-    v = warp_sum_d(v);
-    if (threadIdx.x == 0) *norm = sqrt(v);
+    double u = threadIdx.x < 8 ? sh[threadIdx.x] : 0.0;
+    u = warp_sum_d(u);
+    if (threadIdx.x == 0) *norm = sqrt(u);
   }
 }
 
@@ -171,13 +199,19 @@ extern "C" hn_status hn_band_defect_norm_static(const hn_band* A, const double* 
   const int tiles = (int)((A->N + kTile - 1) / kTile);
   BandPtrs64c bp{};
   for (int k = 0; k < 9; ++k) bp.p[k] = A->band[k];
-  int sms = 0;
-  HN_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device));
-  const int grid = std::max(1, std::min((tiles + 7) / 8, std::max(sms, 1) * 4));
+  const int strips = std::min(tiles, kStrips);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_defect_static<<<grid, 256, 0, s>>>(bp, A->L, A->N, x, b, r, scratch, tiles);
+  k_defect_static<<<(strips + 7) / 8, 256, 0, s>>>(bp, A->L, A->N, x, b, r, scratch, tiles, strips);
   HN_CUDA(cudaGetLastError());
-  k_sum_partials<<<1, 256, 0, s>>>(scratch, tiles, norm);
-  HN_CUDA(cudaGetLastError());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute overlap;
+  overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  overlap.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &overlap;
+  cfg.numAttrs = 1;
+  HN_CUDA(cudaLaunchKernelEx(&cfg, k_sum_partials, static_cast<const double*>(scratch), strips, norm));
   return HN_OK;
 }
