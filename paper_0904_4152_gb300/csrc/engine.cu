@@ -923,6 +923,13 @@ bool Engine::span_tail() const {
          !tune_.staged && !tune_.fuse_up && tune_.cluster == 16 && cap_ == 1 && std::min(T, Lmax_) > kSmallTop && T <= kSpanTop;
 }
 
+// An FP64 problem alone: level l's steps as launches of k_level64 (which has the measurements).
+constexpr int kLevel64Min = 9;
+bool Engine::level64(int l) const {
+  return tune_.march && tune_.sweep == 1 && cap_ == 1 && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
+         mid_top() <= std::max(tune_.tail_level, prm_.coarse) && l >= kLevel64Min;
+}
+
 // The FP64 counterpart over a cluster of 16 blocks (k_wide).
 bool Engine::wide_tail() const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
@@ -969,7 +976,7 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
       }
       continue;
     }
-    if (sweep_level(l) && !top) {
+    if (sweep_level(l) && !top && !level64(l)) {
       // a zero iterate: both smoothing steps, the defect and the restriction in one launch
       HN_LAUNCH(KC_SWEEP_DOWN, l, launch_sweep_down(E_, lists_[l], l, want, 0, s));
       continue;
@@ -977,6 +984,17 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
     // an engine of one problem takes the check inside the first smoothing step when the norm is
     // one group of partials (the register-path kernel; saves the control launch)
     const bool fuse = top && cap_ == 1 && !tune_.staged && pitch_of(l) / kTile <= kSumGroup;
+    if (level64(l)) {
+      HN_LAUNCH(KC_JACOBI_FIRST, l, launch_level64(E_, lists_[l], 0, l, want, 0, fuse ? 1 : 0, s));
+      if (top) {
+        if (!fuse) HN_LAUNCH(KC_CONTROL, l, launch_control(E_, CTRL_PRE, s, l));
+        HN_TRY(after_check());
+      }
+      HN_LAUNCH(KC_JACOBI, l, launch_level64(E_, lists_[l], 1, l, want, 1, 0, s));
+      HN_LAUNCH(KC_DEFECT, l, launch_level64(E_, lists_[l], 2, l, want, 0, 0, s));
+      HN_LAUNCH(KC_RESTRICT, l, launch_restrict(E_, lists_[l - 1], l, want, grid_[l - 1], s));
+      continue;
+    }
     if (pre >= 2) {
       HN_LAUNCH(KC_JACOBI_FIRST, l, launch_pre12(E_, lists_[l], l, want, grid_[l], s, fuse ? 1 : 0));
       if (top) {
@@ -1016,7 +1034,7 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
       e_sel = 0;
       continue;
     }
-    if (sweep_level(l) && !is_top(l)) {
+    if (sweep_level(l) && !is_top(l) && !level64(l)) {
       // prolongation and both post-smoothing steps in one launch; the result in buffer 1 (a
       // problem's own finest level keeps its iterate in buffer 0)
       HN_LAUNCH(KC_SWEEP_UP, l, launch_sweep_up(E_, lists_[l], l, want, e_sel, s));
@@ -1032,6 +1050,11 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
       HN_LAUNCH(KC_PROLONG, l, launch_prolong(E_, lists_[l], l, want, (pre & 1) | (e_sel << 1), grid_[l], s));
     }
     e_sel = 0;
+    if (level64(l)) {
+      HN_LAUNCH(KC_JACOBI, l, launch_level64(E_, lists_[l], 1, l, want, 0, 0, s));
+      HN_LAUNCH(KC_JACOBI, l, launch_level64(E_, lists_[l], 1, l, want, 1, 0, s));
+      continue;
+    }
     for (; sw <= post; ++sw)
       HN_LAUNCH(KC_JACOBI, l, launch_jacobi(E_, lists_[l], l, want, (pre + sw - 1) & 1, 0, grid_[l], s));
   }

@@ -290,6 +290,7 @@ class Engine {
   bool sweep_on() const;            // the fused level sweeps run (tuning sweep, and they apply)
   bool sweep_level(int l) const;    // level l's down / up parts run as fused sweeps
   bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
+  bool level64(int l) const;        // level l's steps run as launches of k_level64
   bool wide_tail() const;           // the FP64 tail of a cluster of 16 blocks (k_wide)
   bool span_tail() const;           // the FP32 / FP16 tail of a cluster of 16 blocks (k_span)
   bool small_tail() const;          // the tail runs in one block's shared memory (k_small)

@@ -251,6 +251,11 @@ cudaError_t launch_wide(const EngineDev& E, int T, int want, int loop, cudaStrea
 // the same on levels coarse..T <= kSpanTop of FP32 / FP16 hierarchies (k_span.cu); finest levels above 5 only
 constexpr int kSpanTop = 8;
 cudaError_t launch_span(const EngineDev& E, int T, int want, int loop, cudaStream_t s);
+// One step of FP64 level `level` of a problem solved alone (k_fine.cu): 0: the first smoothing step (buffer 0 to 1; on the
+// finest level, from a nonzero iterate, with the norm partials and, fuse, the lagged check), 1: a smoothing
+// step from buffer in_sel to the other, 2: the defect of buffer in_sel.
+cudaError_t launch_level64(const EngineDev& E, const TileList& tl, int kind, int level, int want, int in_sel, int fuse,
+                           cudaStream_t s);
 // The start and the end of a solve (k_io.cu).  b: right-hand side to copy in (or null: it is in place); x: at the start
 // the given iterate to copy in (or null: clear: start from zeros, else it is in place), at the end where the result
 // goes (or null).  Device vectors, 16-byte aligned.  first: reset / read the engine's counters too.

@@ -391,7 +391,96 @@ cudaError_t launch_fine_p(const EngineDev& E, int solo_tiles, int summary, cudaG
                            : launch_fine_t<OP, float>(E, solo_tiles, summary, h, use_handle, s);
 }
 
+// A smoothing step or the defect of an FP64 level of a problem solved alone (k_band's step, same bits).  Bound by the
+// FP64 pipe (10 operations a node, 20 us at L = 10) once the vectors come from L2: there the level and those below
+// it (157 MB) are more than L2 holds, so from level 10 on the bands are marked to be evicted first and the
+// vectors, which every step reads or writes, stay (solve at L = 10 2421 -> 2257 us, with all bands kept 2325 us;
+// L = 11 6180 -> 5993).  Level 9 below them the same way, against fused sweeps of recomputed halos, which cost the
+// FP64 pipe more than the launches saved: L = 10 2257 -> 2202 us, L = 11 5993 -> 5907; level 8 too is slower
+// (2430 against 2350 us, bands kept).  Two, three, four blocks an SM: 2518 / 2432 / 2475 us (bands kept).
+enum { LV_FIRST = 0, LV_SMOOTH, LV_DEFECT };
+template <int OP, int LKB>
+__global__ void __launch_bounds__(kFineThreads, 3)
+    k_level64(EngineDev E, TileList tl, int level, int want, int in_sel, int fuse) {
+  pdl_start();
+  if (tl.solo_d.n == 0) return;
+  const ProbState& st = E.S[0];
+  if (st.phase != want) return;
+  if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
+  const LevelDev& d = tl.solo_d;
+  const bool zero = OP == LV_FIRST && (tl.solo_L > level || st.zero_top);
+  const bool summed = OP == LV_FIRST && tl.solo_L == level && !zero;
+  const int lane = threadIdx.x & 31, src = OP == LV_FIRST ? 0 : in_sel;
+  const double* x = static_cast<const double*>(d.x[src]);
+  double* out = static_cast<double*>(OP == LV_DEFECT ? d.r : d.x[1 - src]);
+  const int step = (int)gridDim.x * kFineWarps;
+  for (int t = (int)blockIdx.x * kFineWarps + (int)(threadIdx.x >> 5); t < tl.solo_tiles; t += step) {
+    const long long i0 = (long long)t * kTile + lane * kLaneNodes;
+    double r[4], v[4];
+    ld4<LD_NC>(static_cast<const double*>(d.rhs) + i0, r);
+    if (zero) {
+      double wd[4];
+      ld4<LKB>(d.wdinv + i0, wd);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = wd[j] * r[j];
+    } else {
+      double w[3][8], dg[4];
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) load_row<double, LD_NC>(x, i0 + dy * (1LL << level), lane, w[dy + 1]);
+      stencil_windows<F64, LKB, true>(d.band, nullptr, w, i0, r, dg);
+      if constexpr (OP == LV_DEFECT) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = r[j];
+      } else {
+        double wd[4];
+        ld4<LKB>(d.wdinv + i0, wd);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = fma(wd[j], r[j], w[1][j + 2]);
+      }
+    }
+    st4(out + i0, v);
+    if (summed) {
+      const double q = tile_sumsq(r);
+      if (lane == 0) E.partial[t] = q;
+    }
+  }
+  if (OP == LV_FIRST && fuse) solo_fused_check(E, level, summed, want);
+}
+
+template <int OP, int LKB>
+cudaError_t launch_level64_t(const EngineDev& E, const TileList& tl, int level, int want, int in_sel, int fuse,
+                             cudaStream_t s) {
+  auto kern = k_level64<OP, LKB>;
+  static const int per_sm = [&] {
+    int b = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kFineThreads, 0) == cudaSuccess && b > 0 ? b : 1;
+  }();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)std::max(1, std::min(per_sm * sm_count(), (tl.solo_tiles + kFineWarps - 1) / kFineWarps)), 1, 1);
+  cfg.blockDim = dim3((unsigned)kFineThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  if (E.pdl == 1 || (E.pdl && (int)cfg.gridDim.x < (E.pdl == 3 ? 2 : 1) * sm_count())) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, kern, E, tl, level, want, in_sel, fuse);
+}
+
 }  // namespace
+
+cudaError_t launch_level64(const EngineDev& E, const TileList& tl, int kind, int level, int want, int in_sel, int fuse,
+                           cudaStream_t s) {
+  const bool stream = level >= 10;
+  if (kind == LV_FIRST) return stream ? launch_level64_t<LV_FIRST, LD_EF>(E, tl, level, want, in_sel, fuse, s)
+                                      : launch_level64_t<LV_FIRST, LD_NC>(E, tl, level, want, in_sel, fuse, s);
+  if (kind == LV_SMOOTH) return stream ? launch_level64_t<LV_SMOOTH, LD_EF>(E, tl, level, want, in_sel, fuse, s)
+                                       : launch_level64_t<LV_SMOOTH, LD_NC>(E, tl, level, want, in_sel, fuse, s);
+  return stream ? launch_level64_t<LV_DEFECT, LD_EF>(E, tl, level, want, in_sel, fuse, s)
+                : launch_level64_t<LV_DEFECT, LD_NC>(E, tl, level, want, in_sel, fuse, s);
+}
 
 cudaError_t launch_fine(const EngineDev& E, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                         int use_handle, cudaStream_t s) {

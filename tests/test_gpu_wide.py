@@ -1,5 +1,5 @@
 """The tails over a cluster of 16 blocks (FP64: levels to 6; FP32 / FP16 alone: to 8; the lagged check and, for a
-problem whose finest level is in it, all cycles in one launch) against the general tail: the same bits, for each top
+problem whose finest level is in it, all cycles in one launch) and the FP64 steps on finer levels against the general tail: the same bits, for each top
 level, coarsest level, boundary mask, zero and given iterates (nonzero on Dirichlet nodes too), CG, a cycle limit
 and batches."""
 import numpy as np
@@ -28,7 +28,7 @@ def outcome(hn, mg, L, b, guess=None):
 @pytest.mark.parametrize("solver", [0, 1])
 @pytest.mark.parametrize("prec,L,coarse,bc", [
     (0, 2, 2, 15), (0, 3, 2, 7), (0, 3, 3, 15), (0, 4, 2, 15), (0, 4, 3, 10), (0, 4, 4, 1), (0, 5, 2, 15), (0, 5, 4, 5),
-    (0, 5, 3, 8), (0, 6, 2, 15), (0, 6, 3, 4), (0, 6, 4, 2), (0, 6, 2, 1), (0, 7, 2, 15), (0, 8, 3, 11),
+    (0, 5, 3, 8), (0, 6, 2, 15), (0, 6, 3, 4), (0, 6, 4, 2), (0, 6, 2, 1), (0, 7, 2, 15), (0, 8, 3, 11), (0, 9, 2, 6), (0, 10, 2, 15),
     (1, 4, 2, 15), (1, 6, 2, 15), (1, 6, 3, 4), (2, 6, 4, 2), (1, 7, 4, 10), (2, 7, 2, 15), (1, 8, 2, 15), (2, 8, 3, 11),
     (1, 8, 4, 5), (1, 8, 2, 8), (2, 8, 2, 1), (1, 9, 2, 15), (2, 10, 3, 2)])
 def test_cluster_tails_give_the_bits_of_the_general_tail(hn, prec, L, coarse, bc, solver):
