@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "hn_internal.h"
+#include "k_convert.cuh"
 
 namespace hn {
 

@@ -91,7 +91,7 @@ __device__ __forceinline__ double fine_tile(const ProblemDev& P, ProbState& st, 
     const double s = st.s;
     V out[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) out[j] = V(r[j] * s);
+    for (int j = 0; j < 4; ++j) out[j] = from_f64<V>(r[j] * s);
     q = lane_norm(r);
     st4(static_cast<V*>(top.rhs) + i0, out);
     if (pcg) st4(P.r64 + i0, r);
@@ -103,7 +103,7 @@ __device__ __forceinline__ double fine_tile(const ProblemDev& P, ProbState& st, 
     ld4c(P.x64 + i0, x);
     const double inv_s = st.inv_s;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = fma(double(c[j]), inv_s, x[j]);
+    for (int j = 0; j < 4; ++j) x[j] = fma(to_f64(c[j]), inv_s, x[j]);
     st4(P.x64 + i0, x);
   } else if constexpr (OP == F_PCG_Q) {
     // q = A p (p with zero halos) and (p, q)
@@ -128,7 +128,7 @@ __device__ __forceinline__ double fine_tile(const ProblemDev& P, ProbState& st, 
       x[j] = fma(alpha, pv[j], x[j]);
       r[j] = fma(-alpha, qv[j], r[j]);
       q = fma(r[j], r[j], q);
-      out[j] = V(r[j] * s);
+      out[j] = from_f64<V>(r[j] * s);
     }
     st4(P.x64 + i0, x);
     st4(P.r64 + i0, r);
@@ -140,7 +140,7 @@ __device__ __forceinline__ double fine_tile(const ProblemDev& P, ProbState& st, 
     ld4<LD_NC>(P.r64 + i0, r);
     ld4<LD_NC>(static_cast<const V*>(top.x[0]) + i0, c);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) q = fma(r[j], double(c[j]), q);
+    for (int j = 0; j < 4; ++j) q = fma(r[j], to_f64(c[j]), q);
   } else {
     // p = c / s + beta p (the new search direction)
     V c[4];
@@ -149,7 +149,7 @@ __device__ __forceinline__ double fine_tile(const ProblemDev& P, ProbState& st, 
     ld4c(P.p64 + i0, pv);
     const double beta = st.beta, inv_s = st.inv_s;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) pv[j] = fma(beta, pv[j], double(c[j]) * inv_s);
+    for (int j = 0; j < 4; ++j) pv[j] = fma(beta, pv[j], to_f64(c[j]) * inv_s);
     st4(P.p64 + i0, pv);
   }
   return q;
