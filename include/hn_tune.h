@@ -12,8 +12,11 @@
  *
  * A hierarchy whose shape was not set by hn_mg_set_tuning (the default, or an autotuned shape with
  * sweep 1 and mid 0) runs the larger levels of an FP32 / FP16 V(2,2) cycle, alone, in batches and in the
- * server, as marching sweeps: one pass over the level each way.  hn_mg_set_tuning selects exactly
- * the forms described below.
+ * server, as marching sweeps: one pass over the level each way, above a one-block tail (tail_level <= 5);
+ * problems of level 6..8 alone run their inner solves in one launch of 16 blocks.  FP64 V(2,2) cycles alone
+ * and in batches of up to 31 run the levels to tail_level (5 or 6, cluster 16) so, with all cycles in one launch
+ * where the finest level is among them, and those from 9 as one launch per step.  hn_mg_set_tuning selects
+ * exactly the forms described below.
  */
 #ifndef HN_TUNE_H
 #define HN_TUNE_H

@@ -63,14 +63,10 @@ constexpr int kMidCandidate = 10;
 // fused tail pays from level 6 down (its levels then fit in distributed shared memory); the
 // FP32/FP16 inner cycles fuse from level 5 down (block 0's shared memory alone), the levels
 // above it up to 9 running as fused sweeps (autotuned at L = 10: 1.537 ms against >= 1.576 ms
-// with the tail from level 7).  A problem of L = 6..8 that k_span serves runs its whole inner solves in
-// one launch each: L = 7 715 -> 415 us, L = 8 796 -> 613 us; as the tail of a larger one, which comes back
-// every cycle, its launch takes longer than the sweeps and the one-block tail (L = 9 968 against 1052 us, L = 10 1394
-// against 1494 us; from level 7 967 / 1435, from level 6 964 / 1407 us).
-Tuning default_tuning(const Params& prm, int L) {
+// with the tail from level 7)
+Tuning default_tuning(const Params& prm) {
   Tuning t;
-  const bool span = L <= kSpanTop && prm.pre == 2 && prm.post == 2 && !prm.coarse_cg;
-  t.tail_level = prm.prec == P64 ? 6 : span ? kSpanTop : 5;
+  t.tail_level = prm.prec == P64 ? 6 : 5;
   return t;
 }
 
@@ -82,7 +78,7 @@ hn_status ensure_solo(hn_mg* mg) {
   std::unique_ptr<Engine> e(new Engine());
   HN_TRY(e->create(mg->prm, 1, mg->L, caps, fine, mg->stream));
   HN_TRY(e->set_members({mg}));
-  e->set_tuning(mg->tuned ? mg->tuning : default_tuning(mg->prm, mg->L));
+  e->set_tuning(mg->tuned ? mg->tuning : default_tuning(mg->prm));
   mg->solo = e.release();
   return HN_OK;
 }
@@ -539,7 +535,7 @@ hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t) { return set_shape(mg,
 hn_status hn_mg_get_tuning(const hn_mg* mg, hn_tuning* t) {
   clear_error();
   if (!mg || !t) return set_error(HN_ERR_ARG, "null argument");
-  const Tuning tu = mg->solo ? mg->solo->tuning() : (mg->tuned ? mg->tuning : default_tuning(mg->prm, mg->L));
+  const Tuning tu = mg->solo ? mg->solo->tuning() : (mg->tuned ? mg->tuning : default_tuning(mg->prm));
   t->tail_level = tu.tail_level;
   t->cluster = tu.cluster;
   t->pdl = tu.pdl;

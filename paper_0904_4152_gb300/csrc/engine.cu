@@ -750,7 +750,7 @@ long long Engine::launch_bytes(int cls, int level) const {
     case KC_JACOBI: per = 9 * bb + 3 * vb + wd; break;
     case KC_JACOBI_FIRST: per = 9 * bb + 2 * vb + (prec == P64 ? 8 : 4); break;   // fused from x = 0
     case KC_DEFECT: per = 9 * bb + 3 * vb; break;
-    case KC_CHECK: per = 9 * bb + 2 * vb; break;
+    case KC_CHECK: per = level > 0 && march_level(level) ? 2 : 9 * bb + 2 * vb; break;   // (a march's squares)
     case KC_RESTRICT: per = 1.25 * vb; break;                   // per fine node
     case KC_PROLONG: per = 2.25 * vb; break;                    // per fine node
     case KC_PROLONG_JACOBI: per = 9 * bb + 3.25 * vb + wd; break; // Jacobi + coarse reads
@@ -767,15 +767,15 @@ long long Engine::launch_bytes(int cls, int level) const {
       for (hn_mg* mg : members_) {
         if (!mg || level > mg->L || level <= mg->coarse) continue;
         const bool own = level == mg->L && prm_.solver != SOLVER_PCG;
-        // (a marching sweep also reads omega / D from a nonzero iterate)
+        // (a marching sweep reads five bands, and omega / D from a nonzero iterate too)
         const double wdm = march_level(level) ? 4 : wd;
-        const double pn = 9 * bb + vb + (own ? vb + wdm : (prec == P64 ? 8 : 4)) + vb + 0.25 * vb;
+        const double pn = (march_level(level) ? 5 : 9) * bb + vb + (own ? vb + wdm : (prec == P64 ? 8 : 4)) + vb + 0.25 * vb;
         sum += (long long)(pn * (double)N_of(level));
       }
       return sum;
     }
     case KC_SWEEP_UP:                                          // bands, x, e_c, rhs; write
-      per = 9 * bb + vb + 0.25 * vb + vb + (march_level(level) ? 4 : wd) + vb;
+      per = (march_level(level) ? 5 : 9) * bb + vb + 0.25 * vb + vb + (march_level(level) ? 4 : wd) + vb;
       break;
     case KC_MID_DOWN:
     case KC_MID_UP: {
@@ -913,15 +913,22 @@ bool Engine::march_level(int l) const {
 // conditions of the marching sweeps and with the exact coarse solver.
 bool Engine::small_tail() const {
   return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
-         !tune_.staged && !tune_.fuse_up && std::min(std::max(tune_.tail_level, prm_.coarse), cap_ == 1 ? Lmax_ : kMaxLevel) <= kSmallTop;
+         !tune_.staged && !tune_.fuse_up && std::max(tune_.tail_level, prm_.coarse) <= kSmallTop;
 }
 
-// An FP32 / FP16 problem alone: the tail over a cluster of 16 blocks (k_span).
+// An FP32 / FP16 problem of L = 6..8 alone whose shape would have the one-block tail: its whole inner solves in one launch
+// each (k_span).  L = 7 715 -> 415 us, L = 8 796 -> 613 us.  As the tail of a larger problem, which comes back every
+// cycle, its launch takes longer than the sweeps and the one-block tail: L = 9 968 against 1052 us, L = 10 1394
+// against 1494 us (from level 7 967 / 1435, from level 6 964 / 1407 us).
 bool Engine::span_tail() const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
   return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
-         !tune_.staged && !tune_.fuse_up && tune_.cluster == 16 && cap_ == 1 && std::min(T, Lmax_) > kSmallTop && T <= kSpanTop;
+         !tune_.staged && !tune_.fuse_up && tune_.mid <= T && T <= kSmallTop && small_.L == Lmax_ &&
+         Lmax_ > kSmallTop && Lmax_ <= kSpanTop;   // (small_: an engine of one problem; a server's may be of a lower level)
 }
+
+// the highest level of the fused tail
+int Engine::tail_top() const { return span_tail() ? kSpanTop : std::max(tune_.tail_level, prm_.coarse); }
 
 // An FP64 problem alone: level l's steps as launches of k_level64 (which has the measurements).
 constexpr int kLevel64Min = 9;
@@ -939,7 +946,7 @@ bool Engine::wide_tail() const {
 
 hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   const int c = prm_.coarse, pre = prm_.pre, post = prm_.post;
-  const int T = std::max(tune_.tail_level, c);
+  const int T = tail_top();
   cudaStream_t s = s0;
   bool opened = false;
   int c0 = 0;
@@ -1021,8 +1028,8 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
     HN_LAUNCH(KC_RESTRICT, l, launch_restrict(E_, lists_[l - 1], l, want, grid_[l - 1], s));
   }
   if (M > T) HN_LAUNCH(KC_MID_DOWN, M, launch_mid(E_, dLists_, M, T, want, 0, s));
-  if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, std::min(T, kSmallTop), want, s));
-  else if (span_tail()) HN_LAUNCH(KC_TAIL, T, launch_span(E_, T, want, Lmax_ <= T, s));
+  if (span_tail()) HN_LAUNCH(KC_TAIL, T, launch_span(E_, T, want, 1, s));
+  else if (small_tail()) HN_LAUNCH(KC_TAIL, T, launch_small(E_, small_, T, want, s));
   else if (wide_tail()) HN_LAUNCH(KC_TAIL, T, launch_wide(E_, T, want, Lmax_ <= T, s));
   else HN_LAUNCH(KC_TAIL, T, launch_tail(E_, T, want, tune_.cluster, s));
   if (M > T) HN_LAUNCH(KC_MID_UP, M, launch_mid(E_, dLists_, M, T, want, 1, s));
@@ -1192,7 +1199,7 @@ hn_status Engine::capture_solve(bool cond) {
     // taken), so only the rest of a V cycle after the lagged check gets one, and only in the
     // defect correction, where every outer step ends with one cycle that its check stops.  (The
     // outer defect and the update would each skip two small launches: not worth an IF node.)
-    const int T = std::max(std::max(tune_.tail_level, prm_.coarse), mid_top());
+    const int T = std::max(tail_top(), mid_top());
     if (Lmax_ > T && prm_.prec != P64 && prm_.solver != SOLVER_PCG) cd.mask |= 1u;
     const unsigned defaults[3] = {0u, 1u, 0u};
     // two sets: the loop body holds two iterations, each with IF nodes of its own handles

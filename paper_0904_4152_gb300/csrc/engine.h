@@ -292,7 +292,8 @@ class Engine {
   bool march_level(int l) const;    // level l's down / up parts run as marching sweeps
   bool level64(int l) const;        // level l's steps run as launches of k_level64
   bool wide_tail() const;           // the FP64 tail of a cluster of 16 blocks (k_wide)
-  bool span_tail() const;           // the FP32 / FP16 tail of a cluster of 16 blocks (k_span)
+  bool span_tail() const;           // a small FP32 / FP16 problem's inner solves by a cluster of 16 blocks (k_span)
+  int tail_top() const;             // the highest level of the fused tail
   bool small_tail() const;          // the tail runs in one block's shared memory (k_small)
   SmallSolo small_{};               // its descriptors, for an engine of one problem
   // level l may be a member's own finest level (the server's engines: any level)

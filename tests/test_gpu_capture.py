@@ -1,4 +1,5 @@
-"""Reductions in a captured graph, and on several streams and threads at once: each call's scratch is its own."""
+"""Reductions and the defect with norm in a captured graph, reductions on several streams and threads at
+once: each call's scratch is its own."""
 import threading
 
 import numpy as np
@@ -31,6 +32,21 @@ def test_reductions_captured_and_side_by_side(hn, n):
         graph.replay()
         torch.cuda.synchronize()
         assert float(out[0, 0]) == want and float(out[1, 0]) == np.sqrt(want)
+    A = hn.hn_band_create(6)
+    try:
+        b = torch.ones(hn.hn_band_nodes(A), device="cuda", dtype=torch.float64)
+        r, norm, again = torch.zeros_like(b), out.new_zeros(1), out.new_zeros(1)
+        hn.hn_band_defect_norm_static(A, x.new_zeros(b.numel()), b, r, norm)
+        graph = torch.cuda.CUDAGraph()
+        zeros = torch.zeros_like(b)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            hn.hn_band_defect_norm_static(A, zeros, b, r, again, stream)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert float(norm) == float(again) == np.sqrt(b.numel()) and torch.equal(r, b)      # x = 0: r = b
+    finally:
+        hn.hn_band_destroy(A)
     got = {}
 
     def work(k):

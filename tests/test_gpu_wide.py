@@ -1,7 +1,7 @@
-"""The tails over a cluster of 16 blocks (FP64: levels to 6; FP32 / FP16 alone: to 8; the lagged check and, for a
-problem whose finest level is in it, all cycles in one launch) and the FP64 steps on finer levels against the general tail: the same bits, for each top
-level, coarsest level, boundary mask, zero and given iterates (nonzero on Dirichlet nodes too), CG, a cycle limit
-and batches."""
+"""The tails over a cluster of 16 blocks (FP64: levels to 6; FP32 / FP16 alone: to 8; the lagged check and,
+for a problem whose finest level is in it, all cycles in one launch) and the FP64 steps on finer levels
+against the general kernels: the same bits, for each top level, coarsest level, boundary mask, zero and
+given iterates (nonzero on Dirichlet nodes too), CG, a cycle limit and batches."""
 import numpy as np
 import pytest
 
