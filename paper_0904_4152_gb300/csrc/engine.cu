@@ -89,7 +89,8 @@ struct LevelLayout {
   long long pitch, halo;
 };
 
-size_t vec_elems(int l) { return (size_t)(pitch_of(l) + 2 * halo_of(l)); }
+// elements of an array of level l of a hierarchy of precision prec (the FP64 vectors beside it: P64)
+size_t vec_elems(int l, int prec) { return (size_t)(pitch_of(l) + 2 * halo_of(l, prec)); }
 
 template <class F>
 void walk_layout(int L, int coarse, int prec, int solver, F&& take) {
@@ -97,20 +98,20 @@ void walk_layout(int L, int coarse, int prec, int solver, F&& take) {
   const size_t vs = prec == P64 ? 8 : 4;
   const size_t bs = prec == P64 ? 8 : (prec == P32 ? 4 : 2);
   for (int l = L; l >= coarse; --l) {
-    for (int v = 0; v < 4; ++v) take(vec_elems(l) * vs);
-    for (int k = 0; k < 9; ++k) take(vec_elems(l) * bs);
-    take(vec_elems(l) * (prec == P64 ? 8 : 4));    // omega / diag
+    for (int v = 0; v < 4; ++v) take(vec_elems(l, prec) * vs);
+    for (int k = 0; k < 9; ++k) take(vec_elems(l, prec) * bs);
+    take(vec_elems(l, prec) * (prec == P64 ? 8 : 4));    // omega / diag
   }
   if (prec != P64) {
-    for (int k = 0; k < 9; ++k) take(vec_elems(L) * 8);
-    take(vec_elems(L) * 8);
-    take(vec_elems(L) * 8);
+    for (int k = 0; k < 9; ++k) take(vec_elems(L, P64) * 8);
+    take(vec_elems(L, P64) * 8);
+    take(vec_elems(L, P64) * 8);
   } else if (solver == SOLVER_PCG) {               // x, b apart from the cycle's vectors
-    take(vec_elems(L) * 8);
-    take(vec_elems(L) * 8);
+    take(vec_elems(L, P64) * 8);
+    take(vec_elems(L, P64) * 8);
   }
   if (solver == SOLVER_PCG)
-    for (int v = 0; v < 3; ++v) take(vec_elems(L) * 8);   // r, p, q
+    for (int v = 0; v < 3; ++v) take(vec_elems(L, P64) * 8);   // r, p, q
   const long long m = n_of(coarse) * n_of(coarse);   // unknowns of the coarsest level, at most
   take((size_t)(m * m) * 8);
 }
@@ -308,10 +309,10 @@ hn_status build_hierarchy(const hn_band* A, const hn_mg_opts& o, cudaStream_t s,
     d.n = (int)n_of(l);
     d.pitch = (int)pitch_of(l);
     d.bc = (int)A->bc;
-    const long long H = halo_of(l);
+    const long long H = halo_of(l, prec);
     void* vecs[4];
     for (int v = 0; v < 4; ++v) {
-      char* base = b.take<char>(vec_elems(l) * vsz);
+      char* base = b.take<char>(vec_elems(l, prec) * vsz);
       vecs[v] = base + H * vsz;
     }
     d.x[0] = vecs[0];
@@ -319,32 +320,32 @@ hn_status build_hierarchy(const hn_band* A, const hn_mg_opts& o, cudaStream_t s,
     d.rhs = vecs[2];
     d.r = vecs[3];
     for (int k = 0; k < 9; ++k) {
-      if (prec == P64) d.band[k] = b.take<double>(vec_elems(l)) + H;
-      else if (prec == P32) d.band[k] = b.take<float>(vec_elems(l)) + H;
-      else d.band[k] = b.take<__half>(vec_elems(l)) + H;
+      if (prec == P64) d.band[k] = b.take<double>(vec_elems(l, prec)) + H;
+      else if (prec == P32) d.band[k] = b.take<float>(vec_elems(l, prec)) + H;
+      else d.band[k] = b.take<__half>(vec_elems(l, prec)) + H;
     }
     for (int k = 0; k < 9; ++k) d.scale[k] = 1.0f;
-    if (prec == P64) d.wdinv = b.take<double>(vec_elems(l)) + H;
-    else d.wdf = b.take<float>(vec_elems(l)) + H;
+    if (prec == P64) d.wdinv = b.take<double>(vec_elems(l, prec)) + H;
+    else d.wdf = b.take<float>(vec_elems(l, prec)) + H;
   }
   if (prec != P64) {
-    for (int k = 0; k < 9; ++k) P.band64[k] = b.take<double>(vec_elems(L)) + halo_of(L);
-    P.x64 = b.take<double>(vec_elems(L)) + halo_of(L);
-    P.b64 = b.take<double>(vec_elems(L)) + halo_of(L);
+    for (int k = 0; k < 9; ++k) P.band64[k] = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
+    P.x64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
+    P.b64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
   } else {
     for (int k = 0; k < 9; ++k) P.band64[k] = static_cast<const double*>(P.lev[L].band[k]);
     if (prm.solver == SOLVER_PCG) {   // the cycle's top vectors are the preconditioner's
-      P.x64 = b.take<double>(vec_elems(L)) + halo_of(L);
-      P.b64 = b.take<double>(vec_elems(L)) + halo_of(L);
+      P.x64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
+      P.b64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
     } else {
       P.x64 = static_cast<double*>(P.lev[L].x[0]);
       P.b64 = static_cast<double*>(P.lev[L].rhs);
     }
   }
   if (prm.solver == SOLVER_PCG) {
-    P.r64 = b.take<double>(vec_elems(L)) + halo_of(L);
-    P.p64 = b.take<double>(vec_elems(L)) + halo_of(L);
-    P.q64 = b.take<double>(vec_elems(L)) + halo_of(L);
+    P.r64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
+    P.p64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
+    P.q64 = b.take<double>(vec_elems(L, P64)) + halo_of(L, P64);
   }
   // the coarse inverse (m x m), or for the CG coarse solver the 9 coarse bands (9 N_c); the
   // layout reserves (N_c)^2 >= both

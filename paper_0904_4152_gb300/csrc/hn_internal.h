@@ -26,12 +26,16 @@ inline long long N_of(int L) { return n_of(L) * n_of(L); }
 inline long long round_up(long long v, long long m) { return (v + m - 1) / m * m; }
 // padded length of a level: multiple of the tile, and every row/tile index is in range
 inline long long pitch_of(int L) { return round_up(N_of(L), kTile); }
-// zero halo in front of / behind every vector: covers the +-(n+1) stencil reach of the padded range
-// and the rows that a marching sweep reads around it (up to five rows of 2^L and 8 columns); a
-// multiple of 32 elements keeps every vector 256-byte aligned
-inline long long halo_of(int L) { return round_up(5 * n_of(L) + 16, 32); }
-
 enum Prec { P64 = 0, P32 = 1, P16 = 2 };
+// smallest level in marching sweeps (k_march.cu)
+constexpr int kMarchMinLevel = 6;
+// zero halo in front of / behind every vector: covers the +-(n+1) stencil reach of the padded range
+// and, on the FP32 / FP16 levels in marching sweeps, the rows that these read around it (up to five rows
+// of 2^L and 8 columns; a level's coarse neighbour is read on its grid only); a multiple of 32 elements
+// keeps every vector 256-byte aligned
+inline long long halo_of(int L, int prec) {
+  return round_up(prec != P64 && L >= kMarchMinLevel ? 5 * n_of(L) + 16 : n_of(L) + 8, 32);
+}
 enum Solver { SOLVER_MG = 0, SOLVER_PCG = 1 };
 
 // unpreconditioned CG on the coarsest level: stop at ||r|| <= kCoarseCgTol ||b|| or after
@@ -41,7 +45,7 @@ __host__ __device__ inline int coarse_cg_steps(int m) { return 2 * m + 10; }
 
 // ------------------------------------------------------------------- device descriptors
 // One level of one problem.  Vectors and bands point at element 0 of pitch elements; a zero halo
-// of halo_of(L) elements sits on either side of every array, so stencil windows of any padded row
+// of halo_of elements sits on either side of every array, so stencil windows of any padded row
 // stay inside the allocation.
 struct LevelDev {
   const void* band[9];   // double (FP64 hierarchy), float (FP32), __half (FP16 codes)
@@ -297,7 +301,6 @@ cudaError_t launch_sweep_up(const EngineDev& E, TileList tl, int level, int want
 // one problem; launch_march_group: of all problems that have a finer level, or (level 0) every problem's
 // own finest level above T.  launch_march_check / _group: the lagged check after the down part of the
 // finest level.
-constexpr int kMarchMinLevel = 6;
 constexpr int kMarchSoloLevel = 9;   // an engine of one problem: from here
 cudaError_t launch_march(const EngineDev& E, const TileList& tl, int level, int want, int up, int e_sel, cudaStream_t s);
 cudaError_t launch_march_group(const EngineDev& E, int level, int T, int want, int up, cudaStream_t s);
