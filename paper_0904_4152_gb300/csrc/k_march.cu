@@ -618,8 +618,13 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march(EngineDev E, TileList 
   unsigned char* ring = smem + warp * kSlots * slot_bytes<Pol>();
   const int gw = (int)blockIdx.x * kWarps + warp, G = (int)gridDim.x * kWarps;
   View& v = views[warp];                          // (in shared memory: its pointers take no registers)
-  if (tl.solo_c.n == 0) return;                   // (the coarsest level, or one that the problem does not have)
-  if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
+  // the coarsest level, or one that the problem does not have (a server's engine of one slot may be built for a
+  // larger one): nothing to do, but the launch must not end before the one it follows, which the next one's wait
+  // would then no longer cover
+  if (tl.solo_c.n == 0 || !dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) {
+    pdl_wait();
+    return;
+  }
   // (a zero iterate leaves no squares)
   make_view<Pol, UPWARD>(v, tl.solo_d, tl.solo_c, e_sel, scale[warp], E.prm.solver != SOLVER_PCG);
   const int items = g.strips * g.chunks;

@@ -427,7 +427,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_span(const __grid_constant__ En
   const int p = blockIdx.x / kBlocks, rank = (int)cl.block_rank();
   const ProblemDev& P = E.P[p];
   const int L = P.L, top = min(L, T);
-  if (top <= 5) return;                   // (not launched for such a problem; an empty slot)
+  if (top <= 5) {                         // (not launched for such a problem; an empty slot)
+    pdl_wait();
+    return;
+  }
   const Job j{E, P, E.S + p, sm, cl.map_shared_rank(sm, max(rank - 1, 0)), cl.map_shared_rank(sm, min(rank + 1, kBlocks - 1)),
               cl.map_shared_rank(sm, 0), p, rank, top, P.coarse, P.lev[top].bc, want};
   for (int i = threadIdx.x; i < kBytes / 16; i += kThreads) reinterpret_cast<float4*>(sm)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
