@@ -360,6 +360,13 @@ __device__ __forceinline__ void run(const Job& j, const Peers& c, Node* q, bool 
     for (int i = threadIdx.x; i < (yb - ya) * n; i += kWideThreads)
       vecs<l>(*c.me)[0][g.at(i % n, ya + i / n)] = __ldcg(static_cast<const double*>(d.x[0]) + ya * n + i);
   }
+  // An iterate that another kernel reads is 0 on the Dirichlet nodes, whatever a caller has put there (hn_mg_apply takes
+  // any vector); that of a solve's own cycles is so from the start, or `full`.
+  if (!loop && !j.full)
+    for (int i = threadIdx.x; i < (g.R1 - g.R0) * n; i += kWideThreads) {
+      const int y = g.R0 + i / n, x = i % n;
+      if (is_dirichlet(x, y, n, j.bc)) static_cast<double*>(d.x[0])[y * n + x] = 0.0;
+    }
   step_sync<l>();
   for (;;) {
     if constexpr (l > 4) {
