@@ -198,7 +198,8 @@ __device__ __forceinline__ void load_bands_ahead(Bands& B, const View& v, int f,
 //
 // Dirichlet sides only: the nodes that count lie inside the grid, where the rows of a column are
 // alternately coarse rows (both coordinates even) and rows between two of them (both odd): one sum per
-// column.  (The others' coarse right-hand side is 0 from the set-up and stays so.)
+// column.  The coarse nodes on the sides get 0 in every cycle, whatever a caller has put there (hn_mg_apply takes
+// any vector): the left one of coarse row Y lies a row before the fine grid's last column, in which x = n - 1.
 struct RestrictInner {
   float s[2];
   __device__ __forceinline__ void row(const View& v, const float (&d)[4], int x, int y, int, bool store) {
@@ -219,10 +220,11 @@ struct RestrictInner {
         u = fmaf(h, c[1], u);
         u = fmaf(q, c[2], u);
         // the node on row r - 1 is (x + 1, y - 1)
-        if (store && x + 1 < n1 && y > 1 && y < n1) v.coarse[(y >> 1) * ((n1 >> 1) + 1) + ((x + 1) >> 1)] = u;
+        if (store && y <= n1 + 1) v.coarse[(y >> 1) * ((n1 >> 1) + 1) + ((x + 1) >> 1)] = x + 1 < n1 && y > 1 && y < n1 ? u : 0.0f;
         s[e] = fmaf(q, c[0], fmaf(h, c[-1], q * c[-2]));
       } else {
         s[e] = fmaf(h, c[1], fmaf(h, c[-1], s[e]) + c[0]);
+        if (store && x == n1 && y <= n1) v.coarse[(y >> 1) * ((n1 >> 1) + 1)] = 0.0f;     // node (0, y) on row r - 1
       }
     }
   }

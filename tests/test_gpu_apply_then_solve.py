@@ -25,7 +25,7 @@ def outcomes(hn, mgs, levels, bs):
 
 @pytest.mark.parametrize("solver", [0, 1])
 @pytest.mark.parametrize("bc", [15, LR])
-@pytest.mark.parametrize("prec", [0])
+@pytest.mark.parametrize("prec", [0, 1, 2])
 @pytest.mark.parametrize("levels", [(6, 4), (8, 7), (10, 9)])
 def test_solves_after_single_kernel_calls_give_the_bits_of_fresh_ones(hn, levels, prec, bc, solver):
     dt = np.float64 if prec == 0 else np.float32
