@@ -198,8 +198,7 @@ __device__ __forceinline__ void load_bands_ahead(Bands& B, const View& v, int f,
 //
 // Dirichlet sides only: the nodes that count lie inside the grid, where the rows of a column are
 // alternately coarse rows (both coordinates even) and rows between two of them (both odd): one sum per
-// column.  The coarse nodes on the sides get 0 in every cycle, whatever a caller has put there (hn_mg_apply takes
-// any vector): the left one of coarse row Y lies a row before the fine grid's last column, in which x = n - 1.
+// column.  (zero_sides sets the others.)
 struct RestrictInner {
   float s[2];
   __device__ __forceinline__ void row(const View& v, const float (&d)[4], int x, int y, int, bool store) {
@@ -220,15 +219,26 @@ struct RestrictInner {
         u = fmaf(h, c[1], u);
         u = fmaf(q, c[2], u);
         // the node on row r - 1 is (x + 1, y - 1)
-        if (store && y <= n1 + 1) v.coarse[(y >> 1) * ((n1 >> 1) + 1) + ((x + 1) >> 1)] = x + 1 < n1 && y > 1 && y < n1 ? u : 0.0f;
+        if (store && x + 1 < n1 && y > 1 && y < n1) v.coarse[(y >> 1) * ((n1 >> 1) + 1) + ((x + 1) >> 1)] = u;
         s[e] = fmaf(q, c[0], fmaf(h, c[-1], q * c[-2]));
       } else {
         s[e] = fmaf(h, c[1], fmaf(h, c[-1], s[e]) + c[0]);
-        if (store && x == n1 && y <= n1) v.coarse[(y >> 1) * ((n1 >> 1) + 1)] = 0.0f;     // node (0, y) on row r - 1
       }
     }
   }
 };
+// The coarse right-hand side on the sides, all Dirichlet: 0 in every cycle, whatever a caller has put there (hn_mg_apply
+// takes any vector).  Coarse rows r0 / 2 .. r1 / 2 by the warp that has rows r0 .. r1 - 1 (of R) of the first strip.  (As stores
+// of the restriction itself, a branch more in each row: L = 10 solve 1342 -> 1362 us, FP16 L = 12 8333 -> 8578.)
+__device__ __forceinline__ void zero_sides(float* coarse, int n, int r0, int r1, int R, int lane) {
+  const int nc = (n >> 1) + 1;
+  for (int J = (r0 + 1) / 2 + lane; J < min((r1 + 1) / 2, nc); J += 32) coarse[J * nc] = coarse[J * nc + nc - 1] = 0.0f;
+  if (r0 != 0 && r1 != R) return;
+  for (int I = lane; I < nc; I += 32) {
+    if (r0 == 0) coarse[I] = 0.0f;
+    if (r1 == R) coarse[(nc - 1) * nc + I] = 0.0f;
+  }
+}
 // Any sides: the sums and packed coordinates of the nodes on the row itself ([0]) and on the next one
 // ([1]); a neighbour off the grid, next to a free side, adds 0.
 struct RestrictAny {
@@ -600,6 +610,7 @@ __device__ __forceinline__ void sweep(const View& v, const Strip& st, const Item
                                       int lane, bool live) {
   if constexpr (UPWARD) march_up<Pol>(v, st, it, ring, early, lane, live);
   else if (v.bc == (int)HN_DIRICHLET_ALL) {
+    if (it.c0 == 0) zero_sides(v.coarse, v.n, it.r0, it.r1, (v.pitch + (1 << v.L) - 1) >> v.L, lane);
     if (zero) march_down<Pol, DOWN_ZERO, RestrictInner>(v, st, it, ring, early, lane, live);
     else march_down<Pol, DOWN, RestrictInner>(v, st, it, ring, early, lane, live);
   } else {
