@@ -334,5 +334,11 @@ enum ControlKind {
 };
 
 int sm_count();
+// Whether a launch of `blocks` blocks is a programmatic dependent one under the tuning's rule (hn_tuning.pdl): 1: every
+// launch; 2: launches of fewer blocks than SMs (their waiting blocks take no occupancy from a kernel that still runs,
+// of this stream or of another); 3: fewer blocks than twice the SMs.
+inline bool pdl_launch(int pdl, int blocks) {
+  return pdl == 1 || (pdl == 2 && blocks < sm_count()) || (pdl == 3 && blocks < 2 * sm_count());
+}
 
 }  // namespace hn

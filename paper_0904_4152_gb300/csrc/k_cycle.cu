@@ -2296,10 +2296,7 @@ cudaError_t launch_kt(void (*kern)(KArgs...), int grid, int threads, size_t smem
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   int na = 0;
-  // pdl: 1 = every launch; 2 = launches of fewer blocks than SMs (their waiting blocks do not
-  // take occupancy from a bandwidth-bound predecessor); 3 = fewer blocks than twice the SMs
-  if (pdl == 1 || (pdl == 2 && grid_or_one(grid) < sm_count()) ||
-      (pdl == 3 && grid_or_one(grid) < 2 * sm_count())) {
+  if (pdl_launch(pdl, grid_or_one(grid))) {
     attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;

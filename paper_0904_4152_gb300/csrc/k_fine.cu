@@ -366,9 +366,7 @@ cudaError_t launch_fine_f(const EngineDev& E, int solo_tiles, int summary, cudaG
   cfg.blockDim = dim3((unsigned)kFineThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  // programmatic dependent launch for small grids: their waiting blocks take no occupancy from the
-  // kernel before them
-  if (E.pdl == 1 || (E.pdl && (int)cfg.gridDim.x < (E.pdl == 3 ? 2 : 1) * sm_count())) {
+  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
@@ -460,7 +458,7 @@ cudaError_t launch_level64_t(const EngineDev& E, const TileList& tl, int level, 
   cfg.blockDim = dim3((unsigned)kFineThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  if (E.pdl == 1 || (E.pdl && (int)cfg.gridDim.x < (E.pdl == 3 ? 2 : 1) * sm_count())) {
+  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;

@@ -850,7 +850,7 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int threads, size_t sme
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  if (pdl) {
+  if (pdl_launch(pdl, grid)) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 1;
@@ -877,7 +877,10 @@ cudaError_t launch_march_t(const EngineDev& E, const TileList& tl, int level, in
   Geom g = march_strips(level, UPWARD ? 1 : 0);
   march_chunks(g, (unsigned)g.strips, (unsigned)(per_sm * sm_count() * kWarps));
   const int grid = std::min(per_sm * sm_count(), (g.strips * g.chunks + kWarps - 1) / kWarps);
-  return launch_pdl(k_march<Pol, UPWARD>, grid, kWarps * 32, smem, s, E.pdl, E, tl, level, want, e_sel, g);
+  // programmatic at any size (unless off): the waiting blocks fetch their first rows' constant data meanwhile.  By the
+  // rule (pdl_launch) the large levels' would not be: L = 10 solve 1344 -> 1383 us, L = 12 9300 -> 9524, FP16 9369 ->
+  // 9687, CG at L = 11 3379 -> 3492.
+  return launch_pdl(k_march<Pol, UPWARD>, grid, kWarps * 32, smem, s, E.pdl ? 1 : 0, E, tl, level, want, e_sel, g);
 }
 
 template <class Pol, bool UPWARD>
@@ -885,7 +888,11 @@ cudaError_t launch_group_t(const EngineDev& E, int level, int T, int want, cudaS
   constexpr int smem = kWarps * kSlots * slot_bytes<Pol>();
   static const int per_sm = march_resident(k_march_group<Pol, UPWARD>, smem);
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  return launch_pdl(k_march_group<Pol, UPWARD>, per_sm * sm_count(), kWarps * 32, smem, s, E.pdl, E, level, T, want);
+  // never programmatic: what they can do before their predecessor ends is little, and blocks of 230 registers a thread
+  // that wait on every SM hold up whatever else runs, such as a server's set-up of the next requests (24 requests of
+  // L = 6..8, FP16 13.2 -> 10.4 ms, of L = 6..9 in FP32 11.1 -> 9.8; a batch of 64 6.26 -> 6.13; below the number of SMs
+  // too: 2 problems of L = 5..7 1467 -> 1515 us)
+  return launch_pdl(k_march_group<Pol, UPWARD>, per_sm * sm_count(), kWarps * 32, smem, s, 0, E, level, T, want);
 }
 
 }  // namespace

@@ -346,7 +346,7 @@ cudaError_t launch_small_t(const EngineDev& E, const SmallSolo& solo, int T, int
   cfg.dynamicSmemBytes = (size_t)small_smem<Pol>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  if (E.pdl) {
+  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 1;

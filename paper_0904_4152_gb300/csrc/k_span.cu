@@ -483,7 +483,7 @@ cudaError_t launch_span_t(const EngineDev& E, int T, int want, int loop, cudaStr
   attr[0].val.clusterDim.x = (unsigned)kBlocks;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.numAttrs = 1;
-  if (E.pdl) {
+  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
