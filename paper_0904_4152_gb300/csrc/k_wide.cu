@@ -451,7 +451,9 @@ cudaError_t launch_wide(const EngineDev& E, int T, int want, int loop, cudaStrea
   attr[0].val.clusterDim.x = (unsigned)kWideBlocks;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.numAttrs = 1;
-  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
+  // programmatic at any size (unless off): the blocks fetch their nodes' bands while they wait (10 problems of L = 8 4028 us
+  // by the rule, 3969 so; 14 of L = 6..9 5849, 5772)
+  if (pdl_launch(E.pdl ? 1 : 0, (int)cfg.gridDim.x)) {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
