@@ -101,7 +101,9 @@ Tuning batch_tuning(const std::vector<hn_mg*>& list) {
   bool same = list[0]->tuned;
   for (hn_mg* mg : list) same = same && mg->tuned && mg->tuning == list[0]->tuning;
   if (same) return list[0]->tuning;
-  return group_tuning(list[0]->prm, (int)list.size());
+  GroupSize size;
+  for (hn_mg* mg : list) ++size.problems[mg->L];
+  return group_tuning(list[0]->prm, size, false);
 }
 
 hn_status copy_in(double* dst, const double* src, long long N, int device_ptrs, cudaStream_t s) {

@@ -674,6 +674,13 @@ hn_status Engine::set_members(const std::vector<hn_mg*>& slots) {
     if (mg) mask |= 1u << mg->L;
   if (mask != topMask_ && !topMaskAll_) drop_graphs();
   topMask_ = mask;
+  if (!topMaskAll_) {                              // (a server's engine: sized once, by its slots)
+    GroupSize size;
+    for (hn_mg* mg : members_)
+      if (mg) ++size.problems[mg->L];
+    if (std::memcmp(&size, &groupSize_, sizeof size) != 0) drop_graphs();
+    groupSize_ = size;
+  }
   return HN_OK;
 }
 
@@ -966,13 +973,13 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
     if (march_level(l) && cap_ != 1) {
       // the finest level of every problem and its check, then level by level the problems above it
       if (l == Lmax_) {
-        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, 0, T, want, 0, s));
+        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, groupSize_, 0, T, want, 0, s));
         if (prm_.solver != SOLVER_PCG) {
-          HN_LAUNCH(KC_CHECK, l, launch_march_check_group(E_, T, want, s));
+          HN_LAUNCH(KC_CHECK, l, launch_march_check_group(E_, groupSize_, T, want, s));
           HN_TRY(after_check());
         }
       } else {
-        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, l, T, want, 0, s));
+        HN_LAUNCH(KC_SWEEP_DOWN, l, launch_march_group(E_, groupSize_, l, T, want, 0, s));
       }
       continue;
     }
@@ -1037,7 +1044,7 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   int e_sel = 0;                           // buffer of the coarse iterate (the tail's: 0)
   for (int l = std::max(T, M) + 1; l <= Lmax_; ++l) {
     if (march_level(l)) {                  // prolongation and both post-smoothing steps, buffer 1 to 0
-      if (cap_ != 1) HN_LAUNCH(KC_SWEEP_UP, l, launch_march_group(E_, l == Lmax_ ? 0 : l, T, want, 1, s));
+      if (cap_ != 1) HN_LAUNCH(KC_SWEEP_UP, l, launch_march_group(E_, groupSize_, l == Lmax_ ? 0 : l, T, want, 1, s));
       else HN_LAUNCH(KC_SWEEP_UP, l, launch_march(E_, lists_[l], l, want, 1, e_sel, s));
       e_sel = 0;
       continue;
@@ -1077,8 +1084,8 @@ hn_status Engine::issue_init(cudaStream_t s, cudaGraphConditionalHandle h, int u
   // the boundary check and ||b||; CG: the initial residual r = b - A x and its check (then the first
   // cycle preconditions it).  An engine of one problem ends the start in the last of these kernels.
   const bool pcg = prm_.solver == SOLVER_PCG;
-  HN_LAUNCH0(launch_fine(E_, FINE_NORM_B, soloTiles_, cap_ == 1 && !pcg ? 2 : 0, h, use_h, s));
-  if (pcg) HN_LAUNCH0(launch_fine(E_, FINE_OUTER, soloTiles_, cap_ == 1 ? 2 : 0, h, use_h, s));
+  HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_NORM_B, soloTiles_, cap_ == 1 && !pcg ? 2 : 0, h, use_h, s));
+  if (pcg) HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_OUTER, soloTiles_, cap_ == 1 ? 2 : 0, h, use_h, s));
   if (cap_ != 1) HN_LAUNCH0(launch_summary(E_, h, use_h, 0, s));
   return HN_OK;
 }
@@ -1098,21 +1105,21 @@ hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h,
     // z = M r (one cycle from zero), rho' = (r, z), beta, p = z + beta p, then the CG step
     // q = A p, alpha, x += alpha p, r -= alpha q, and its check
     HN_TRY(issue_vcycle(s, PH_PRECOND));
-    HN_LAUNCH(KC_PCG_DOT, -1, launch_fine(E_, FINE_PCG_DOT, soloTiles_, 0, h, use_h, s));
-    HN_LAUNCH(KC_PCG_P, -1, launch_fine(E_, FINE_PCG_P, soloTiles_, 0, h, use_h, s));
-    HN_LAUNCH(KC_PCG_Q, -1, launch_fine(E_, FINE_PCG_Q, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_PCG_DOT, -1, launch_fine(E_, groupSize_, FINE_PCG_DOT, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_PCG_P, -1, launch_fine(E_, groupSize_, FINE_PCG_P, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_PCG_Q, -1, launch_fine(E_, groupSize_, FINE_PCG_Q, soloTiles_, 0, h, use_h, s));
     count_base(end ? 1 : 2);
-    HN_LAUNCH(KC_PCG_X, -1, launch_fine(E_, FINE_PCG_X, soloTiles_, end, h, use_h, s));
+    HN_LAUNCH(KC_PCG_X, -1, launch_fine(E_, groupSize_, FINE_PCG_X, soloTiles_, end, h, use_h, s));
   } else if (prm_.prec == P64) {
     HN_TRY(issue_vcycle(s, PH_CYCLE));
     count_base(1);
     HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
     return HN_OK;
   } else {
-    HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_fine(E_, FINE_OUTER, soloTiles_, 0, h, use_h, s));
+    HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_fine(E_, groupSize_, FINE_OUTER, soloTiles_, 0, h, use_h, s));
     HN_TRY(issue_vcycle(s, PH_INNER));
     count_base(end ? 1 : 2);
-    HN_LAUNCH(KC_UPDATE, -1, launch_fine(E_, FINE_UPDATE, soloTiles_, end, h, use_h, s));
+    HN_LAUNCH(KC_UPDATE, -1, launch_fine(E_, groupSize_, FINE_UPDATE, soloTiles_, end, h, use_h, s));
   }
   if (!end) HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
   return HN_OK;

@@ -108,20 +108,60 @@ struct Tuning {
   }
 };
 
-// Launch shape of an engine of several problems (slots): FP32 / FP16 hierarchies take the one-block tail
-// (levels to kSmallTop) below the marching sweeps; FP64 ones, whose levels 5 and 6 are too slow for one
-// SM, by the number of problems: up to 31 the cluster tail of 16 blocks (k_wide; measured against the general
-// tail: 4 problems of L = 3..6 1901 -> 563 us, 16 of L = 3..9 5.48 -> 4.57 ms), more of them one block each
-// (64 problems 12.3 against 13.0 ms, 256 36.6 against 43.4 ms).
-inline bool wide_options(const Params& prm) {
-  return prm.prec == P64 && prm.pre == 2 && prm.post == 2 && !prm.coarse_cg;
-}
-inline Tuning group_tuning(const Params& prm, int slots) {
+// Launch shape of an engine of several problems.
+//
+// FP32 / FP16: the marching sweeps above the one-block tail, where they have work for the chip.  A launch that serves
+// several problems takes ~8 us however few they are (it lists them and cuts their strips first), and where few small
+// problems wait for it, levels inside a cluster's tail, or one launch per step, are faster (us, marching -> the form
+// chosen here; `fill`: the problems' nodes against as many of the largest, 1 where all have one level, 0.3 where levels
+// 5..8 are mixed):
+//   2..7 problems, Lmax 6..8: the whole cycle in the cluster tail.  2 of L = 6, 7 1328 -> 1043, 7 of L = 8 2470 -> 2067, FP16, 2
+//     of L = 8, 2246 -> 1899;
+//   Lmax 9, up to 4 problems (FP16: 7): one launch per step above the tail of level 7, 2 of L = 9 2599 -> 2383, FP16 2568 ->
+//     2258, 7 3476 -> 3303 (FP32, 7: 3585 against 3873, marching); up to 4 of mixed levels: the cluster tail to level 8
+//     below one march, 2 of L = 6..9 1845 -> 1565 (by steps 1750);
+//   8..11 problems (FP16: 31), Lmax 6..8, most of them as large (FP16: or Lmax 6, 7): one launch per step above a tail of level 6.  9 of L = 8
+//     3384 -> 3214, FP16 3555 -> 3235, 24 4388 -> 4257 (FP32, 24: 4211 against 4519; 10 of L = 5..8 3188 against 3401, marching);
+//   Lmax 10, marching always: 2 problems 3827 against 4274 by steps, 24 15647 against 28666;
+//   CG, whose cycles have no check: marching but for 2..7 problems of Lmax 6, 7 (10 of L = 8 1409 against 1562 by steps).
+// FP64, whose levels 5 and 6 are too slow for one SM, by the number of problems: up to 31 the cluster tail of 16
+// blocks (k_wide; measured against the general tail: 4 problems of L = 3..6 1901 -> 563 us, 16 of L = 3..9 5.48 -> 4.57
+// ms), more of them one block each (64 problems 12.3 against 13.0 ms, 256 36.6 against 43.4 ms).
+// A server's engine (any_level: its problems may end on any of its levels, which a launch per step would check one by
+// one), up to 15 slots and level 9: whole cycles in the cluster tail (12 requests of L = 6, 7 on 4 slots 8735 -> 7825,
+// FP16 9647 -> 8689; 16 of L = 6..9 on 8 slots, FP16, 11105 -> 10929).
+// Other cycles than V(2,2) have the general tail and per-step launches only, the CG coarse solver the general tail.
+inline bool fused_options(const Params& prm) { return prm.pre == 2 && prm.post == 2 && !prm.coarse_cg; }
+inline bool wide_options(const Params& prm) { return prm.prec == P64 && fused_options(prm); }
+inline Tuning group_tuning(const Params& prm, const GroupSize& size, bool any_level) {
   Tuning t;
-  if (prm.prec != P64 || slots >= 32) { t.tail_level = kSmallTop; t.cluster = 1; }
-  else if (wide_options(prm)) t.tail_level = kWideTop;
-  else if (slots >= 8) { t.tail_level = 6; t.cluster = 4; }
-  return t;
+  auto shape = [&](int tail_level, int cluster, int march) {
+    t.tail_level = tail_level;
+    t.cluster = cluster;
+    t.march = march;
+    return t;
+  };
+  const long long slots = size.sum([](int) { return 1; });
+  int Lmax = 0;
+  for (int l = 0; l <= kMaxLevel; ++l)
+    if (size.problems[l]) Lmax = l;
+  if (slots >= 32) return shape(kSmallTop, 1, 1);
+  if (!fused_options(prm)) {
+    if (any_level) return t;
+    if (slots < 8) return shape(7, 16, Lmax >= 10);
+    return prm.pre == 2 && prm.post == 2 && Lmax >= 9 ? shape(kSmallTop, 1, 1) : shape(6, 4, 0);
+  }
+  if (prm.prec == P64) return shape(kWideTop, 16, 1);
+  const bool half = prm.prec == P16;
+  if (any_level) return slots < 16 && Lmax <= 9 ? shape(8, 16, 1) : shape(kSmallTop, 1, 1);
+  if (slots < 8 && Lmax > kSmallTop && Lmax <= (prm.solver == SOLVER_PCG ? 7 : 8)) return shape(8, 16, 1);
+  if (prm.solver != SOLVER_PCG && slots > 0) {
+    const double fill = (double)size.sum([](int l) { return N_of(l); }) / ((double)slots * (double)N_of(Lmax));
+    if (Lmax == 9 && fill >= 0.5 && slots < (half ? 8 : 5)) return shape(7, 16, 0);
+    if (Lmax == 9 && fill < 0.5 && slots < 5) return shape(8, 16, 1);
+    if (Lmax > kSmallTop && Lmax <= 8 && slots < (half ? 32 : 12) && (half ? Lmax <= 7 || fill >= 0.6 : fill >= 0.8)) return shape(6, 4, 0);
+  }
+  return shape(kSmallTop, 1, 1);
 }
 
 class Engine;
@@ -231,7 +271,12 @@ class Engine {
   const Tuning& tuning() const { return tune_; }
   // levels that may be some problem's finest level (their first smoothing step may start from a
   // nonzero iterate); all levels for the server
-  void set_top_mask_all() { topMaskAll_ = true; drop_graphs(); }
+  void set_top_mask_all() {
+    topMaskAll_ = true;
+    groupSize_ = GroupSize{};
+    groupSize_.problems[Lmax_] = cap_;
+    drop_graphs();
+  }
   int kernel_times(hn_kernel_time* out, int max) const;
 
   long long last_launches() const { return lastLaunches_; }
@@ -282,6 +327,7 @@ class Engine {
   long long fineCap_ = 0;
   TileList lists_[kMaxLevel + 1] = {};
   int soloTiles_ = 0;               // an engine of one problem: the tiles of its finest level
+  GroupSize groupSize_{};           // the most problems of each finest level that a launch serves
   int grid_[kMaxLevel + 1] = {};
   TileList* dLists_ = nullptr;      // device copy of lists_ (read by the persistent kernels)
   TileList* hLists_ = nullptr;      // its pinned staging copy

@@ -293,6 +293,17 @@ SweepGeom sweep_geom(int level);
 size_t sweep_smem_bytes(int prec, const SweepGeom& g);
 cudaError_t launch_sweep_down(const EngineDev& E, TileList tl, int level, int want, int top, cudaStream_t s);
 cudaError_t launch_sweep_up(const EngineDev& E, TileList tl, int level, int want, int e_sel, cudaStream_t s);
+// The problems an engine of several has at most, by finest level: what the launches that serve them all are sized by
+// (a server's engine, whose members come and go: as many of its highest level as it has slots).
+struct GroupSize {
+  int problems[kMaxLevel + 1] = {};
+  template <class F> long long sum(F&& of_level) const {     // of_level(finest level): work items of a problem
+    long long t = 0;
+    for (int l = 0; l <= kMaxLevel; ++l)
+      if (problems[l]) t += (long long)problems[l] * of_level(l);
+    return t;
+  }
+};
 // Marching sweeps (k_march.cu) for FP32 / FP16 hierarchies with V(2,2) cycles, levels from
 // kMarchMinLevel: the down part (both smoothing steps, from the zero iterate or from buffer 0 of a
 // problem's own finest level, whose residual squares it leaves in the level's defect array; the defect,
@@ -303,9 +314,9 @@ cudaError_t launch_sweep_up(const EngineDev& E, TileList tl, int level, int want
 // finest level.
 constexpr int kMarchSoloLevel = 9;   // an engine of one problem: from here
 cudaError_t launch_march(const EngineDev& E, const TileList& tl, int level, int want, int up, int e_sel, cudaStream_t s);
-cudaError_t launch_march_group(const EngineDev& E, int level, int T, int want, int up, cudaStream_t s);
+cudaError_t launch_march_group(const EngineDev& E, const GroupSize& size, int level, int T, int want, int up, cudaStream_t s);
 cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, int level, int want, cudaStream_t s);
-cudaError_t launch_march_check_group(const EngineDev& E, int T, int want, cudaStream_t s);
+cudaError_t launch_march_check_group(const EngineDev& E, const GroupSize& size, int T, int want, cudaStream_t s);
 // x_sel: bit 0 the fine buffer corrected in place, bit 1 the buffer of the coarse iterate
 cudaError_t launch_prolong(const EngineDev& E, TileList tl, int level, int want, int x_sel,
                            int grid, cudaStream_t s);
@@ -318,7 +329,7 @@ cudaError_t launch_coarse(const EngineDev& E, TileList tl, int want, int grid, c
 // last block.  solo_tiles: the tiles of an engine of one problem, else 0.  summary (an engine of one
 // problem): 1: the iteration ends here (WHILE handle h if use_handle), 2: the start of a solve ends here.
 enum FineKind { FINE_NORM_B = 0, FINE_OUTER, FINE_UPDATE, FINE_PCG_Q, FINE_PCG_X, FINE_PCG_DOT, FINE_PCG_P };
-cudaError_t launch_fine(const EngineDev& E, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+cudaError_t launch_fine(const EngineDev& E, const GroupSize& size, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                         int use_handle, cudaStream_t s);
 // kind: ControlKind; level: for CTRL_PRE, the finest level whose problems are checked
 cudaError_t launch_control(const EngineDev& E, int kind, cudaStream_t s, int level = -1);

@@ -471,7 +471,7 @@ __device__ double problem_partial_sum(const double* part, int ntiles, double* sh
 // group: each group by problem_partial_sum, then the group sums in group order.  (One block adding
 // 131,072 FP64 partials at L = 12 is bound by one SM's FP64 rate, ~30 us; the control kernel
 // gives each group its own block.)  Every path that forms a problem's norm uses this order.
-__device__ __forceinline__ int sum_groups(int ntiles) { return (ntiles + kSumGroup - 1) / kSumGroup; }
+__host__ __device__ inline int sum_groups(int ntiles) { return (ntiles + kSumGroup - 1) / kSumGroup; }
 
 __device__ double group_partial_sum(const double* part, int ntiles, int j, double* sh, bool df = false) {
   const int lo = j * kSumGroup;

@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kFineThreads, OP == F_OUTER || OP == F_PCG_Q ?
 }
 
 template <int OP, class V, int FORM>
-cudaError_t launch_fine_f(const EngineDev& E, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+cudaError_t launch_fine_f(const EngineDev& E, const GroupSize& size, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                           int use_handle, cudaStream_t s) {
   auto kern = k_fine<OP, V, FORM>;
   static const int per_sm = [&] {
@@ -359,14 +359,19 @@ cudaError_t launch_fine_f(const EngineDev& E, int solo_tiles, int summary, cudaG
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kFineThreads, 0) == cudaSuccess && b > 0 ? b : 1;
   }();
   cudaLaunchConfig_t cfg = {};
-  // no more than one wave of blocks
-  const int wave = per_sm * sm_count(), want = FORM == SOLO_TILES ? (solo_tiles + kFineWarps - 1) / kFineWarps
-                                              : FORM == SOLO_LINKS ? (solo_tiles + kLink - 1) / kLink : wave;
-  cfg.gridDim = dim3((unsigned)std::min(wave, want), 1, 1);
+  // no more than one wave of blocks, nor than have work: a tile for each warp; a link for all warps, which share it.  The steps
+  // of CG on several problems take a block for each tile: few problems leave SMs idle, and eight stencils on one
+  // SM wait for its FP64 pipe (2 problems of L = 5 551 -> 489 us, of L = 5..7 823 -> 756; a whole wave 523, 773; as programmatic
+  // launches, where the rule would have them so, 487, 774).  The defect correction's two steps a solve gain more
+  // from a grid below that rule's line (4 problems of L = 5..7 1317 against 1352 us, a whole wave 1360).
+  const bool by_tile = FORM == GROUPS && E.prm.solver == SOLVER_PCG;
+  const long long tiles = FORM == GROUPS ? size.sum([](int l) { return fine_tiles(l); }) : solo_tiles;
+  const int share = FORM == SOLO_LINKS ? kLink : by_tile ? 1 : kFineWarps;
+  cfg.gridDim = dim3((unsigned)std::max<long long>(1, std::min<long long>(per_sm * sm_count(), (tiles + share - 1) / share)), 1, 1);
   cfg.blockDim = dim3((unsigned)kFineThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  if (pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
+  if (!by_tile && pdl_launch(E.pdl, (int)cfg.gridDim.x)) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
@@ -375,18 +380,18 @@ cudaError_t launch_fine_f(const EngineDev& E, int solo_tiles, int summary, cudaG
   return cudaLaunchKernelEx(&cfg, kern, E, solo_tiles, summary, h, use_handle);
 }
 template <int OP, class V>
-cudaError_t launch_fine_t(const EngineDev& E, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+cudaError_t launch_fine_t(const EngineDev& E, const GroupSize& size, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                           int use_handle, cudaStream_t s) {
-  if (!solo_tiles) return launch_fine_f<OP, V, GROUPS>(E, solo_tiles, summary, h, use_handle, s);
+  if (!solo_tiles) return launch_fine_f<OP, V, GROUPS>(E, size, solo_tiles, summary, h, use_handle, s);
   if constexpr (fine_sums(OP))
-    if (solo_tiles > kSumGroup) return launch_fine_f<OP, V, SOLO_LINKS>(E, solo_tiles, summary, h, use_handle, s);
-  return launch_fine_f<OP, V, SOLO_TILES>(E, solo_tiles, summary, h, use_handle, s);
+    if (solo_tiles > kSumGroup) return launch_fine_f<OP, V, SOLO_LINKS>(E, size, solo_tiles, summary, h, use_handle, s);
+  return launch_fine_f<OP, V, SOLO_TILES>(E, size, solo_tiles, summary, h, use_handle, s);
 }
 template <int OP>
-cudaError_t launch_fine_p(const EngineDev& E, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+cudaError_t launch_fine_p(const EngineDev& E, const GroupSize& size, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                           int use_handle, cudaStream_t s) {
-  return E.prm.prec == P64 ? launch_fine_t<OP, double>(E, solo_tiles, summary, h, use_handle, s)
-                           : launch_fine_t<OP, float>(E, solo_tiles, summary, h, use_handle, s);
+  return E.prm.prec == P64 ? launch_fine_t<OP, double>(E, size, solo_tiles, summary, h, use_handle, s)
+                           : launch_fine_t<OP, float>(E, size, solo_tiles, summary, h, use_handle, s);
 }
 
 // A smoothing step or the defect of an FP64 level of a problem solved alone (k_band's step, same bits).  Bound by the
@@ -480,16 +485,16 @@ cudaError_t launch_level64(const EngineDev& E, const TileList& tl, int kind, int
                 : launch_level64_t<LV_DEFECT, LD_NC>(E, tl, level, want, in_sel, fuse, s);
 }
 
-cudaError_t launch_fine(const EngineDev& E, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
+cudaError_t launch_fine(const EngineDev& E, const GroupSize& size, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                         int use_handle, cudaStream_t s) {
   switch (kind) {
-    case FINE_NORM_B: return launch_fine_t<F_NORM_B, float>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_OUTER: return launch_fine_p<F_OUTER>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_UPDATE: return launch_fine_t<F_UPDATE, float>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_PCG_Q: return launch_fine_t<F_PCG_Q, float>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_PCG_X: return launch_fine_p<F_PCG_X>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_PCG_DOT: return launch_fine_p<F_PCG_DOT>(E, solo_tiles, summary, h, use_handle, s);
-    case FINE_PCG_P: return launch_fine_p<F_PCG_P>(E, solo_tiles, summary, h, use_handle, s);
+    case FINE_NORM_B: return launch_fine_t<F_NORM_B, float>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_OUTER: return launch_fine_p<F_OUTER>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_UPDATE: return launch_fine_t<F_UPDATE, float>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_PCG_Q: return launch_fine_t<F_PCG_Q, float>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_PCG_X: return launch_fine_p<F_PCG_X>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_PCG_DOT: return launch_fine_p<F_PCG_DOT>(E, size, solo_tiles, summary, h, use_handle, s);
+    case FINE_PCG_P: return launch_fine_p<F_PCG_P>(E, size, solo_tiles, summary, h, use_handle, s);
   }
   return cudaErrorInvalidValue;
 }

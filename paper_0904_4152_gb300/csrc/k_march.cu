@@ -542,6 +542,7 @@ __device__ void march_up(const View& v, const Strip& st, const Item& it, unsigne
 struct Geom {
   int strips, own, chunks, rows, R;
 };
+constexpr int kLeastRows = 2;            // of a chunk, in a launch that serves several problems
 __host__ __device__ inline Geom march_strips(int L, int up) {
   Geom g;
   const unsigned W = 1u << L, widest = kTile - 2 * (up ? 4 : 8);
@@ -698,7 +699,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march_group(EngineDev E, int
     if (threadIdx.x < 32) {
       int total = 0;
       for (int l = kMarchMinLevel; l <= kMaxLevel; ++l) total += hist[l] * cut[l].x * cut[l].y;
-      const int least = max(2, (total + G - 1) / G), rows = least + lane * max(1, least / 16);
+      const int least = max(kLeastRows, (total + G - 1) / G), rows = least + lane * max(1, least / 16);
       int items = 0;
       for (int l = kMarchMinLevel; l <= kMaxLevel; ++l)
         if (hist[l]) items += hist[l] * cut[l].x * ((cut[l].y + rows - 1) / rows);
@@ -813,19 +814,20 @@ __global__ void __launch_bounds__(256) k_march_check(EngineDev E, TileList tl, i
   }
   check_part(E, 0, static_cast<const float*>(tl.solo_d.r), level, (int)blockIdx.x / nb, (int)blockIdx.x % nb, nb, want, sh);
 }
-// ... and of all problems whose finest level is above the tail, one block per 1024 tiles at most
+// ... and of all problems whose finest level is above the tail, one block per 1024 tiles at most: the blocks of a problem
+// (whole groups of kSumGroup tiles)
+__host__ __device__ inline int check_blocks(int L, int T) {
+  const int tiles = fine_tiles(L), first = tiles < kSumGroup ? tiles : kSumGroup;
+  return L <= T ? 1 : sum_groups(tiles) * ((first + 1023) / 1024);
+}
 __global__ void __launch_bounds__(256) k_march_check_group(EngineDev E, int T, int want) {
   pdl_start();
   __shared__ double sh[32];
   __shared__ Served q;
-  auto blocks = [T](int l) {                      // of a problem: whole groups of kSumGroup tiles
-    const int tiles = fine_tiles(l);
-    return l <= T ? 1 : sum_groups(tiles) * ((min(tiles, kSumGroup) + 1023) / 1024);
-  };
   for (int base = 0; base < E.nprob; base += kListMax) {
     const int n = list_served(E, q, base, 0, [](const ProbState&, int L) { return L >= HN_MIN_LEVEL; });
     if (n == 0) continue;
-    const int items = number_items(q, n, blocks);
+    const int items = number_items(q, n, [T](int l) { return check_blocks(l, T); });
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
       const int m = served_of(q, n, it), p = q.slot[m], l = q.level[m], blk = it - q.start[m];
       // (a problem leaves the phase only after every block of its check has counted itself in)
@@ -884,15 +886,22 @@ cudaError_t launch_march_t(const EngineDev& E, const TileList& tl, int level, in
 }
 
 template <class Pol, bool UPWARD>
-cudaError_t launch_group_t(const EngineDev& E, int level, int T, int want, cudaStream_t s) {
+cudaError_t launch_group_t(const EngineDev& E, const GroupSize& size, int level, int T, int want, cudaStream_t s) {
   constexpr int smem = kWarps * kSlots * slot_bytes<Pol>();
   static const int per_sm = march_resident(k_march_group<Pol, UPWARD>, smem);
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  // no more than one wave of blocks, nor than have work where every chunk has the least height
+  const long long items = size.sum([&](int l) {
+    if (l <= (level ? level : T)) return 0;
+    const Geom g = march_strips(level ? level : l, UPWARD ? 1 : 0);
+    return g.strips * ((g.R + kLeastRows - 1) / kLeastRows);
+  });
+  const int grid = (int)std::max<long long>(1, std::min<long long>(per_sm * sm_count(), (items + kWarps - 1) / kWarps));
   // never programmatic: what they can do before their predecessor ends is little, and blocks of 230 registers a thread
   // that wait on every SM hold up whatever else runs, such as a server's set-up of the next requests (24 requests of
   // L = 6..8, FP16 13.2 -> 10.4 ms, of L = 6..9 in FP32 11.1 -> 9.8; a batch of 64 6.26 -> 6.13; below the number of SMs
   // too: 2 problems of L = 5..7 1467 -> 1515 us)
-  return launch_pdl(k_march_group<Pol, UPWARD>, per_sm * sm_count(), kWarps * 32, smem, s, 0, E, level, T, want);
+  return launch_pdl(k_march_group<Pol, UPWARD>, grid, kWarps * 32, smem, s, 0, E, level, T, want);
 }
 
 }  // namespace
@@ -906,12 +915,12 @@ cudaError_t launch_march(const EngineDev& E, const TileList& tl, int level, int 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_march_group(const EngineDev& E, int level, int T, int want, int up, cudaStream_t s) {
+cudaError_t launch_march_group(const EngineDev& E, const GroupSize& size, int level, int T, int want, int up, cudaStream_t s) {
   if ((level ? level : T + 1) < kMarchMinLevel) return cudaErrorInvalidValue;
   if (E.prm.prec == P32)
-    return up ? launch_group_t<F32, true>(E, level, T, want, s) : launch_group_t<F32, false>(E, level, T, want, s);
+    return up ? launch_group_t<F32, true>(E, size, level, T, want, s) : launch_group_t<F32, false>(E, size, level, T, want, s);
   if (E.prm.prec == P16)
-    return up ? launch_group_t<F16, true>(E, level, T, want, s) : launch_group_t<F16, false>(E, level, T, want, s);
+    return up ? launch_group_t<F16, true>(E, size, level, T, want, s) : launch_group_t<F16, false>(E, size, level, T, want, s);
   return cudaErrorInvalidValue;
 }
 
@@ -922,8 +931,10 @@ cudaError_t launch_march_check(const EngineDev& E, const TileList& tl, int level
   return launch_pdl(k_march_check, groups * nb, 256, 0, s, E.pdl, E, tl, level, want, nb);
 }
 
-cudaError_t launch_march_check_group(const EngineDev& E, int T, int want, cudaStream_t s) {
-  return launch_pdl(k_march_check_group, 2 * sm_count(), 256, 0, s, E.pdl, E, T, want);
+cudaError_t launch_march_check_group(const EngineDev& E, const GroupSize& size, int T, int want, cudaStream_t s) {
+  const long long items = size.sum([&](int l) { return check_blocks(l, T); });
+  const int grid = (int)std::max<long long>(1, std::min<long long>(2 * sm_count(), items));
+  return launch_pdl(k_march_check_group, grid, 256, 0, s, E.pdl, E, T, want);
 }
 
 }  // namespace hn

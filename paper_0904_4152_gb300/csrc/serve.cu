@@ -580,7 +580,9 @@ void hn_server::run(int lane) {
           fail_all(hn_last_error());
           break;
         }
-        engine->set_tuning(group_tuning(engine->params(), max_active));
+        GroupSize most;
+        most.problems[Lcap] = max_active;
+        engine->set_tuning(group_tuning(engine->params(), most, true));
         engine->set_iter_limit(UINT_MAX - 1);
         engine->set_top_mask_all();
         engine_lmax = Lcap;
