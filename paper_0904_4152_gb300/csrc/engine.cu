@@ -1082,25 +1082,23 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
 
 hn_status Engine::issue_init(cudaStream_t s, cudaGraphConditionalHandle h, int use_h) {
   // the boundary check and ||b||; CG: the initial residual r = b - A x and its check (then the first
-  // cycle preconditions it).  An engine of one problem ends the start in the last of these kernels.
+  // cycle preconditions it).  The last of these kernels ends the start.
   const bool pcg = prm_.solver == SOLVER_PCG;
-  HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_NORM_B, soloTiles_, cap_ == 1 && !pcg ? 2 : 0, h, use_h, s));
-  if (pcg) HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_OUTER, soloTiles_, cap_ == 1 ? 2 : 0, h, use_h, s));
-  if (cap_ != 1) HN_LAUNCH0(launch_summary(E_, h, use_h, 0, s));
+  HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_NORM_B, soloTiles_, pcg ? 0 : 2, h, use_h, s));
+  if (pcg) HN_LAUNCH0(launch_fine(E_, groupSize_, FINE_OUTER, soloTiles_, 2, h, use_h, s));
   return HN_OK;
 }
 
 hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h, int use_h) {
   cudaStream_t s = s0;
   const int start = counting_;
-  // the kernels outside the IF node, those still to be launched included
-  auto count_base = [&](int to_come) {
+  // the kernels outside the IF node, the last one, still to be launched, included
+  auto count_base = [&] {
     if (!condCapture_) return;
     const CondDev& cd = E_.prm.cond;
-    E_.prm.cond.n_base = (unsigned)(counting_ + to_come - start) - cd.n_cycle - cd.n_outer - cd.n_update;
+    E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle - cd.n_outer - cd.n_update;
   };
-  // an engine of one problem ends the iteration in its last vector step
-  const int end = cap_ == 1 ? 1 : 0;
+  // the last vector step ends the iteration
   if (prm_.solver == SOLVER_PCG) {
     // z = M r (one cycle from zero), rho' = (r, z), beta, p = z + beta p, then the CG step
     // q = A p, alpha, x += alpha p, r -= alpha q, and its check
@@ -1108,20 +1106,18 @@ hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h,
     HN_LAUNCH(KC_PCG_DOT, -1, launch_fine(E_, groupSize_, FINE_PCG_DOT, soloTiles_, 0, h, use_h, s));
     HN_LAUNCH(KC_PCG_P, -1, launch_fine(E_, groupSize_, FINE_PCG_P, soloTiles_, 0, h, use_h, s));
     HN_LAUNCH(KC_PCG_Q, -1, launch_fine(E_, groupSize_, FINE_PCG_Q, soloTiles_, 0, h, use_h, s));
-    count_base(end ? 1 : 2);
-    HN_LAUNCH(KC_PCG_X, -1, launch_fine(E_, groupSize_, FINE_PCG_X, soloTiles_, end, h, use_h, s));
+    count_base();
+    HN_LAUNCH(KC_PCG_X, -1, launch_fine(E_, groupSize_, FINE_PCG_X, soloTiles_, 1, h, use_h, s));
   } else if (prm_.prec == P64) {
     HN_TRY(issue_vcycle(s, PH_CYCLE));
-    count_base(1);
+    count_base();
     HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
-    return HN_OK;
   } else {
     HN_LAUNCH(KC_OUTER_DEFECT, -1, launch_fine(E_, groupSize_, FINE_OUTER, soloTiles_, 0, h, use_h, s));
     HN_TRY(issue_vcycle(s, PH_INNER));
-    count_base(end ? 1 : 2);
-    HN_LAUNCH(KC_UPDATE, -1, launch_fine(E_, groupSize_, FINE_UPDATE, soloTiles_, end, h, use_h, s));
+    count_base();
+    HN_LAUNCH(KC_UPDATE, -1, launch_fine(E_, groupSize_, FINE_UPDATE, soloTiles_, 1, h, use_h, s));
   }
-  if (!end) HN_LAUNCH0(launch_summary(E_, h, use_h, 1, s));
   return HN_OK;
 }
 

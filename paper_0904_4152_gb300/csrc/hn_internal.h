@@ -326,8 +326,8 @@ cudaError_t launch_prolong_jacobi(const EngineDev& E, TileList tl, int level, in
                                   int grid, cudaStream_t s);
 cudaError_t launch_coarse(const EngineDev& E, TileList tl, int want, int grid, cudaStream_t s);
 // The FP64 vector steps on each problem's finest level (k_fine.cu), with the problems' control steps in the
-// last block.  solo_tiles: the tiles of an engine of one problem, else 0.  summary (an engine of one
-// problem): 1: the iteration ends here (WHILE handle h if use_handle), 2: the start of a solve ends here.
+// last block.  solo_tiles: the tiles of an engine of one problem, else 0.  summary: 1: the iteration ends here (WHILE
+// handle h if use_handle), 2: the start of a solve ends here.
 enum FineKind { FINE_NORM_B = 0, FINE_OUTER, FINE_UPDATE, FINE_PCG_Q, FINE_PCG_X, FINE_PCG_DOT, FINE_PCG_P };
 cudaError_t launch_fine(const EngineDev& E, const GroupSize& size, int kind, int solo_tiles, int summary, cudaGraphConditionalHandle h,
                         int use_handle, cudaStream_t s);

@@ -289,8 +289,8 @@ __device__ __forceinline__ void fine_links(const EngineDev& E, int p, int a, int
   }
 }
 
-// summary: 1: (an engine of one problem) the last block, or block 0 where there is nothing to do, also ends
-// the iteration (2: only counts it: the start of a solve).
+// summary: 1: the last block (of an engine of one problem with nothing to do: block 0) also ends the iteration
+// (2: only counts it: the start of a solve).
 enum FineForm { SOLO_TILES, SOLO_LINKS, GROUPS };   // (links: where the sum has more than kSumGroup tiles)
 template <int OP, class V, int FORM>
 __global__ void __launch_bounds__(kFineThreads, OP == F_OUTER || OP == F_PCG_Q ? 3 : 4)
@@ -347,6 +347,8 @@ __global__ void __launch_bounds__(kFineThreads, OP == F_OUTER || OP == F_PCG_Q ?
       if (E.P[p].L >= HN_MIN_LEVEL && fine_serves(OP, st, pcg))
         control_apply(E, st, fine_control(OP), fine_sums(OP) ? __ldcg(E.gsum + (long long)p * E.ctl_groups) : 0.0);
     }
+    __syncthreads();
+    if (summary) summary_apply(E, h, use_handle, summary == 1, sh);
   }
 }
 
