@@ -1384,6 +1384,10 @@ int Engine::kernel_times(hn_kernel_time* out, int max) const {
 }
 
 hn_status Engine::read_states(std::vector<ProbState>& out) {
+  if (E_.states_host) {                            // there since finish_iteration
+    out.assign(host_states(), host_states() + cap_);
+    return HN_OK;
+  }
   out.resize(cap_);
   HN_CUDA(cudaMemcpyAsync(out.data(), dS_, sizeof(ProbState) * cap_, cudaMemcpyDeviceToHost, s_));
   HN_CUDA(cudaStreamSynchronize(s_));

@@ -275,6 +275,7 @@ class Engine {
     topMaskAll_ = true;
     groupSize_ = GroupSize{};
     groupSize_.problems[Lmax_] = cap_;
+    E_.states_host = reinterpret_cast<ProbState*>(dActive_ + 128);   // (no copy and second wait an iteration)
     drop_graphs();
   }
   int kernel_times(hn_kernel_time* out, int max) const;

@@ -200,6 +200,7 @@ struct EngineDev {
   int pad;
   Params prm;
   unsigned int* active_host;   // mapped host word: problems not done after the iteration
+  ProbState* states_host;      // mapped host memory: every problem's state after the iteration (or null)
   unsigned int* iter;          // iterations since the solve started (device)
   unsigned int iter_limit;     // beyond it every running problem stops as not converged
   int pdl;                     // launch with programmatic dependent launch (host-side flag)

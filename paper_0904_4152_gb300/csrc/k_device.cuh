@@ -795,6 +795,7 @@ __device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, 
     if (st.phase != PH_DONE && over) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
     // after an iteration the finest-level iterate of a running cycle is no longer zero
     if (end_of_iteration && (st.phase == PH_INNER || st.phase == PH_CYCLE)) st.zero_top = 0;
+    if (E.states_host) E.states_host[p] = st;
     c += st.phase != PH_DONE ? 1.0 : 0.0;
     o += st.phase == PH_OUTER ? 1.0 : 0.0;
   }
