@@ -822,7 +822,7 @@ __device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, 
 // what `on` looks at must not change before every block has listed.
 constexpr int kListMax = 1024;
 struct Served {
-  unsigned short slot[kListMax];
+  int slot[kListMax];                    // (a batch may have any number of problems)
   unsigned char level[kListMax];
   int start[kListMax + 1];
   int count[32];
@@ -854,7 +854,7 @@ __device__ int list_served(const EngineDev& E, Served& q, int base, int level, F
     const unsigned m = __ballot_sync(kFull, on);
     if (on) {
       const int i = at + __popc(m & ((1u << lane) - 1u)), p = base + lo + k * 32 + lane;
-      q.slot[i] = (unsigned short)p;
+      q.slot[i] = p;
       q.level[i] = (unsigned char)(level ? level : E.P[p].L);
     }
     at += __popc(m);
