@@ -10,13 +10,11 @@
  * when they fit) or are read through L2.  The best split depends on the levels and the batch;
  * hn_mg_autotune measures candidates on the hierarchy itself.
  *
- * A hierarchy whose shape was not set by hn_mg_set_tuning (the default, or an autotuned shape with
- * sweep 1 and mid 0) runs the larger levels of an FP32 / FP16 V(2,2) cycle, alone, in batches and in the
- * server, as marching sweeps: one pass over the level each way, above a one-block tail (tail_level <= 5);
- * problems of level 6..8 alone run their inner solves in one launch of 16 blocks.  FP64 V(2,2) cycles alone
- * and in batches of up to 31 run the levels to tail_level (5 or 6, cluster 16) so, with all cycles in one launch
- * where the finest level is among them, and those from 9 as one launch per step.  hn_mg_set_tuning selects
- * exactly the forms described below.
+ * The default shape runs V(2,2) cycles in the forms measured to be best (sweep -1): the larger levels of an FP32 /
+ * FP16 hierarchy, alone, in batches and in the server, as marching sweeps, one pass over the level each way, above a
+ * one-block tail (tail_level <= 5); problems of level 6..8 alone run their inner solves in one launch of 16 blocks.
+ * FP64 cycles alone and in batches of up to 31 run the levels to tail_level (5 or 6, cluster 16) so, with all cycles in
+ * one launch where the finest level is among them, and those from 9 as one launch per step.
  */
 #ifndef HN_TUNE_H
 #define HN_TUNE_H
@@ -47,7 +45,8 @@ typedef struct {
                        <= tail_level: none); not combined with staged or fuse_up, which are forms
                        of the per-step launches (default 0: on this part a grid barrier plus the
                        memory latency of a step costs as much as a kernel boundary) */
-  int sweep;        /* 1 (default): a hierarchy solved alone with V(2,2) cycles runs the down
+  int sweep;        /* -1 (default): each level in the form measured to be best for it (above); where
+                       none of these applies, as 1.  1: a hierarchy solved alone with V(2,2) cycles runs the down
                        part of each level between tail_level and the finest, up to level 9 (both
                        pre-smoothing steps, the defect and the restriction), and the up part (the
                        prolongation and both post-smoothing steps) as one launch each, over 2-D
@@ -55,8 +54,7 @@ typedef struct {
                        another; 2: every level above tail_level and, on the finest level, the steps
                        after the first smoothing step (the second step, the defect, the
                        restriction) in one launch; 0: one launch per step.  Not combined with
-                       staged or mid; 1 and 2 are for a hierarchy solved alone (in batches and in the
-                       server, without a set shape, 1 stands for the marching sweeps) */
+                       staged or mid; 1 and 2 are for a hierarchy solved alone */
 } hn_tuning;
 
 /* Set / read the launch shape used by mg's later solves.  HN_ERR_ARG on values out of range. */
@@ -64,15 +62,16 @@ hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t);
 hn_status hn_mg_get_tuning(const hn_mg* mg, hn_tuning* t);
 
 /* Time `reps` solves of b (host vector, N doubles) for every candidate shape (three forms of the
- * levels above the tail: one launch per step (mid 0, sweep 0), persistent kernels (mid 10), fused
- * sweeps (sweep 1); tail_level from coarse_L to min(L, 9); cluster 1..16) and keep the fastest; the
+ * levels above the tail: one launch per step (mid 0, sweep 0), persistent kernels (mid 10), each
+ * level's best (sweep -1); tail_level from coarse_L to min(L, 9); cluster 1..16) and keep the fastest; the
  * candidate timings are returned in `times_ms` (may be NULL, capacity `cap` entries, row-major
- * 3 forms x tail_level x 5 cluster sizes) and the chosen shape in *best.  The solution is unchanged
- * by the shape. */
+ * 3 forms x tail_level x 5 cluster sizes; shapes that run the same kernels are timed once) and the
+ * chosen shape in *best, which hn_mg_set_tuning gives to any hierarchy.  The solution is unchanged by
+ * the shape. */
 hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, double* times_ms,
                          int cap);
 
-/* The same for a batch (hn_mg_solve_batch over mgs[0..count)): candidates mid 0 and 10,
+/* The same for a batch (hn_mg_solve_batch over mgs[0..count)): candidates mid 0 (sweep -1) and 10,
  * tail_level coarse_L..8, cluster 1, 2, 4; the fastest shape is stored in every member and used by
  * later batch solves of the same members (a batch whose members carry no common tuned shape picks
  * one by its size). */

@@ -164,9 +164,7 @@ void fill_stats(const hn_mg* mg, const ProbState& st, long long t0, hn_mg_stats*
   out->solve_ns = now_ns() - t0;
 }
 
-// march: whether the shape may run its levels as marching sweeps (Tuning::march)
-hn_status set_shape(hn_mg* mg, const hn_tuning* t, int march) {
-  clear_error();
+hn_status set_shape(hn_mg* mg, const hn_tuning* t) {
   if (!mg || !t) return set_error(HN_ERR_ARG, "null argument");
   const int c = t->cluster;
   if (t->tail_level < mg->coarse || t->tail_level > HN_MAX_LEVEL || !(c == 1 || c == 2 || c == 4 || c == 8 || c == 16))
@@ -177,7 +175,7 @@ hn_status set_shape(hn_mg* mg, const hn_tuning* t, int march) {
   if (t->dsm != 0 && t->dsm != 1) return set_error(HN_ERR_ARG, "dsm must be 0 or 1");
   if (t->fuse_up != 0 && t->fuse_up != 1) return set_error(HN_ERR_ARG, "fuse_up must be 0 or 1");
   if (t->mid < 0 || t->mid > HN_MAX_LEVEL) return set_error(HN_ERR_ARG, "mid must be in [0, %d]", HN_MAX_LEVEL);
-  if (t->sweep < 0 || t->sweep > 2) return set_error(HN_ERR_ARG, "sweep must be 0, 1 or 2");
+  if (t->sweep < -1 || t->sweep > 2) return set_error(HN_ERR_ARG, "sweep must be -1, 0, 1 or 2");
   Tuning tu;
   tu.tail_level = t->tail_level;
   tu.cluster = c;
@@ -187,7 +185,6 @@ hn_status set_shape(hn_mg* mg, const hn_tuning* t, int march) {
   tu.fuse_up = t->fuse_up;
   tu.mid = t->mid;
   tu.sweep = t->sweep;
-  tu.march = march;
   mg->solo->set_tuning(tu);
   mg->tuning = tu;
   mg->tuned = true;
@@ -532,7 +529,10 @@ hn_status hn_mg_set_profiling(hn_mg* mg, int enable) {
   return HN_OK;
 }
 
-hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t) { return set_shape(mg, t, 0); }
+hn_status hn_mg_set_tuning(hn_mg* mg, const hn_tuning* t) {
+  clear_error();
+  return set_shape(mg, t);
+}
 
 hn_status hn_mg_get_tuning(const hn_mg* mg, hn_tuning* t) {
   clear_error();
@@ -559,8 +559,8 @@ hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, 
   HN_CUDA(cudaMallocHost(reinterpret_cast<void**>(&x), (size_t)N * 8));
   struct Free { double* p; ~Free() { cudaFreeHost(p); } } fr{x};
   const int clusters[5] = {1, 2, 4, 8, 16};
-  // the per-level forms: per-step launches, persistent kernels of the middle levels, fused sweeps
-  const int mids[3] = {0, kMidCandidate, 0}, sweeps[3] = {0, 0, 1};
+  // the per-level forms: per-step launches, persistent kernels of the middle levels, each level's own
+  const int mids[3] = {0, kMidCandidate, 0}, sweeps[3] = {0, 0, kSweepAuto};
   double best_ms = 1e300;
   const Tuning cur = mg->solo->tuning();
   hn_tuning bt{cur.tail_level, cur.cluster, 2, 0, 1, 0, cur.mid, cur.sweep};
@@ -569,11 +569,22 @@ hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, 
   HN_CUDA(cudaEventCreate(&e1));
   struct Ev { cudaEvent_t a, b; ~Ev() { cudaEventDestroy(a); cudaEventDestroy(b); } } ev{e0, e1};
   const int tmax = std::min(mg->L, 9);
+  // times of a form that no tail level to kSmallTop changes, of a tail that no cluster size changes
+  double same_tail = 0.0, same = 0.0;
   for (int mi = 0; mi < 3; ++mi)
   for (int T = mg->coarse; T <= tmax; ++T)
     for (int ci = 0; ci < 5; ++ci) {
+      if (ci == 0) same = 0.0;
+      if (ci == 0 && T == mg->coarse) same_tail = 0.0;
       hn_tuning t{T, clusters[ci], 2, 0, 1, 0, mids[mi], sweeps[mi]};
-      HN_TRY(set_shape(mg, &t, 1));
+      HN_TRY(set_shape(mg, &t));
+      const int idx = (mi * (tmax - mg->coarse + 1) + (T - mg->coarse)) * 5 + ci;
+      // (a shape that runs the kernels of one timed before: that one's time, which cannot be the best)
+      const double known = !mg->solo->uses_tail_level() ? same_tail : !mg->solo->uses_cluster() ? same : 0.0;
+      if (known > 0.0) {
+        if (times_ms && idx < cap) times_ms[idx] = known;
+        continue;
+      }
       HN_TRY(hn_mg_solve(mg, b, x, 0, 0, nullptr));            // capture + warm-up
       HN_CUDA(cudaEventRecord(e0, mg->solo->stream()));
       for (int r = 0; r < reps; ++r) {
@@ -584,12 +595,12 @@ hn_status hn_mg_autotune(hn_mg* mg, const double* b, int reps, hn_tuning* best, 
       HN_CUDA(cudaEventSynchronize(e1));
       float ms = 0.0f;
       HN_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      const double per = ms / reps;
-      const int idx = (mi * (tmax - mg->coarse + 1) + (T - mg->coarse)) * 5 + ci;
+      const double per = same = ms / reps;
+      if (!mg->solo->uses_tail_level()) same_tail = per;
       if (times_ms && idx < cap) times_ms[idx] = per;
       if (per < best_ms) { best_ms = per; bt = t; }
     }
-  HN_TRY(set_shape(mg, &bt, 1));
+  HN_TRY(set_shape(mg, &bt));
   if (best) *best = bt;
   if (const char* path = std::getenv("HN_TUNE_CACHE")) {
     char gpu[256];
@@ -616,16 +627,27 @@ hn_status hn_mg_autotune_batch(hn_mg* const* mgs, int count, const double* const
   for (int j = 0; j < count; ++j) Lmax = std::max(Lmax, mgs[j]->L);
   double best_ms = 1e300;
   const int mids[2] = {0, kMidCandidate};
-  hn_tuning bt{5, 1, 2, 0, 1, 0, mids[1], 0};
+  const int sweeps[2] = {kSweepAuto, 0};
+  hn_tuning bt{5, 1, 2, 0, 1, 0, mids[1], sweeps[1]};
+  auto give = [&](const hn_tuning& t) {
+    for (int j = 0; j < count; ++j) {
+      Tuning tu;
+      tu.tail_level = t.tail_level;
+      tu.cluster = t.cluster;
+      tu.pdl = t.pdl;
+      tu.mid = t.mid;
+      tu.sweep = t.sweep;
+      mgs[j]->tuning = tu;
+      mgs[j]->tuned = true;
+    }
+  };
   for (int mi = 0; mi < 2; ++mi)
   for (int T = mgs[0]->coarse; T <= std::min(Lmax, 8); ++T)
     for (int ci = 0; ci < 3; ++ci) {
-      hn_tuning t{T, clusters[ci], 2, 0, 1, 0, mids[mi], 0};
-      for (int j = 0; j < count; ++j) {
-        Tuning tu; tu.tail_level = T; tu.cluster = clusters[ci]; tu.pdl = 2; tu.mid = mids[mi];
-        mgs[j]->tuning = tu;
-        mgs[j]->tuned = true;
-      }
+      hn_tuning t{T, clusters[ci], 2, 0, 1, 0, mids[mi], sweeps[mi]};
+      if (ci > 0 && sweeps[mi] == kSweepAuto && T <= kSmallTop && mgs[0]->prm.prec != P64 && fused_options(mgs[0]->prm))
+        continue;                             // (the one-block tail: no cluster size changes it)
+      give(t);
       HN_TRY(hn_mg_solve_batch(mgs, count, b, xs.data(), 0, nullptr));   // capture + warm-up
       const long long t0 = now_ns();
       for (int r = 0; r < reps; ++r) {
@@ -635,11 +657,7 @@ hn_status hn_mg_autotune_batch(hn_mg* const* mgs, int count, const double* const
       const double ms = (now_ns() - t0) * 1e-6 / reps;
       if (ms < best_ms) { best_ms = ms; bt = t; }
     }
-  for (int j = 0; j < count; ++j) {
-    Tuning tu; tu.tail_level = bt.tail_level; tu.cluster = bt.cluster; tu.pdl = bt.pdl; tu.mid = bt.mid;
-    mgs[j]->tuning = tu;
-    mgs[j]->tuned = true;
-  }
+  give(bt);
   {
     std::lock_guard<std::mutex> lk(g_batch_mu);
     g_batch_engine.reset();

@@ -912,7 +912,7 @@ bool Engine::sweep_level(int l) const {
 // solve with level 9 marching or not: 1.490 / 1.518 ms).
 bool Engine::march_level(int l) const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
-  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !tune_.staged &&
+  return tune_.sweep == kSweepAuto && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !tune_.staged &&
          !tune_.fuse_up && mid_top() <= T && l >= (cap_ == 1 ? kMarchSoloLevel : kMarchMinLevel) &&
          (cap_ == 1 || T + 1 >= kMarchMinLevel);
 }
@@ -920,7 +920,7 @@ bool Engine::march_level(int l) const {
 // The levels of the tail in one block's shared memory (k_small) in place of the cluster kernel, under the
 // conditions of the marching sweeps and with the exact coarse solver.
 bool Engine::small_tail() const {
-  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
+  return tune_.sweep == kSweepAuto && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
          !tune_.staged && !tune_.fuse_up && std::max(tune_.tail_level, prm_.coarse) <= kSmallTop;
 }
 
@@ -930,7 +930,7 @@ bool Engine::small_tail() const {
 // against 1494 us (from level 7 967 / 1435, from level 6 964 / 1407 us).
 bool Engine::span_tail() const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
-  return tune_.march && tune_.sweep == 1 && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
+  return tune_.sweep == kSweepAuto && prm_.prec != P64 && prm_.pre == 2 && prm_.post == 2 && !prm_.coarse_cg &&
          !tune_.staged && !tune_.fuse_up && tune_.mid <= T && T <= kSmallTop && small_.L == Lmax_ &&
          Lmax_ > kSmallTop && Lmax_ <= kSpanTop;   // (small_: an engine of one problem; a server's may be of a lower level)
 }
@@ -941,14 +941,14 @@ int Engine::tail_top() const { return span_tail() ? kSpanTop : std::max(tune_.ta
 // An FP64 problem alone: level l's steps as launches of k_level64 (which has the measurements).
 constexpr int kLevel64Min = 9;
 bool Engine::level64(int l) const {
-  return tune_.march && tune_.sweep == 1 && cap_ == 1 && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
+  return tune_.sweep == kSweepAuto && cap_ == 1 && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
          mid_top() <= std::max(tune_.tail_level, prm_.coarse) && l >= kLevel64Min;
 }
 
 // The FP64 counterpart over a cluster of 16 blocks (k_wide).
 bool Engine::wide_tail() const {
   const int T = std::max(tune_.tail_level, prm_.coarse);
-  return tune_.march && tune_.sweep == 1 && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
+  return tune_.sweep == kSweepAuto && wide_options(prm_) && !tune_.staged && !tune_.fuse_up &&
          tune_.cluster == 16 && T > 4 && T <= kWideTop;
 }
 

@@ -76,6 +76,7 @@ enum KClass {
 // launch shape of the schedule: levels <= tail_level run fused in one cluster launch of
 // `cluster` blocks per problem; levels above run as one launch per step
 constexpr int kSweepMaxLevel = 9;   // largest level in fused sweeps under tuning sweep 1
+constexpr int kSweepAuto = -1;      // tuning sweep: each level as the form that is best for it
 
 struct Tuning {
   int tail_level = 7;
@@ -91,20 +92,21 @@ struct Tuning {
                     // kernels (default: a grid barrier plus the memory latency of a step measured
                     // as long as a kernel boundary, ~3.5 us at L = 10, so they did not pay).
                     // Not combined with staged or fuse_up, which are per-step forms.
-  int sweep = 1;    // an engine of one problem with V(2,2) cycles: the down part of each level
+  int sweep = kSweepAuto;
+                    // kSweepAuto (-1), V(2,2) cycles: FP32 / FP16 levels from kMarchMinLevel above the
+                    // tail as marching sweeps (k_march.cu), also in batches and in the server, the
+                    // one-block and cluster tails (k_small, k_wide, k_span) and FP64 levels by
+                    // k_level64 where these apply; elsewhere as 1.
+                    // 1: an engine of one problem with V(2,2) cycles: the down part of each level
                     // between the tail and the finest, up to kSweepMaxLevel (smoothing, defect,
                     // restriction), and the up part (prolongation, smoothing) as one launch each
                     // over 2-D tiles with recomputed halos (k_sweep_down / k_sweep_up); 2: every
                     // level above the tail, with the finest level's steps after its first smoothing
-                    // step.  Default 1 (measured at L = 9 / 10 / 12: FP32-inner DC -3.6 / -1.0 /
+                    // step.  (1 against 0, measured at L = 9 / 10 / 12: FP32-inner DC -3.6 / -1.0 /
                     // -0.4 %, FP64 MG -11.5 / -2.3 / -0.3 %); 2 was slower from L = 10 up.
-  int march = 1;    // FP32 / FP16 hierarchies with V(2,2) cycles, sweep on: the levels from
-                    // kMarchMinLevel above the tail run as marching sweeps (k_march.cu), also in
-                    // batches and in the server.  A shape set by hn_mg_set_tuning has it off (the
-                    // forms hn_tune.h describes, as they are); not part of hn_tuning.
   bool operator==(const Tuning& o) const {
     return tail_level == o.tail_level && cluster == o.cluster && pdl == o.pdl && staged == o.staged && dsm == o.dsm &&
-           fuse_up == o.fuse_up && mid == o.mid && sweep == o.sweep && march == o.march;
+           fuse_up == o.fuse_up && mid == o.mid && sweep == o.sweep;
   }
 };
 
@@ -135,33 +137,33 @@ inline bool fused_options(const Params& prm) { return prm.pre == 2 && prm.post =
 inline bool wide_options(const Params& prm) { return prm.prec == P64 && fused_options(prm); }
 inline Tuning group_tuning(const Params& prm, const GroupSize& size, bool any_level) {
   Tuning t;
-  auto shape = [&](int tail_level, int cluster, int march) {
+  auto shape = [&](int tail_level, int cluster, bool march) {
     t.tail_level = tail_level;
     t.cluster = cluster;
-    t.march = march;
+    t.sweep = march ? kSweepAuto : 0;
     return t;
   };
   const long long slots = size.sum([](int) { return 1; });
   int Lmax = 0;
   for (int l = 0; l <= kMaxLevel; ++l)
     if (size.problems[l]) Lmax = l;
-  if (slots >= 32) return shape(kSmallTop, 1, 1);
+  if (slots >= 32) return shape(kSmallTop, 1, true);
   if (!fused_options(prm)) {
     if (any_level) return t;
     if (slots < 8) return shape(7, 16, Lmax >= 10);
-    return prm.pre == 2 && prm.post == 2 && Lmax >= 9 ? shape(kSmallTop, 1, 1) : shape(6, 4, 0);
+    return prm.pre == 2 && prm.post == 2 && Lmax >= 9 ? shape(kSmallTop, 1, true) : shape(6, 4, false);
   }
-  if (prm.prec == P64) return shape(kWideTop, 16, 1);
+  if (prm.prec == P64) return shape(kWideTop, 16, true);
   const bool half = prm.prec == P16;
-  if (any_level) return slots < 16 && Lmax <= 9 ? shape(8, 16, 1) : shape(kSmallTop, 1, 1);
-  if (slots < 8 && Lmax > kSmallTop && Lmax <= (prm.solver == SOLVER_PCG ? 7 : 8)) return shape(8, 16, 1);
+  if (any_level) return slots < 16 && Lmax <= 9 ? shape(8, 16, true) : shape(kSmallTop, 1, true);
+  if (slots < 8 && Lmax > kSmallTop && Lmax <= (prm.solver == SOLVER_PCG ? 7 : 8)) return shape(8, 16, true);
   if (prm.solver != SOLVER_PCG && slots > 0) {
     const double fill = (double)size.sum([](int l) { return N_of(l); }) / ((double)slots * (double)N_of(Lmax));
-    if (Lmax == 9 && fill >= 0.5 && slots < (half ? 8 : 5)) return shape(7, 16, 0);
-    if (Lmax == 9 && fill < 0.5 && slots < 5) return shape(8, 16, 1);
-    if (Lmax > kSmallTop && Lmax <= 8 && slots < (half ? 32 : 12) && (half ? Lmax <= 7 || fill >= 0.6 : fill >= 0.8)) return shape(6, 4, 0);
+    if (Lmax == 9 && fill >= 0.5 && slots < (half ? 8 : 5)) return shape(7, 16, false);
+    if (Lmax == 9 && fill < 0.5 && slots < 5) return shape(8, 16, true);
+    if (Lmax > kSmallTop && Lmax <= 8 && slots < (half ? 32 : 12) && (half ? Lmax <= 7 || fill >= 0.6 : fill >= 0.8)) return shape(6, 4, false);
   }
-  return shape(kSmallTop, 1, 1);
+  return shape(kSmallTop, 1, true);
 }
 
 class Engine;
@@ -269,6 +271,9 @@ class Engine {
     tune_ = t; E_.pdl = t.pdl; E_.staged = t.staged; E_.dsm = t.dsm; drop_graphs();
   }
   const Tuning& tuning() const { return tune_; }
+  // whether the shape's cluster size, or its tail level among those to kSmallTop, changes the kernels that run
+  bool uses_cluster() const { return !span_tail() && !small_tail(); }
+  bool uses_tail_level() const { return !span_tail(); }
   // levels that may be some problem's finest level (their first smoothing step may start from a
   // nonzero iterate); all levels for the server
   void set_top_mask_all() {

@@ -404,7 +404,7 @@ def hn_mg_autotune(mg, b, reps=3, coarse_L=2):
     _check(lib().hn_mg_autotune(mg, _host_ptr(b, np.float64), reps, ctypes.byref(best),
                                 times.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), cap))
     clusters = (1, 2, 4, 8, 16)
-    modes = ((0, 0), (10, 0), (0, 1))                        # (mid, sweep) of the three forms
+    modes = ((0, 0), (10, 0), (0, -1))                       # (mid, sweep) of the three forms
     rows = int(np.count_nonzero(~np.isnan(times))) // 15     # tail levels per form
     table = {}
     for i, v in enumerate(times):
