@@ -41,7 +41,7 @@ hn_status device_error(const Engine& e) {
   switch (d[0]) {
     case 0: return HN_OK;
     case 3: return set_error(HN_ERR_CUDA, "a grid barrier of the persistent kernels timed out");
-    case 5: return set_error(HN_ERR_STATE, "debug check failed (k_cycle.cu line %d, indices %d, %d)", d[1], d[2], d[3]);
+    case 5: return set_error(HN_ERR_STATE, "debug check failed (%s line %d, indices %d, %d)", source_name(d[1]), d[1] & 0xffff, d[2], d[3]);
     default: return set_error(HN_ERR_CUDA, "a bounded device wait for a bulk copy gave up");
   }
 }

@@ -346,6 +346,12 @@ enum ControlKind {
 };
 
 int sm_count();
+// the source file of a failed index check (debug builds), from the upper 16 bits of its recorded place
+inline const char* source_name(int place) {
+  static const char* const names[] = {"k_cycle.cu", "k_march.cu", "k_fine.cu"};
+  const unsigned i = (unsigned)place >> 16;
+  return i < sizeof names / sizeof *names ? names[i] : "?";
+}
 // Whether a launch of `blocks` blocks is a programmatic dependent one under the tuning's rule (hn_tuning.pdl): 1: every
 // launch; 2: launches of fewer blocks than SMs (their waiting blocks take no occupancy from a kernel that still runs,
 // of this stream or of another); 3: fewer blocks than twice the SMs.

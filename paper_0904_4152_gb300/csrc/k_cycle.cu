@@ -17,6 +17,7 @@
 #include <unordered_map>
 #include <cooperative_groups.h>
 
+#define HN_SOURCE 0
 #include "k_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -554,7 +555,7 @@ __global__ void __launch_bounds__(256, band_min_blocks<Pol, MODE>()) k_band(Engi
   if (tl.solo_tiles > 0 && level >= 0) {          // one problem: descriptors by value
     const ProbState& st = E.S[0];
     if (st.phase != want) return;
-    if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
+    if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, HN_HERE)) return;
     if constexpr (MODE == M_PJ) {
       if (tl.solo_c.n == 0) return;               // (no coarser level: nothing to prolong)
       for (int t = gw; t < tl.solo_tiles; t += nw)
@@ -582,7 +583,7 @@ __global__ void __launch_bounds__(256, band_min_blocks<Pol, MODE>()) k_band(Engi
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, level, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, level, HN_HERE)) continue;
     const ProbState& st = E.S[p];
     if (st.phase != want) continue;
     const ProblemDev& P = E.P[p];
@@ -712,8 +713,8 @@ __global__ void __launch_bounds__(256) k_restrict(EngineDev E, TileList tl, int 
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   if (tl.solo_tiles > 0) {                        // one problem: tl is the coarse level's list
     if (tl.solo_L < fine_level || E.S[0].phase != want) return;   // (no finer level: no descriptor)
-    if (!dbg_level(E, tl.solo_d, fine_level - 1, tl.solo_tiles, __LINE__) ||
-        !dbg_level(E, tl.solo_f, fine_level, 0, __LINE__)) return;
+    if (!dbg_level(E, tl.solo_d, fine_level - 1, tl.solo_tiles, HN_HERE) ||
+        !dbg_level(E, tl.solo_f, fine_level, 0, HN_HERE)) return;
     for (int t = gw; t < tl.solo_tiles; t += nw)
       restrict_tile<V, LD_NC>(tl.solo_f, tl.solo_d, (long long)t * kTile, lane);
     return;
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(256) k_restrict(EngineDev E, TileList tl, int 
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, fine_level - 1, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, fine_level - 1, HN_HERE)) continue;
     const ProblemDev& P = E.P[p];
     if (P.L < fine_level || E.S[p].phase != want) continue;
     restrict_tile<V, LD_NC>(P.lev[fine_level], P.lev[fine_level - 1], (long long)it.y * kTile, lane);
@@ -738,8 +739,8 @@ __global__ void __launch_bounds__(256) k_prolong(EngineDev E, TileList tl, int l
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   if (tl.solo_tiles > 0) {                        // one problem: descriptors by value
     if (tl.solo_c.n == 0 || E.S[0].phase != want) return;   // (no coarser level: nothing to add)
-    if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__) ||
-        !dbg_level(E, tl.solo_c, level - 1, 0, __LINE__)) return;
+    if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, HN_HERE) ||
+        !dbg_level(E, tl.solo_c, level - 1, 0, HN_HERE)) return;
     for (int t = gw; t < tl.solo_tiles; t += nw)
       prolong_tile<V, LD_NC>(tl.solo_d, tl.solo_c, x_sel, (long long)t * kTile + lane * kLaneNodes);
     return;
@@ -748,7 +749,7 @@ __global__ void __launch_bounds__(256) k_prolong(EngineDev E, TileList tl, int l
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, level, __LINE__) || !dbg_item(E, p, 0, level - 1, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, level, HN_HERE) || !dbg_item(E, p, 0, level - 1, HN_HERE)) continue;
     if (E.S[p].phase != want) continue;
     const ProblemDev& P = E.P[p];
     prolong_tile<V, LD_NC>(P.lev[level], P.lev[level - 1], x_sel,
@@ -1719,8 +1720,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_sweep_down(EngineDev E, TileL
   const LevelDev& g = tl.solo_d;
   const LevelDev& gc = tl.solo_c;
   if (tl.solo_tiles == 0 || gc.n == 0) return;    // (a level the problem does not have, or no coarser)
-  if (!dbg_level(E, g, level, tl.solo_tiles, __LINE__) || !dbg_level(E, gc, level - 1, 0, __LINE__) ||
-      !sweep_geom_ok(E, sg, gc.n, __LINE__))
+  if (!dbg_level(E, g, level, tl.solo_tiles, HN_HERE) || !dbg_level(E, gc, level - 1, 0, HN_HERE) ||
+      !sweep_geom_ok(E, sg, gc.n, HN_HERE))
     return;
   // below the problem's own finest level the iterate starts at zero whatever the launch says (an
   // engine whose graphs serve any member level launches every level as a possible top)
@@ -1808,8 +1809,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_sweep_up(EngineDev E, TileLis
   const LevelDev& g = tl.solo_d;
   const LevelDev& gc = tl.solo_c;
   if (tl.solo_tiles == 0 || gc.n == 0) return;
-  if (!dbg_level(E, g, level, tl.solo_tiles, __LINE__) || !dbg_level(E, gc, level - 1, 0, __LINE__) ||
-      !sweep_geom_ok(E, sg, gc.n, __LINE__))
+  if (!dbg_level(E, g, level, tl.solo_tiles, HN_HERE) || !dbg_level(E, gc, level - 1, 0, HN_HERE) ||
+      !sweep_geom_ok(E, sg, gc.n, HN_HERE))
     return;
   LevelDev t;
   V* es;
@@ -1987,7 +1988,7 @@ __device__ void mid_solo_load(const EngineDev& E, const TileList* lists, int M, 
   __syncthreads();
   if (threadIdx.x == 0 && ms.on)
     for (int l = T; l <= M; ++l)
-      if (!dbg_level(E, ms.lev[l], l, (int)(ms.lev[l].pitch / kTile), __LINE__)) ms.in_phase = 0;
+      if (!dbg_level(E, ms.lev[l], l, (int)(ms.lev[l].pitch / kTile), HN_HERE)) ms.in_phase = 0;
   __syncthreads();
 }
 
@@ -2013,7 +2014,7 @@ __device__ __forceinline__ void mid_band_pass(const EngineDev& E, const MidSolo&
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, l, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, l, HN_HERE)) continue;
     const ProbState& st = E.S[p];
     if (__ldcg(&st.phase) != want) continue;
     const ProblemDev& P = E.P[p];
@@ -2041,7 +2042,7 @@ __device__ __forceinline__ void mid_restrict_pass(const EngineDev& E, const MidS
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, l - 1, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, l - 1, HN_HERE)) continue;
     const ProblemDev& P = E.P[p];
     if (P.L < l || __ldcg(&E.S[p].phase) != want) continue;
     restrict_tile<V, LD_CG>(P.lev[l], P.lev[l - 1], (long long)it.y * kTile, lane);
@@ -2063,7 +2064,7 @@ __device__ __forceinline__ void mid_prolong_pass(const EngineDev& E, const MidSo
   for (int g = gw; g < count; g += nw) {
     const int2 it = tl.items[g];
     const int p = it.x;
-    if (!dbg_item(E, p, it.y, l, __LINE__) || !dbg_item(E, p, 0, l - 1, __LINE__)) continue;
+    if (!dbg_item(E, p, it.y, l, HN_HERE) || !dbg_item(E, p, 0, l - 1, HN_HERE)) continue;
     if (__ldcg(&E.S[p].phase) != want) continue;
     const ProblemDev& P = E.P[p];
     prolong_tile<V, LD_CG>(P.lev[l], P.lev[l - 1], x_sel, (long long)it.y * kTile + lane * kLaneNodes);

@@ -37,6 +37,8 @@ __device__ __forceinline__ void pdl_start() {
 #ifndef HN_DEBUG_CHECKS
 #define HN_DEBUG_CHECKS 0
 #endif
+// (a file with checks defines HN_SOURCE, its place among source_name's)
+#define HN_HERE (HN_SOURCE << 16 | __LINE__)
 __device__ __forceinline__ void dbg_fail(const EngineDev& E, int line, int a, int b) {
   if (atomicCAS(E.err, 0, 5) == 0) {
     E.err[1] = line;

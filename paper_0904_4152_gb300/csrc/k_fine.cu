@@ -21,6 +21,7 @@
 // measured 1414 us at L = 10, two 7000 us at L = 12.
 #include <algorithm>
 
+#define HN_SOURCE 2
 #include "k_device.cuh"
 
 namespace hn {
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kFineThreads, OP == F_OUTER || OP == F_PCG_Q ?
       const int lo = (int)(blk * all / G), hi = (int)((blk + 1) * all / G);     // the block's run of tiles
       for (int m = hi > lo ? served_of(q, n, lo) : n; m < n && q.start[m] < hi; ++m) {
         const int p = q.slot[m], tiles = fine_tiles(q.level[m]);
-        if (!dbg_item(E, p, 0, -1, __LINE__)) continue;
+        if (!dbg_item(E, p, 0, -1, HN_HERE)) continue;
         const int a = max(0, lo - q.start[m]), b = min(tiles, hi - q.start[m]);
         if (fine_sums(OP) && tiles > kSumGroup) {   // (a link belongs to the block that has its first tile)
           fine_links<OP, V>(E, p, (a + kLink - 1) / kLink, (b + kLink - 1) / kLink, 1, pcg);
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(kFineThreads, 3)
   if (tl.solo_d.n == 0) return;
   const ProbState& st = E.S[0];
   if (st.phase != want) return;
-  if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) return;
+  if (!dbg_level(E, tl.solo_d, level, tl.solo_tiles, HN_HERE)) return;
   const LevelDev& d = tl.solo_d;
   const bool zero = OP == LV_FIRST && (tl.solo_L > level || st.zero_top);
   const bool summed = OP == LV_FIRST && tl.solo_L == level && !zero;

@@ -30,6 +30,7 @@
 // the same bits.
 #include <algorithm>
 
+#define HN_SOURCE 1
 #include "k_device.cuh"
 
 namespace hn {
@@ -635,7 +636,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march(EngineDev E, TileList 
   // the coarsest level, or one that the problem does not have (a server's engine of one slot may be built for a
   // larger one): nothing to do, but the launch must not end before the one it follows, which the next one's wait
   // would then no longer cover
-  if (tl.solo_c.n == 0 || !dbg_level(E, tl.solo_d, level, tl.solo_tiles, __LINE__)) {
+  if (tl.solo_c.n == 0 || !dbg_level(E, tl.solo_d, level, tl.solo_tiles, HN_HERE)) {
     pdl_wait();
     return;
   }
@@ -712,7 +713,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_march_group(EngineDev E, int
     const int items = number_items(q, n, [&](int l) { return cut[l].x * ((cut[l].y + rows - 1) / rows); });
     for (int it = gw; it < items; it += G) {
       const int m = served_of(q, n, it), p = q.slot[m], l = q.level[m];
-      if (!dbg_item(E, p, 0, l, __LINE__)) continue;
+      if (!dbg_item(E, p, 0, l, HN_HERE)) continue;
       const ProblemDev& P = E.P[p];
       const bool zero = P.L > l || E.S[p].zero_top;
       make_view<Pol, UPWARD>(v, P.lev[l], P.lev[l - 1], 0, scale[warp], E.prm.solver != SOLVER_PCG);
@@ -831,7 +832,7 @@ __global__ void __launch_bounds__(256) k_march_check_group(EngineDev E, int T, i
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
       const int m = served_of(q, n, it), p = q.slot[m], l = q.level[m], blk = it - q.start[m];
       // (a problem leaves the phase only after every block of its check has counted itself in)
-      if (!dbg_item(E, p, 0, l, __LINE__) || __ldcg(&E.S[p].phase) != want) continue;
+      if (!dbg_item(E, p, 0, l, HN_HERE) || __ldcg(&E.S[p].phase) != want) continue;
       if (l <= T || E.S[p].zero_top) {            // no check (or the tail's own): the cycle goes on
         if (blk == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 0, 1u);
         continue;
