@@ -515,7 +515,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   fineCap_ = fine_cap;
   take(sizeof(double) * (size_t)std::max<long long>(fine_cap, 1));
   take(sizeof(unsigned));
-  take(sizeof(unsigned) * 4);
+  take(sizeof(unsigned));
   take(sizeof(unsigned long long));
   // the control kernel's groups: as many as the largest problem's norm sum has
   const int ctl_groups = (int)((pitch_of(Lmax) / kTile + kSumGroup - 1) / kSumGroup);
@@ -542,7 +542,7 @@ hn_status Engine::create(const Params& prm, int cap, int Lmax, const std::vector
   dErr_ = b.take<int>(4);
   double* part = b.take<double>((size_t)std::max<long long>(fine_cap, 1));
   unsigned* iter = b.take<unsigned>(1);
-  dTaken_ = b.take<unsigned>(4);
+  dTaken_ = b.take<unsigned>(1);
   dLaunches_ = b.take<unsigned long long>(1);
   double* gsum = b.take<double>((size_t)cap * ctl_groups);
   unsigned* gticket = b.take<unsigned>((size_t)cap * ticket_words(ctl_groups));
@@ -852,7 +852,7 @@ hn_status Engine::mark(cudaStream_t s, int cls, int level, bool begin) {
     ++counting_;                                    \
   } while (0)
 
-hn_status Engine::open_if(cudaStream_t& s, int which) {
+hn_status Engine::open_if(cudaStream_t& s) {
   cudaStreamCaptureStatus cst;
   cudaGraph_t g = nullptr;
   const cudaGraphNode_t* deps = nullptr;
@@ -862,8 +862,7 @@ hn_status Engine::open_if(cudaStream_t& s, int which) {
   if (cst != cudaStreamCaptureStatusActive) return set_error(HN_ERR_STATE, "IF node outside a capture");
   cudaGraphNodeParams cp = {};
   cp.type = cudaGraphNodeTypeConditional;
-  const CondDev& cdv = E_.prm.cond;               // the handles of the half being captured
-  cp.conditional.handle = which == 0 ? cdv.h_cycle : (which == 1 ? cdv.h_outer : cdv.h_update);
+  cp.conditional.handle = E_.prm.cond.cycle;      // of the half being captured
   cp.conditional.type = cudaGraphCondTypeIf;
   cp.conditional.size = 1;
   cudaGraphNode_t node;
@@ -960,8 +959,8 @@ hn_status Engine::issue_vcycle(cudaStream_t s0, int want) {
   int c0 = 0;
   // inside the closed-world loop the rest of the cycle after the first lagged check is an IF body
   auto after_check = [&]() -> hn_status {
-    if (!cond_on(0) || opened) return HN_OK;
-    HN_TRY(open_if(s, 0));
+    if (!condCapture_ || opened) return HN_OK;
+    HN_TRY(open_if(s));
     opened = true;
     c0 = counting_;
     return HN_OK;
@@ -1096,7 +1095,7 @@ hn_status Engine::issue_iteration(cudaStream_t s0, cudaGraphConditionalHandle h,
   auto count_base = [&] {
     if (!condCapture_) return;
     const CondDev& cd = E_.prm.cond;
-    E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle - cd.n_outer - cd.n_update;
+    E_.prm.cond.n_base = (unsigned)(counting_ + 1 - start) - cd.n_cycle;
   };
   // the last vector step ends the iteration
   if (prm_.solver == SOLVER_PCG) {
@@ -1204,16 +1203,11 @@ hn_status Engine::capture_solve(bool cond) {
     // defect correction, where every outer step ends with one cycle that its check stops.  (The
     // outer defect and the update would each skip two small launches: not worth an IF node.)
     const int T = std::max(tail_top(), mid_top());
-    if (Lmax_ > T && prm_.prec != P64 && prm_.solver != SOLVER_PCG) cd.mask |= 1u;
-    const unsigned defaults[3] = {0u, 1u, 0u};
-    // two sets: the loop body holds two iterations, each with IF nodes of its own handles
-    for (int w = 0; w < 3; ++w)
-      if ((cd.mask >> w) & 1u)
-        for (int half = 0; half < 2; ++half)
-          HN_CUDA(cudaGraphConditionalHandleCreate(&hCond_[half][w], main, defaults[w], cudaGraphCondAssignDefault));
-    cd.h_cycle = hCond_[0][0];
-    cd.h_outer = hCond_[0][1];
-    cd.h_update = hCond_[0][2];
+    if (Lmax_ > T && prm_.prec != P64 && prm_.solver != SOLVER_PCG) cd.on = 1u;
+    // two: the loop body holds two iterations, each with an IF node of its own handle
+    for (int half = 0; half < 2 && cd.on; ++half)
+      HN_CUDA(cudaGraphConditionalHandleCreate(&hCond_[half], main, 0u, cudaGraphCondAssignDefault));
+    cd.cycle = hCond_[0];
     cd.taken = dTaken_;
     cd.launches = dLaunches_;
   }
@@ -1242,19 +1236,15 @@ hn_status Engine::capture_solve(bool cond) {
   // second one's sets it (a problem that finishes in the first runs the second as no-ops).  Each
   // turn of a device-side loop costs several microseconds; this halves their number.
   E_.prm.cond = cd;
-  condCapture_ = cd.mask != 0;
+  condCapture_ = cd.on != 0;
   counting_ = 0;
   st = issue_iteration(cs, h, 0);
   iterLaunches_ = counting_;
   if (st == HN_OK) {
     CondDev cd2 = cd;
-    cd2.h_cycle = hCond_[1][0];
-    cd2.h_outer = hCond_[1][1];
-    cd2.h_update = hCond_[1][2];
+    cd2.cycle = hCond_[1];
     cd2.n_base = E_.prm.cond.n_base;               // the counts of the first half (same shape)
     cd2.n_cycle = E_.prm.cond.n_cycle;
-    cd2.n_outer = E_.prm.cond.n_outer;
-    cd2.n_update = E_.prm.cond.n_update;
     E_.prm.cond = cd2;
     st = issue_iteration(cs, h, 1);
   }
@@ -1266,7 +1256,7 @@ hn_status Engine::capture_solve(bool cond) {
   HN_CUDA(cudaGraphInstantiate(&exec, main, 0));
   if (gSolve_) cudaGraphExecDestroy(gSolve_);
   gSolve_ = exec;
-  condUsed_ = cd.mask != 0;
+  condUsed_ = cd.on != 0;
   return HN_OK;
 }
 

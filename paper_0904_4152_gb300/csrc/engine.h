@@ -302,11 +302,10 @@ class Engine {
   hn_status issue_iteration(cudaStream_t s, cudaGraphConditionalHandle h, int use_h);
   hn_status issue_vcycle(cudaStream_t s, int want);
   // IF node at the current end of stream s's capture; further launches go to its body (on aux_)
-  hn_status open_if(cudaStream_t& s, int which);
+  hn_status open_if(cudaStream_t& s);
   hn_status close_if(cudaStream_t& s, cudaStream_t outer);
   hn_status capture_solve(bool cond);
   void clear_marks();
-  bool cond_on(int which) const { return condCapture_ && ((E_.prm.cond.mask >> which) & 1u); }
   int grid_for(long long tiles) const;
   hn_status mark(cudaStream_t s, int cls, int level, bool begin);
   void destroy_graphs();
@@ -371,7 +370,7 @@ class Engine {
   // IF nodes inside the closed-world loop (see CondDev)
   cudaStream_t aux_ = nullptr;
   bool condCapture_ = false, condUsed_ = false, pdlBarrier_ = false;
-  cudaGraphConditionalHandle hCond_[2][3] = {};   // IF handles of the two halves of the loop body
+  cudaGraphConditionalHandle hCond_[2] = {};      // IF handles of the two halves of the loop body
   unsigned* dTaken_ = nullptr;
   unsigned long long* dLaunches_ = nullptr;
   // profiling

@@ -127,20 +127,19 @@ struct ProbState {
   double beta;           // PCG: (r_new, z_new) / (r, z)
 };
 
-// solver parameters shared by every problem of an engine
-// IF nodes of the device-side solve loop (closed-world graph only).  One iteration of the loop
-// runs [IF outer: outer defect, control] [top-level first smoothing step, check] [IF cycle: rest
-// of the V cycle] [IF update: update, control] summary.  The kernel that takes a phase decision
-// sets the matching value (and its mirror in `taken`); the summary counts the launches the
-// iteration ran and resets the values for the next one.
+// The IF node of the device-side solve loop (closed-world graph only).  One iteration of the loop
+// runs outer defect, first smoothing step of the finest level, check, [IF: rest of the V cycle], update.  The kernel that
+// decides that a cycle goes on sets the value (and its mirror `taken`); the end of the iteration counts the
+// launches it ran and resets the value for the next one.
 struct CondDev {
-  unsigned long long h_cycle = 0, h_outer = 0, h_update = 0;   // cudaGraphConditionalHandle
-  unsigned* taken = nullptr;              // [0] cycle, [1] outer, [2] update
+  unsigned long long cycle = 0;           // cudaGraphConditionalHandle
+  unsigned* taken = nullptr;
   unsigned long long* launches = nullptr; // kernels launched by the loop's iterations
-  unsigned n_base = 0, n_cycle = 0, n_outer = 0, n_update = 0;
-  unsigned mask = 0;                      // handles that exist: bit w for taken[w]
+  unsigned n_base = 0, n_cycle = 0;       // launches outside the IF node, in it
+  unsigned on = 0;                        // the node exists
 };
 
+// solver parameters shared by every problem of an engine
 struct Params {
   int prec, pre, post, coarse;
   int max_cycles, max_outer, inner_max, solver;
@@ -339,7 +338,7 @@ cudaError_t launch_summary(const EngineDev& E, cudaGraphConditionalHandle h, int
                            int end_of_iteration, cudaStream_t s);
 
 enum ControlKind {
-  CTRL_INIT = 0, CTRL_CHECK = 1, CTRL_OUTER = 2, CTRL_POST = 4, CTRL_CHECK0 = 5,
+  CTRL_INIT = 0, CTRL_OUTER = 2, CTRL_POST = 4, CTRL_CHECK0 = 5,
   CTRL_PRE = 6,  // lagged convergence test after the first smoothing step of a cycle
   CTRL_PCG_ALPHA = 7,  // PCG: alpha = rho / (p, q)
   CTRL_PCG_BETA = 8    // PCG: rho' = (r, z), beta = rho' / rho

@@ -2250,11 +2250,11 @@ __global__ void __launch_bounds__(256) k_control(EngineDev E, int kind, int leve
     }
     // the rest of the V cycle runs if any problem is still in it
     if (owner && threadIdx.x == 0 && (st.phase == PH_INNER || st.phase == PH_CYCLE))
-      cond_set(E.prm.cond, 0, 1u);
+      cond_set(E.prm.cond, 1u);
     return;
   }
   // (the steps on the finest level's FP64 norms are taken by the kernels that form them, k_fine.cu)
-  if (!(kind == CTRL_CHECK0 && ph == PH_CHECK) && !(kind == CTRL_CHECK && ph == PH_CYCLE)) return;
+  if (kind != CTRL_CHECK0 || ph != PH_CHECK) return;
   double sum = 0.0;
   // the checks of the cycle's own precision: double-float partials in FP32 / FP16 cycles
   if (!control_sum(E, p, j, E.partial + E.fine_off[p], fine_tiles(E.P[p].L), sh, &sum, E.prm.prec != P64)) return;

@@ -1,4 +1,4 @@
-// Device code shared by the V-cycle kernels (k_cycle.cu, k_march.cu): programmatic dependent
+// Device code shared by the V-cycle kernels (k_*.cu): programmatic dependent
 // launch, the debug build's index checks, precision policies and loads, the deterministic norm
 // sums and the lagged convergence test, the transfer formulas, and the mbarrier / bulk-copy helpers.
 #pragma once
@@ -502,10 +502,10 @@ __host__ __device__ inline int fine_tiles(int L) {
 // iterate in buffer 0 is the result) or at the cycle cap; inner cycles of the defect correction
 // stop at the inner tolerance or the inner caps (the correction goes to the update).  Otherwise
 // the cycle proceeds and is counted.
-__device__ __forceinline__ void cond_set(const CondDev& c, int which, unsigned v) {
-  if (!((c.mask >> which) & 1u)) return;
-  cudaGraphSetConditional(which == 0 ? c.h_cycle : (which == 1 ? c.h_outer : c.h_update), v);
-  c.taken[which] = v;
+__device__ __forceinline__ void cond_set(const CondDev& c, unsigned v) {
+  if (!c.on) return;
+  cudaGraphSetConditional(c.cycle, v);
+  *c.taken = v;
 }
 
 __device__ void pre_check(ProbState& st, const Params& prm, double nrm) {
@@ -521,7 +521,6 @@ __device__ void pre_check(ProbState& st, const Params& prm, double nrm) {
     if (nrm <= prm.inner_tol * st.inner_ref || st.inner_k >= prm.inner_max ||
         st.inner_cycles >= prm.max_cycles) {
       st.phase = PH_UPDATE;
-      cond_set(prm.cond, 2, 1u);
     } else { st.inner_k += 1; st.inner_cycles += 1; st.cycles += 1; }
   }
 }
@@ -678,7 +677,7 @@ __device__ void solo_fused_check(const EngineDev& E, int level, bool checked, in
   if (checked) sum = problem_norm_sum(E.partial, fine_tiles(level), sh, E.prm.prec != P64);
   if (threadIdx.x == 0) {
     if (checked) pre_check(st, E.prm, sqrt(sum));
-    if (st.phase == want && (st.phase == PH_INNER || st.phase == PH_CYCLE)) cond_set(E.prm.cond, 0, 1u);
+    if (st.phase == want && (st.phase == PH_INNER || st.phase == PH_CYCLE)) cond_set(E.prm.cond, 1u);
     *E.ticket = 0u;                                 // ready for the next launch
   }
 }
@@ -708,8 +707,6 @@ __device__ void control_apply(const EngineDev& E, ProbState& st, int kind, doubl
       }
       break;
     case CTRL_CHECK0:
-    case CTRL_CHECK:
-      if (ph == PH_CYCLE) { st.cycles += 1; st.zero_top = 0; st.x_zero = 0; }
       st.dnorm = nrm;
       st.relres = nrm / st.bnorm;
       if (!isfinite(nrm)) { st.status = HN_ERR_NONFINITE; st.phase = PH_DONE; }
@@ -791,7 +788,7 @@ __device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, 
     over = (E.iter && it > E.iter_limit) ? 1u : 0u;
   }
   __syncthreads();
-  double c = 0.0, o = 0.0;
+  double c = 0.0;
   for (int p = threadIdx.x; p < E.nprob; p += blockDim.x) {
     ProbState& st = E.S[p];
     if (st.phase != PH_DONE && over) { st.status = HN_ERR_NOT_CONVERGED; st.phase = PH_DONE; }
@@ -799,21 +796,16 @@ __device__ void summary_apply(const EngineDev& E, cudaGraphConditionalHandle h, 
     if (end_of_iteration && (st.phase == PH_INNER || st.phase == PH_CYCLE)) st.zero_top = 0;
     if (E.states_host) E.states_host[p] = st;
     c += st.phase != PH_DONE ? 1.0 : 0.0;
-    o += st.phase == PH_OUTER ? 1.0 : 0.0;
   }
   c = block_sum256(c, sh);
-  o = block_sum256(o, sh);
   if (threadIdx.x == 0) {
     const unsigned active = (unsigned)c;
     if (E.active_host) *E.active_host = active;
     if (use_handle) cudaGraphSetConditional(h, active > 0 ? 1u : 0u);
     const CondDev& cd = E.prm.cond;
-    if (cd.mask) {
-      *cd.launches += cd.n_base + (cd.taken[0] ? cd.n_cycle : 0u) + (cd.taken[1] ? cd.n_outer : 0u) +
-                      (cd.taken[2] ? cd.n_update : 0u);
-      cond_set(cd, 0, 0u);
-      cond_set(cd, 2, 0u);
-      cond_set(cd, 1, o > 0.0 ? 1u : 0u);
+    if (cd.on) {
+      *cd.launches += cd.n_base + (*cd.taken ? cd.n_cycle : 0u);
+      cond_set(cd, 0u);
     }
   }
 }

@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(256) k_begin(const __grid_constant__ EngineDev
   for (int k = 0; k < 4; ++k) E.err[k] = 0;
   for (int k = 0; k < 3; ++k) E.gbar[k] = 0ull;
   *E.ticket = 0u;
-  // mirrors of the IF values as the closed-world graph sets them at its launch
-  for (int k = 0; k < 4; ++k) taken[k] = k == 1;
+  // the mirror of the IF node's value as the closed-world graph sets it at its launch
+  *taken = 0u;
   *launches = 0ull;
 }
 

@@ -799,7 +799,7 @@ __device__ void check_part(const EngineDev& E, int p, const float* squares, int 
     ProbState& st = E.S[p];
     if (groups > 1) ticket[1] = 0u;
     pre_check(st, E.prm, sqrt(sum));
-    if (st.phase == want) cond_set(E.prm.cond, 0, 1u);
+    if (st.phase == want) cond_set(E.prm.cond, 1u);
   }
 }
 
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(256) k_march_check(EngineDev E, TileList tl, i
   const ProbState& st = E.S[0];
   if (st.phase != want) return;
   if (tl.solo_L != level || st.zero_top) {        // nothing to check: the cycle goes on
-    if (blockIdx.x == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 0, 1u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 1u);
     return;
   }
   check_part(E, 0, static_cast<const float*>(tl.solo_d.r), level, (int)blockIdx.x / nb, (int)blockIdx.x % nb, nb, want, sh);
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(256) k_march_check_group(EngineDev E, int T, i
       // (a problem leaves the phase only after every block of its check has counted itself in)
       if (!dbg_item(E, p, 0, l, HN_HERE) || __ldcg(&E.S[p].phase) != want) continue;
       if (l <= T || E.S[p].zero_top) {            // no check (or the tail's own): the cycle goes on
-        if (blk == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 0, 1u);
+        if (blk == 0 && threadIdx.x == 0) cond_set(E.prm.cond, 1u);
         continue;
       }
       const int nb = (min(fine_tiles(l), kSumGroup) + 1023) / 1024;
