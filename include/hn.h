@@ -205,9 +205,9 @@ hn_status hn_mg_apply(hn_mg* mg, hn_op op, int level, int inner, const void* in1
  * (cudaStream_t, NULL = the legacy default stream) and returns without waiting; a caller that
  * launches while another thread captures a graph in global mode must pass a stream created with
  * cudaStreamNonBlocking, since the legacy default stream synchronizes with every blocking stream.
- * The only temporary (one partial sum per 128-node tile) is a fixed device array inside the library
- * (512 KiB, held by every GPU that loads the library until exit), so at most 8,388,608 nodes
- * (level 11) are accepted; larger operators get HN_ERR_ARG.  The call allocates nothing.  The first
+ * The only temporary (one partial sum per strip of tiles) is a fixed device array inside the library
+ * (29 KB, held by every GPU that loads the library until exit).  At most 8,388,608 nodes (level 11)
+ * are accepted; larger operators get HN_ERR_ARG.  The call allocates nothing.  The first
  * call on a device looks up that array's address and should come before any stream capture.  All
  * calls share the array: calls that overlap on the GPU (e.g. on two streams) race and must be
  * ordered by the caller.  Errors: HN_ERR_ARG (null or misaligned pointer, r overlapping x or b,

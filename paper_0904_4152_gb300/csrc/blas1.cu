@@ -181,7 +181,7 @@ hn_status check_common(hn_dtype t, long long n) {
 }
 
 // The pool of the reductions' scratch on the current device.  The device's default pool gives its memory back to the
-// // system at every synchronization, so that the next reduction mapped it anew (a dot at L = 11 after one 121 us, now
+// system at every synchronization, so that the next reduction mapped it anew (a dot at L = 11 after one 121 us, now
 // 36); this one keeps up to 64 MiB, two of the units in which a pool takes memory.  Allocations stay
 // stream-ordered, as before.
 hn_status scratch_pool(cudaMemPool_t* out) {

@@ -16,7 +16,7 @@
 namespace hn {
 namespace {
 
-constexpr long long kStaticMaxNodes = 65536LL * kTile;   // the largest operator: 8,388,608 nodes (level 11)
+constexpr long long kStaticMaxNodes = 65536LL * kTile;   // the largest operator that the contract takes (level 11)
 // Strips of tiles, each with a partial sum in the array: three blocks of 8 warps on each of 152 SMs, also where the
 // chip has another number (the order of the sum is fixed).
 constexpr int kStrips = 3648;
