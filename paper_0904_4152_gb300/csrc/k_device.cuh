@@ -404,7 +404,10 @@ __device__ double block_sum256(double v, double* sh) {
 // df: the partials are double-float pairs (an FP32 / FP16 cycle's), summed in the same order in
 // double-float arithmetic on the FP32 pipe: one SM's FP64 rate (~1.7 operations per cycle) made
 // the 8,209 FP64 additions of an L = 10 norm the longest part of its lagged check (~10 us).
-__device__ double problem_partial_sum_df(const double* part, int ntiles, double* sh) {
+//
+// Not inlined, either of them: inlined, the loads of a batch are issued as the caller's registers allow (the control step
+// after a check at L = 11 16.2 us as a call, 29.1 inlined; a cycle of k_span over level 4's 225 unknowns 92.6, 106.1).
+__device__ __noinline__ double problem_partial_sum_df(const double* part, int ntiles, double* sh) {
   const float2* pp = reinterpret_cast<const float2*>(part);
   float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, l[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (threadIdx.x < 256) {
@@ -437,7 +440,7 @@ __device__ double problem_partial_sum_df(const double* part, int ntiles, double*
   return block_sum_df(h[0], l[0], sh);
 }
 
-__device__ double problem_partial_sum(const double* part, int ntiles, double* sh, bool df = false) {
+__device__ __noinline__ double problem_partial_sum(const double* part, int ntiles, double* sh, bool df = false) {
   if (df) return problem_partial_sum_df(part, ntiles, sh);
   double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
   if (threadIdx.x < 256) {                    // larger blocks: the other threads add +0.0
