@@ -158,15 +158,17 @@ hn_status launch(hn_dtype type, SweArg a, cudaStream_t s) {
   void (*kern)(SweArg) = type == HN_F32 ? (a.nmat == 1 ? k_band4<float, 1> : k_band4<float, 4>)
                                          : (a.nmat == 1 ? k_band4<double, 1> : k_band4<double, 4>);
   // one wave of resident blocks (grid-stride loop); the occupancy of each kernel is asked once.  The FP32 prediction
-  // step, 21 streams of 4-byte values, takes a thread for every four rows instead: as blocks end and begin at
-  // different times, loads stay in flight where a wave's threads all wait at their own next rows (4096^2:
-  // 249 -> 236 us, 5.96 TB/s; cold 280 -> 254; FP64 549 against 554 us keeps its wave).
+  // step, 21 streams of 4-byte values, takes a thread for every four rows instead where a wave would have seven rounds or
+  // more: as blocks end and begin at different times, loads stay in flight where a wave's threads all wait at their own
+  // next rows (4096^2: 249 -> 236 us, 5.96 TB/s; cold 280 -> 254; 2048 x 3000 120 -> 118).  With fewer rounds the waves of
+  // blocks that replace them end unevenly (777 x 4000 77.4 us against 81.2 so, 777 x 1500 44.7 against 46.8), and FP64,
+  // 549 against 554 us, keeps its wave at any size.
   static int occ[2][2] = {{0, 0}, {0, 0}};
   int& per_sm = occ[type == HN_F32 ? 0 : 1][a.nmat == 1 ? 0 : 1];
   if (per_sm == 0) HN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0));
   const long long groups = (a.n + 3) / 4;
   const long long cap = (long long)sm_count() * std::max(per_sm, 1);
-  const bool all = type == HN_F32 && a.nmat == 4;
+  const bool all = type == HN_F32 && a.nmat == 4 && groups >= 7 * cap * kThreads;
   const long long most = all ? (long long)INT_MAX : cap;
   const int grid = (int)std::max<long long>(1, std::min((groups + kThreads - 1) / kThreads, most));
   kern<<<grid, kThreads, 0, s>>>(a);
